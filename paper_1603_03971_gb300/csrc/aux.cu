@@ -248,29 +248,196 @@ __device__ __forceinline__ void fold_range(int m, int n, int nb, int N, int& lo,
     hi = (m == n - 1) ? N - 1 : m + nb;
 }
 
+// A sum kept as an unevaluated pair of floats (about 48 bits). GB300 has
+// about two float64 lanes per SM and clock: a float64 divide, sum and
+// conversion per padded cell bounded the gradient's fold
+struct Pair {
+    float hi, lo;
+};
+// s += a + b, |b| small against a (Knuth's two-sum); an infinite or NaN sum
+// stays in hi
+__device__ __forceinline__ void pair_add(Pair& s, float a, float b) {
+    const float t = s.hi + a, bb = t - s.hi;
+    s.lo += ((s.hi - (t - bb)) + (a - bb)) + b;
+    s.hi = t;
+}
+// s += a / c as a rounded quotient and its correction. Products with 1 / c:
+// most cells of a short propagation hold denormal values, and a float divide
+// takes its slow path on those (0.53 against 0.10 ms for the inner cells at 256^3)
+__device__ __forceinline__ void pair_add_ratio(Pair& s, float a, float c) {
+    if (c > 1e-30f && c < 1e30f) {
+        const float rc = 1.0f / c, q = a * rc;
+        pair_add(s, q, fmaf(-q, c, a) * rc);
+    } else {
+        const float q = a / c;
+        pair_add(s, q, fmaf(-q, c, a) / c);
+    }
+}
+// the pair times a double, rounded once
+struct PairScale {
+    double full;
+    float hi, lo;  // hi + lo = full
+    int fits;      // full is well inside the float range
+};
+__device__ __forceinline__ float pair_scaled(const Pair& s, const PairScale& k) {
+    if (!isfinite(s.hi) || !isfinite(s.lo)) return (float)(s.hi * k.full);
+    if (!k.fits) return (float)(((double)s.hi + (double)s.lo) * k.full);
+    const float p = s.hi * k.hi;
+    if (!isfinite(p)) return p;
+    return p + (fmaf(s.hi, k.hi, -p) + fmaf(s.hi, k.lo, s.lo * k.hi));
+}
+__device__ __forceinline__ Pair warp_pair_sum(Pair s) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const float hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
+        const float lo = __shfl_xor_sync(0xffffffffu, s.lo, o);
+        pair_add(s, hi, lo);
+    }
+    return s;
+}
+
 // grad_v2[model cell] = dt^2 * sum over the padded cells copied from that
-// cell of dx^3 acc / c (the transpose of the edge padding)
+// cell of dx^3 acc / c (the transpose of the edge padding). An inner cell has
+// one padded cell, a face cell nb + 1, an edge cell (nb + 1)^2, a corner cell
+// (nb + 1)^3: one thread per model cell left the eight corner threads with
+// 36 000 dependent sums at nb = 32 (57 ms of a 75 ms gradient at 256^3).
+// So a cell's padded cells decide who sums them: a thread (inner cells; z and
+// y faces, where neighbouring threads read neighbouring columns), a warp
+// (x faces, whose padded cells are a row, and edges) or a block (corners).
+// Memory-bound: 329 MB at 256^3, nb = 32, in 0.27 ms over the three kernels
+struct FoldBox {
+    int x0, x1, y0, y1, z0, z1;
+};
+__device__ __forceinline__ FoldBox fold_box(const Geometry& G, int x, int y, int z) {
+    FoldBox b;
+    fold_range(x, G.nx, G.nb, G.NX, b.x0, b.x1);
+    fold_range(y, G.ny, G.nb, G.NY, b.y0, b.y1);
+    fold_range(z, G.nz, G.nb, G.NZ, b.z0, b.z1);
+    return b;
+}
+enum FoldOwner { FOLD_CELL, FOLD_COLUMN, FOLD_WARP, FOLD_BLOCK };
+__device__ __forceinline__ FoldOwner fold_owner(const FoldBox& b) {
+    const bool x = b.x1 > b.x0, y = b.y1 > b.y0, z = b.z1 > b.z0;
+    if (x && y && z) return FOLD_BLOCK;
+    if (x || (y && z)) return FOLD_WARP;
+    return y || z ? FOLD_COLUMN : FOLD_CELL;
+}
+
+// inner cells, a row per block and pass
 __global__ void k_grad_finalize(Geometry G, const float* __restrict__ acc,
-                                const float* __restrict__ c, double dx3, double dt2,
+                                const float* __restrict__ c, PairScale scale,
                                 float* __restrict__ grad) {
-    const long long n = (long long)G.nx * G.ny * G.nz;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int x = (int)(i % G.nx);
-        const int y = (int)((i / G.nx) % G.ny);
-        const int z = (int)(i / ((long long)G.nx * G.ny));
-        int x0, x1, y0, y1, z0, z1;
-        fold_range(x, G.nx, G.nb, G.NX, x0, x1);
-        fold_range(y, G.ny, G.nb, G.NY, y0, y1);
-        fold_range(z, G.nz, G.nb, G.NZ, z0, z1);
-        double s = 0.0;
-        for (int zz = z0; zz <= z1; zz++)
-            for (int yy = y0; yy <= y1; yy++)
-                for (int xx = x0; xx <= x1; xx++) {
-                    const long long p = ((long long)zz * G.NY + yy) * G.NX + xx;
-                    s += (double)acc[p] / (double)c[p];
-                }
-        grad[i] = (float)(s * dx3 * dt2);
+    const unsigned rows = (unsigned)G.ny * (unsigned)G.nz;
+    for (unsigned row = blockIdx.x; row < rows; row += gridDim.x) {
+        const int z = (int)(row / (unsigned)G.ny), y = (int)(row - (unsigned)z * G.ny);
+        const long long p = ((long long)(z + G.nb) * G.NY + (y + G.nb)) * G.NX + G.nb;
+        float* out = grad + (long long)row * G.nx;
+        const bool yz_inner = fold_owner(fold_box(G, 1 < G.nx - 1 ? 1 : 0, y, z)) == FOLD_CELL;
+        for (int x = threadIdx.x; x < G.nx; x += blockDim.x) {
+            if (G.nb > 0 && (!yz_inner || x == 0 || x == G.nx - 1)) continue;
+            Pair s{0.f, 0.f};
+            pair_add_ratio(s, __ldcs(acc + p + x), __ldcs(c + p + x));
+            out[x] = pair_scaled(s, scale);
+        }
+    }
+}
+
+// sum of a box over `n` threads, thread `t` of them, x fastest (a box holds
+// less than an eighth of the padded grid: 32-bit counts)
+__device__ __forceinline__ Pair fold_sum(const Geometry& G, const FoldBox& b,
+                                         const float* __restrict__ acc,
+                                         const float* __restrict__ c, int t, int n) {
+    const unsigned bx = b.x1 - b.x0 + 1, by = b.y1 - b.y0 + 1, bz = b.z1 - b.z0 + 1;
+    const unsigned cells = bx * by * bz;
+    Pair s{0.f, 0.f};
+#pragma unroll 4
+    for (unsigned k = t; k < cells; k += n) {
+        const unsigned zy = k / bx, zz = zy / by;
+        const long long p = ((long long)(b.z0 + zz) * G.NY + (b.y0 + (zy - zz * by))) * G.NX +
+                            (b.x0 + (k - zy * bx));
+        pair_add_ratio(s, acc[p], c[p]);
+    }
+    return s;
+}
+
+// a row of y- or z-face cells, a column of padded cells per thread
+__device__ void fold_columns(const Geometry& G, int y, int z, const float* __restrict__ acc,
+                             const float* __restrict__ c, const PairScale& scale,
+                             float* __restrict__ grad) {
+    for (int x = threadIdx.x; x < G.nx; x += blockDim.x) {
+        const FoldBox b = fold_box(G, x, y, z);
+        if (fold_owner(b) != FOLD_COLUMN) continue;
+        const bool along_y = b.y1 > b.y0;
+        const int n = along_y ? b.y1 - b.y0 + 1 : b.z1 - b.z0 + 1;
+        const long long step = along_y ? G.NX : (long long)G.NX * G.NY;
+        long long p = ((long long)b.z0 * G.NY + b.y0) * G.NX + b.x0;
+        Pair s{0.f, 0.f};
+#pragma unroll 8
+        for (int k = 0; k < n; k++, p += step) pair_add_ratio(s, __ldcs(acc + p), __ldcs(c + p));
+        grad[((long long)z * G.ny + y) * G.nx + x] = pair_scaled(s, scale);
+    }
+}
+
+__device__ void fold_warp(const Geometry& G, int x, int y, int z, const float* __restrict__ acc,
+                          const float* __restrict__ c, const PairScale& scale,
+                          float* __restrict__ grad) {
+    const FoldBox b = fold_box(G, x, y, z);
+    if (fold_owner(b) != FOLD_WARP) return;  // the same for the whole warp
+    const int lane = threadIdx.x & 31;
+    const Pair s = warp_pair_sum(fold_sum(G, b, acc, c, lane, 32));
+    if (lane == 0) grad[((long long)z * G.ny + y) * G.nx + x] = pair_scaled(s, scale);
+}
+
+// the face and edge cells. blockIdx.y: 0 and 1 the x faces (a warp per cell),
+// 2 and 3 the z faces, 4 and 5 the y faces (a row of cells per block), 6 the
+// four edges along x (a warp per cell)
+__global__ void k_grad_finalize_faces(Geometry G, const float* __restrict__ acc,
+                                      const float* __restrict__ c, PairScale scale,
+                                      float* __restrict__ grad) {
+    const int what = blockIdx.y, far_side = what & 1;
+    const unsigned warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const unsigned nwarps = gridDim.x * (blockDim.x >> 5);
+    if (what < 2) {
+        if (far_side && G.nx == 1) return;
+        const unsigned cells = (unsigned)G.ny * (unsigned)G.nz;
+        for (unsigned f = warp; f < cells; f += nwarps) {
+            const int z = (int)(f / (unsigned)G.ny), y = (int)(f - (unsigned)z * G.ny);
+            fold_warp(G, far_side ? G.nx - 1 : 0, y, z, acc, c, scale, grad);
+        }
+    } else if (what < 4) {
+        if (far_side && G.nz == 1) return;
+        for (int y = blockIdx.x; y < G.ny; y += gridDim.x)
+            fold_columns(G, y, far_side ? G.nz - 1 : 0, acc, c, scale, grad);
+    } else if (what < 6) {
+        if (far_side && G.ny == 1) return;
+        for (int z = blockIdx.x; z < G.nz; z += gridDim.x)
+            fold_columns(G, far_side ? G.ny - 1 : 0, z, acc, c, scale, grad);
+    } else {
+        for (unsigned f = warp; f < 4u * (unsigned)G.nx; f += nwarps) {
+            const int e = (int)(f / (unsigned)G.nx), x = (int)(f - (unsigned)e * G.nx);
+            if (x == 0 || x == G.nx - 1) continue;  // in the x faces
+            if (((e & 1) && G.ny == 1) || ((e & 2) && G.nz == 1)) continue;
+            fold_warp(G, x, e & 1 ? G.ny - 1 : 0, e & 2 ? G.nz - 1 : 0, acc, c, scale, grad);
+        }
+    }
+}
+
+// the corner cells, one per block
+__global__ void __launch_bounds__(1024) k_grad_finalize_corners(Geometry G,
+                                                                const float* __restrict__ acc,
+                                                                const float* __restrict__ c,
+                                                                PairScale scale,
+                                                                float* __restrict__ grad) {
+    __shared__ Pair part[32];
+    const int e = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (((e & 1) && G.nx == 1) || ((e & 2) && G.ny == 1) || ((e & 4) && G.nz == 1)) return;
+    const int x = e & 1 ? G.nx - 1 : 0, y = e & 2 ? G.ny - 1 : 0, z = e & 4 ? G.nz - 1 : 0;
+    const FoldBox b = fold_box(G, x, y, z);
+    Pair s = warp_pair_sum(fold_sum(G, b, acc, c, threadIdx.x, blockDim.x));
+    if (lane == 0) part[wid] = s;
+    __syncthreads();
+    if (wid == 0) {
+        s = warp_pair_sum(part[lane]);
+        if (lane == 0) grad[((long long)z * G.ny + y) * G.nx + x] = pair_scaled(s, scale);
     }
 }
 
@@ -498,8 +665,16 @@ cudaError_t launch_image_laplacian(const float* image, int nx, int ny, int nz,
 
 cudaError_t launch_grad_finalize(const Geometry& G, const float* acc, const float* c,
                                  double dx3, double dt2, float* grad_v2, cudaStream_t s) {
-    const long long n = (long long)G.nx * G.ny * G.nz;
-    k_grad_finalize<<<grid_for(n, 256), 256, 0, s>>>(G, acc, c, dx3, dt2, grad_v2);
+    const double full = dx3 * dt2;
+    const float hi = (float)full;
+    const PairScale scale{full, hi, (float)(full - (double)hi), full > 1e-20 && full < 1e20};
+    const long long rows = (long long)G.ny * G.nz;
+    k_grad_finalize<<<grid_for(rows, 1), 256, 0, s>>>(G, acc, c, scale, grad_v2);
+    if (G.nb > 0) {
+        const dim3 grid(grid_for(std::max(rows / 8, (long long)std::max(G.ny, G.nz)), 1), 7);
+        k_grad_finalize_faces<<<grid, 256, 0, s>>>(G, acc, c, scale, grad_v2);
+        k_grad_finalize_corners<<<8, 1024, 0, s>>>(G, acc, c, scale, grad_v2);
+    }
     return cudaGetLastError();
 }
 
