@@ -7,6 +7,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <string>
@@ -17,6 +18,7 @@
 #include "band.cuh"
 #include "revolve.h"
 #include "rtm_internal.h"
+#include "span.h"
 
 using namespace rtm;
 
@@ -114,7 +116,7 @@ void count_launch(int n = 1) {
 // ---- workspace layout ----------------------------------------------------------
 constexpr size_t kAlign = 256;
 constexpr size_t kStatusBytes = 256;  // status word at 0, model-prep reduction at 16,
-                                      // image-filter maximum at 32
+                                      // image-filter maximum at 32, span control at 64
 size_t up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
@@ -317,6 +319,10 @@ struct Ctx {
     bool snap_padded = false;   // imaging snapshots are padded fields (boundary storage)
     int zchunk_mode[MODE_COUNT] = {0};  // per-mode slab heights (0: base.zchunk)
     const rtm_point_taps* taps = nullptr;  // off-grid source and receivers, or NULL
+    // several steps per launch (span.cu), forward and backward; ok = 0: one
+    // launch per step
+    SpanPlan span_fwd, span_bwd;
+    unsigned int span_count = 0;  // barrier arrivals of this call's spans so far
 
     float* at(size_t off) const { return reinterpret_cast<float*>(ws + off); }
     float* coarse_slot(size_t k) const {
@@ -369,8 +375,10 @@ rtm_status make_ctx(Ctx& C, const rtm_params* p, const float* c, void* ws, rtm_s
     C.base.ny = p->ny;
     C.base.nz = p->nz;
     int zc, var;
+    bool timing;
     {
         std::lock_guard<std::mutex> lk(g_mu);
+        timing = g_timing;
         zc = g_zchunk[p->radius];
         var = g_variant[p->radius];
         for (int m = 0; m < MODE_COUNT; m++) C.zchunk_mode[m] = g_zchunk_mode[p->radius][m];
@@ -382,6 +390,73 @@ rtm_status make_ctx(Ctx& C, const rtm_params* p, const float* c, void* ws, rtm_s
     C.variant = var != 0 ? var : (tma_available() ? 2 : 1);
     C.snap_padded = p->storage == RTM_STORE_BOUNDARY;
     set_region(C.base, MODE_FWD);
+    // spans replace the automatic choice only: a tuned variant or slab height
+    // names the plane-marching kernels, and per-launch timing needs launches
+    bool tuned = zc > 0 || var != 0 || timing;
+    for (int m = 0; m < MODE_COUNT; m++) tuned = tuned || C.zchunk_mode[m] > 0;
+    if (!tuned) {
+        C.span_fwd = span_plan(p->radius, C.d.NX, C.d.NY, C.d.NZ, 0);
+        C.span_bwd = span_plan(p->radius, C.d.NX, C.d.NY, C.d.NZ, 1);
+    }
+    return RTM_OK;
+}
+
+// the span control words start a call at zero
+rtm_status clear_span(Ctx& C) {
+    if (C.span_fwd.ok || C.span_bwd.ok)
+        CU(cudaMemsetAsync(C.ws + C.L.status + kSpanCtrlOffset, 0, sizeof(SpanCtrl), C.s));
+    C.span_count = 0;
+    return RTM_OK;
+}
+
+SpanArgs span_args(const Ctx& C, const SpanPlan& P, float* prev, float* cur, const int32_t* rec,
+                   int first, int nsteps) {
+    SpanArgs a;
+    memset(&a, 0, sizeof a);
+    a.P = P;
+    a.c = C.base.c;
+    a.gx = C.base.gx;
+    a.gy = C.base.gy;
+    a.gz = C.base.gz;
+    a.wav = C.wav();
+    a.f[0] = prev;
+    a.f[1] = cur;
+    a.NX = C.d.NX;
+    a.NY = C.d.NY;
+    a.NZ = C.d.NZ;
+    a.nb = C.p->nb;
+    a.nx = C.p->nx;
+    a.ny = C.p->ny;
+    a.nz = C.p->nz;
+    a.radius = C.p->radius;
+    a.first = first;
+    a.nsteps = nsteps;
+    a.nt = C.p->nt;
+    a.rec = rec;
+    a.taps = C.taps;
+    a.nrec = C.p->nrec;
+    a.src = C.src;
+    a.inv_dx3 = C.inv_dx3;
+    a.every = C.p->image_every;
+    a.div = 1;
+    memcpy(a.a, C.base.a, sizeof a.a);
+    a.ctrl = reinterpret_cast<SpanCtrl*>(C.ws + C.L.status + kSpanCtrlOffset);
+    a.status = C.status();
+    return a;
+}
+
+// launches a span whose steps are of statistics slot `slot` and leaves the
+// newest state in cur
+rtm_status run_span(Ctx& C, SpanArgs& a, int slot, float*& prev, float*& cur) {
+    a.base = C.span_count;
+    CU(launch_span(a, C.s));
+    C.span_count += (unsigned int)a.P.nbricks * (unsigned int)(a.nsteps - 1);
+    {
+        std::lock_guard<std::mutex> lk(g_mu);
+        g_stats.launches += 1;
+        g_stats.stencil_launches[slot] += a.nsteps;
+    }
+    if (a.nsteps & 1) std::swap(prev, cur);
     return RTM_OK;
 }
 
@@ -487,12 +562,45 @@ rtm_status run_forward(Ctx& C, const int32_t* rec, float* data, float* u_last) {
     CU(cudaMemsetAsync(prev, 0, fb, C.s));
     CU(cudaMemsetAsync(cur, 0, fb, C.s));
     CHECK(prepare_tables(C));
+    CHECK(clear_span(C));
     const int k = p->ckpt_every, ie = p->image_every;
+    // a step whose state is coded runs on its own
+    const bool coded = p->storage == RTM_STORE_LEARNED || p->storage == RTM_STORE_DECIMATED;
+    auto is_coded = [&](int n) { return coded && (n + 1) % ie == 0 && n + 1 > p->ckpt_every; };
     for (int n = 0; n < p->nt; n++) {
         if (p->storage == RTM_STORE_CKPT && n > 0 && n % k == 0) {
             const size_t j = (size_t)(n / k);
             CU(cudaMemcpyAsync(C.ckpt_field(j, 0), prev, fb, cudaMemcpyDeviceToDevice, C.s));
             CU(cudaMemcpyAsync(C.ckpt_field(j, 1), cur, fb, cudaMemcpyDeviceToDevice, C.s));
+        }
+        if (C.span_fwd.ok) {
+            int end = p->nt;  // one past the span's last step
+            if (p->storage == RTM_STORE_CKPT) end = std::min(end, (n / k + 1) * k);
+            if (coded) {
+                // the next coded step: its state n + 1 is a multiple of ie past the exact window
+                const int from = std::max(n, p->ckpt_every) + 1;
+                end = std::min(end, (from + ie - 1) / ie * ie - 1);
+            }
+            if (end > n) {
+                SpanArgs a = span_args(C, C.span_fwd, prev, cur, rec, n, end - n);
+                a.data = data;
+                if (p->storage == RTM_STORE_ALL) {
+                    a.grad = p->want_grad;
+                    a.snap = C.snap_slot(0);
+                    a.snap_stride = (long long)C.L.snap_elems;
+                    a.div = a.every;
+                    a.off = 1;
+                }
+                if (p->storage == RTM_STORE_BOUNDARY) {
+                    a.band = C.at(C.L.band);
+                    a.band_stride = (long long)C.L.nband;
+                    a.band_last = p->nt - 2;
+                }
+                const int slot = a.snap ? (a.grad ? MODE_FWD_LU : MODE_FWD_SNAP) : MODE_FWD;
+                CHECK(run_span(C, a, slot, prev, cur));
+                n = end - 1;
+                continue;
+            }
         }
         float* row = (data && n >= 1) ? data + (size_t)(n - 1) * p->nrec : nullptr;
         CHECK(fwd_aux(C, cur, prev, rec, row, C.wav() + n));
@@ -509,10 +617,8 @@ rtm_status run_forward(Ctx& C, const int32_t* rec, float* data, float* u_last) {
         }
         // learned storage: the step that writes a coded snapshot also sums
         // its squares for the encoder's scale (no separate pass over it)
-        const bool code = p->storage == RTM_STORE_LEARNED && (n + 1) % ie == 0 &&
-                          n + 1 > p->ckpt_every;
-        const bool decim = p->storage == RTM_STORE_DECIMATED && (n + 1) % ie == 0 &&
-                           n + 1 > p->ckpt_every;
+        const bool code = p->storage == RTM_STORE_LEARNED && is_coded(n);
+        const bool decim = p->storage == RTM_STORE_DECIMATED && is_coded(n);
         auto* scal = reinterpret_cast<ae::AeScalars*>(C.at(C.L.ae_scalars));
         if (code) {
             CU(cudaMemsetAsync(&scal->sumsq, 0, sizeof(double), C.s));
@@ -553,11 +659,41 @@ rtm_status run_forward(Ctx& C, const int32_t* rec, float* data, float* u_last) {
     return RTM_OK;
 }
 
+// source steps n0 .. n1 - 1 without data, in place over (prev, cur). The state
+// k = n + 1 is kept where snap is given and k % every == 0: its model rows, or
+// with grad L u of the step's u^n, at snap + (k / div - off) * L.snap_elems,
+// or at snap itself with div = 0
+rtm_status forward_steps(Ctx& C, const int32_t* rec, int n0, int n1, float*& prev, float*& cur,
+                         float* snap, int every, int div, int off, bool grad) {
+    if (n1 <= n0) return RTM_OK;
+    const long long stride = div ? (long long)C.L.snap_elems : 0;
+    if (div == 0) div = 1;
+    const int keep_mode = grad ? MODE_FWD_LU : MODE_FWD_SNAP;
+    if (C.span_fwd.ok) {
+        SpanArgs a = span_args(C, C.span_fwd, prev, cur, rec, n0, n1 - n0);
+        a.snap = snap;
+        a.snap_stride = stride;
+        a.every = every;
+        a.div = div;
+        a.off = off;
+        a.grad = grad;
+        return run_span(C, a, snap ? keep_mode : MODE_FWD, prev, cur);
+    }
+    for (int n = n0; n < n1; n++) {
+        CHECK(fwd_aux(C, cur, prev, rec, nullptr, C.wav() + n));
+        const bool keep = snap && (n + 1) % every == 0;
+        CHECK(stencil(C, keep ? keep_mode : MODE_FWD, cur, prev,
+                      keep ? snap + ((n + 1) / div - off) * stride : nullptr, nullptr));
+        std::swap(prev, cur);
+    }
+    return RTM_OK;
+}
+
 // binomial checkpointing: the source states the imaging steps need, in
 // reverse order, from a schedule of forward recomputation, slot stores and
 // restores (revolve.h); backward steps run as their states are delivered
-template <class BackStep>
-rtm_status run_revolve(Ctx& C, const int32_t* rec, BackStep& back_step) {
+template <class BackSteps>
+rtm_status run_revolve(Ctx& C, const int32_t* rec, BackSteps& back_steps) {
     const rtm_params* p = C.p;
     const int ie = p->image_every;
     const int M = p->nt / ie;
@@ -584,15 +720,9 @@ rtm_status run_revolve(Ctx& C, const int32_t* rec, BackStep& back_step) {
                 }
                 break;
             case REV_ADVANCE:
-                for (int n = A.a * ie; n < A.b * ie; n++) {
-                    CHECK(fwd_aux(C, fc, fp, rec, nullptr, C.wav() + n));
-                    const bool snap = A.c && n == A.b * ie - 1;
-                    CHECK(stencil(C, snap ? MODE_FWD_SNAP : MODE_FWD, fc, fp, snap ? slab : nullptr,
-                                  nullptr));
-                    float* t = fp;
-                    fp = fc;
-                    fc = t;
-                }
+                // the snapshot of the last state only
+                CHECK(forward_steps(C, rec, A.a * ie, A.b * ie, fp, fc, A.c ? slab : nullptr,
+                                    A.b * ie, 0, 0, false));
                 break;
             case REV_STORE:
                 CU(cudaMemcpyAsync(C.ckpt_field((size_t)A.a + 1, 0), fp, fb,
@@ -608,11 +738,9 @@ rtm_status run_revolve(Ctx& C, const int32_t* rec, BackStep& back_step) {
                     CU(cudaMemcpy2DAsync(slab, row, u, sizeof(float) * (size_t)C.d.NY * C.d.NX,
                                          row, (size_t)p->nz, cudaMemcpyDeviceToDevice, C.s));
                 }
-                for (; m_next > m_img; m_next--) {
-                    if (m_next % ie == 0) return fail(RTM_ERR_STATE, "schedule skipped step %d", m_next);
-                    CHECK(back_step(m_next, nullptr));
-                }
-                CHECK(back_step(m_img, slab));
+                for (int m = m_next; m > m_img; m--)
+                    if (m % ie == 0) return fail(RTM_ERR_STATE, "schedule skipped step %d", m);
+                CHECK(back_steps(m_next, m_img, slab, 0, 0));
                 m_next = m_img - 1;
                 break;
             }
@@ -620,11 +748,9 @@ rtm_status run_revolve(Ctx& C, const int32_t* rec, BackStep& back_step) {
                 break;
         }
     }
-    for (; m_next >= 1; m_next--) {
-        if (m_next % ie == 0) return fail(RTM_ERR_STATE, "schedule skipped step %d", m_next);
-        CHECK(back_step(m_next, nullptr));
-    }
-    return RTM_OK;
+    for (int m = m_next; m >= 1; m--)
+        if (m % ie == 0) return fail(RTM_ERR_STATE, "schedule skipped step %d", m);
+    return m_next >= 1 ? back_steps(m_next, 1, nullptr, 0, 0) : RTM_OK;
 }
 
 // receiver propagation, imaging (grad = false) or gradient accumulation (grad = true)
@@ -639,6 +765,7 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
     CU(cudaMemsetAsync(mcur, 0, fb, C.s));
     CU(cudaMemsetAsync(acc, 0, sizeof(float) * (grad ? C.d.N : C.d.slab), C.s));
     CHECK(prepare_tables(C));
+    CHECK(clear_span(C));
     const int ie = p->image_every;
 
     auto back_step = [&](int m, float* snap) -> rtm_status {
@@ -661,12 +788,39 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
         return RTM_OK;
     };
 
+    // steps m = hi .. lo; the imaging steps read the snapshot of state m at
+    // snap + (m / div - off) * L.snap_elems, or snap itself with div = 0
+    auto back_steps = [&](int hi, int lo, float* snap, int div, int off) -> rtm_status {
+        if (hi < lo) return RTM_OK;
+        const long long stride = div ? (long long)C.L.snap_elems : 0;
+        if (C.span_bwd.ok && !C.snap_padded) {
+            SpanArgs a = span_args(C, C.span_bwd, mprev, mcur, rec, hi, hi - lo + 1);
+            a.backward = 1;
+            a.grad = grad;
+            a.rdata = rdata;
+            a.src_adj = src_adj;
+            a.snap = snap;
+            a.snap_stride = stride;
+            a.div = div ? div : 1;
+            a.off = off;
+            a.acc = acc;
+            a.illum = C.illum;
+            return run_span(C, a, snap ? (grad ? MODE_BWD_GRAD : MODE_BWD_IMAGE) : MODE_FWD, mprev,
+                            mcur);
+        }
+        for (int m = hi; m >= lo; m--) {
+            float* s = !snap ? nullptr : div ? snap + (m / div - off) * stride : snap;
+            CHECK(back_step(m, m % ie == 0 ? s : nullptr));
+        }
+        return RTM_OK;
+    };
+
     if (p->storage == RTM_STORE_LEARNED || p->storage == RTM_STORE_DECIMATED) {
         const int W = p->ckpt_every;  // exact window: steps 1..W recomputed, not coded
         float* slab = C.snap_slot(0);
         // columns outside the model stay finite (the decoders write model columns)
         CU(cudaMemsetAsync(slab, 0, sizeof(float) * C.d.slab, C.s));
-        for (int m = p->nt; m > W; m--) {
+        for (int m = p->nt; m > W;) {
             if (m % ie == 0) {
                 const size_t k = (size_t)(m / ie - 1);
                 if (p->storage == RTM_STORE_DECIMATED)
@@ -676,27 +830,21 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
                                  C.model_view(slab), nullptr, C.status(), C.s));
                 count_launch(1);
             }
-            CHECK(back_step(m, slab));
+            // down to the state after the next coded one
+            const int lo = std::max(W, (m - 1) / ie * ie) + 1;
+            CHECK(back_steps(m, lo, slab, 0, 0));
+            m = lo - 1;
         }
         if (W > 0) {  // checkpoint-recompute fallback from the zero initial state
             float* rp = C.at(C.L.f[0]);
             float* rc = C.at(C.L.f[1]);
             CU(cudaMemsetAsync(rp, 0, fb, C.s));
             CU(cudaMemsetAsync(rc, 0, fb, C.s));
-            for (int n = 0; n < W; n++) {
-                CHECK(fwd_aux(C, rc, rp, rec, nullptr, C.wav() + n));
-                const bool snap = (n + 1) % ie == 0;
-                CHECK(stencil(C, snap ? MODE_FWD_SNAP : MODE_FWD, rc, rp,
-                              snap ? C.snap_slot((size_t)((n + 1) / ie - 1)) : nullptr, nullptr));
-                float* t = rp;
-                rp = rc;
-                rc = t;
-            }
-            for (int m = W; m >= 1; m--)
-                CHECK(back_step(m, m % ie == 0 ? C.snap_slot((size_t)(m / ie - 1)) : nullptr));
+            CHECK(forward_steps(C, rec, 0, W, rp, rc, C.snap_slot(0), ie, ie, 1, false));
+            CHECK(back_steps(W, 1, C.snap_slot(0), ie, 1));
         }
     } else if (p->storage == RTM_STORE_REVOLVE) {
-        CHECK(run_revolve(C, rec, back_step));
+        CHECK(run_revolve(C, rec, back_steps));
     } else if (p->storage == RTM_STORE_BOUNDARY) {
         // the forward run leaves u^{nt} in f[(nt + 1) % 2] and u^{nt-1} in
         // f[nt % 2]; each earlier state is recovered in the model region by
@@ -720,12 +868,7 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
             CHECK(back_step(m, m % ie == 0 ? lo : nullptr));
         }
     } else if (p->storage == RTM_STORE_ALL) {
-        for (int m = p->nt; m >= 1; m--) {
-            float* snap = nullptr;
-            if (grad) snap = C.snap_slot((size_t)(m - 1));
-            else if (m % ie == 0) snap = C.snap_slot((size_t)(m / ie - 1));
-            CHECK(back_step(m, snap));
-        }
+        CHECK(back_steps(p->nt, 1, C.snap_slot(0), ie, 1));
     } else {
         const int k = p->ckpt_every;
         const int nseg = (p->nt + k - 1) / k;
@@ -742,23 +885,9 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
                 rcur = C.ckpt_field((size_t)j, 1);
             }
             // recompute the segment from its checkpoint (in place)
-            for (int n = n0; n < n1; n++) {
-                CHECK(fwd_aux(C, rcur, rprev, rec, nullptr, C.wav() + n));
-                int mode = MODE_FWD;
-                float* snap = nullptr;
-                if (grad) {
-                    mode = MODE_FWD_LU;
-                    snap = C.snap_slot((size_t)(n - n0));
-                } else if ((n + 1) % ie == 0) {
-                    mode = MODE_FWD_SNAP;
-                    snap = C.snap_slot((size_t)(n - n0));
-                }
-                CHECK(stencil(C, mode, rcur, rprev, snap, nullptr));
-                float* t = rprev;
-                rprev = rcur;
-                rcur = t;
-            }
-            for (int m = n1; m > n0; m--) CHECK(back_step(m, C.snap_slot((size_t)(m - 1 - n0))));
+            CHECK(forward_steps(C, rec, n0, n1, rprev, rcur, C.snap_slot(0), ie, 1, n0 + 1,
+                                grad));
+            CHECK(back_steps(n1, n0 + 1, C.snap_slot(0), 1, n0 + 1));
         }
     }
     // n = 0 terms: source trace and gradient source term of mu^1
