@@ -473,6 +473,15 @@ double stencil_bytes(const Ctx& C, int mode) {
     }
 }
 
+// one step with the plane loads and tile of the context's variant
+cudaError_t launch_variant(const Ctx& C, int mode, const StepArgs& a) {
+    const int r = C.p->radius;
+    if (C.variant == 1) return launch_stencil(r, mode, a, C.s);
+    if (C.variant == 3) return launch_stencil_tma(r, mode, a, C.status(), C.s, 8);
+    return r == 8 ? launch_stencil_rows(mode, a, C.status(), C.s)
+                  : launch_stencil_tma(r, mode, a, C.status(), C.s, 16);
+}
+
 rtm_status stencil(Ctx& C, int mode, const float* cur, float* prev, float* snap, float* acc,
                    double* sumsq = nullptr) {
     StepArgs a = C.base;
@@ -504,16 +513,12 @@ rtm_status stencil(Ctx& C, int mode, const float* cur, float* prev, float* snap,
     if (timing) {
         PendingTiming t{t_timer.get(), t_timer.get(), slot, stencil_bytes(C, slot)};
         CU(cudaEventRecord(t.a, C.s));
-        CU(C.variant >= 2 ? launch_stencil_tma(C.p->radius, mode, a, C.status(), C.s,
-                                               C.variant == 3 ? 8 : 16)
-                          : launch_stencil(C.p->radius, mode, a, C.s));
+        CU(launch_variant(C, mode, a));
         CU(cudaEventRecord(t.b, C.s));
         t_timer.pending.push_back(t);
         if (t_timer.pending.size() >= 2048) CHECK(t_timer.drain(C.s));
     } else {
-        CU(C.variant >= 2 ? launch_stencil_tma(C.p->radius, mode, a, C.status(), C.s,
-                                               C.variant == 3 ? 8 : 16)
-                          : launch_stencil(C.p->radius, mode, a, C.s));
+        CU(launch_variant(C, mode, a));
     }
     return RTM_OK;
 }

@@ -82,6 +82,8 @@ cudaError_t launch_stencil(int radius, int mode, const StepArgs& a, cudaStream_t
 // tile_rows: 16 (256-thread blocks) or 8 (128-thread blocks)
 cudaError_t launch_stencil_tma(int radius, int mode, const StepArgs& a, int* status,
                                cudaStream_t s, int tile_rows = 16);
+// radius 8, 16-row tiles with two rows per thread (stencil_rows.cu)
+cudaError_t launch_stencil_rows(int mode, const StepArgs& a, int* status, cudaStream_t s);
 bool tma_available();
 int auto_zchunk(int radius, int NX, int NY, int NZ);
 

@@ -14,5 +14,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn tma_encoder();
+// map of a dense float32 [nz][ny][nx] array with boxes of by rows of bx, kept
+// per thread by its arguments
+cudaError_t tma_map3(CUtensorMap* m, const float* base, int nx, int ny, int nz, int bx, int by);
 
 }  // namespace rtm
