@@ -317,7 +317,8 @@ struct Ctx {
     const float* ae = nullptr;  // codec parameters (learned storage)
     float* illum = nullptr;     // source illumination, model grid (+=), or NULL
     bool snap_padded = false;   // imaging snapshots are padded fields (boundary storage)
-    int zchunk_mode[MODE_COUNT] = {0};  // per-mode slab heights (0: base.zchunk)
+    int zchunk_mode[MODE_COUNT] = {0};  // per-mode slab heights set by the user (0: base.zchunk)
+    int zchunk_auto[MODE_COUNT] = {0};  // per-mode slab heights sized here (0: not yet)
     const rtm_point_taps* taps = nullptr;  // off-grid source and receivers, or NULL
     // several steps per launch (span.cu), forward and backward; ok = 0: one
     // launch per step
@@ -383,11 +384,13 @@ rtm_status make_ctx(Ctx& C, const rtm_params* p, const float* c, void* ws, rtm_s
         var = g_variant[p->radius];
         for (int m = 0; m < MODE_COUNT; m++) C.zchunk_mode[m] = g_zchunk_mode[p->radius][m];
     }
-    C.base.zchunk = zc > 0 ? zc : auto_zchunk(p->radius, C.d.NX, C.d.NY, C.d.NZ);
-    if ((C.d.NZ + C.base.zchunk - 1) / C.base.zchunk > 65535)
-        C.base.zchunk = (C.d.NZ + 65534) / 65535;  // grid.z limit
-    // automatic: TMA plane loads wherever the driver provides tensor maps
-    C.variant = var != 0 ? var : (tma_available() ? 2 : 1);
+    C.base.zchunk = zc;  // 0: sized per mode (stencil())
+    // automatic: TMA plane loads wherever the driver provides tensor maps;
+    // 8-row tiles at radius 4 (the faster ones at every shape from 192 x 173 x
+    // 159 to 576^3: 454 / 565 / 740 against 459 / 568 / 749 us per launch at
+    // 576^3), 16-row tiles with two rows per thread at radius 8 (534 / 592 /
+    // 780 against 645 / 695 / 795)
+    C.variant = var != 0 ? var : (tma_available() ? (p->radius == 4 ? 3 : 2) : 1);
     C.snap_padded = p->storage == RTM_STORE_BOUNDARY;
     set_region(C.base, MODE_FWD);
     // spans replace the automatic choice only: a tuned variant or slab height
@@ -493,13 +496,18 @@ rtm_status stencil(Ctx& C, int mode, const float* cur, float* prev, float* snap,
     // the statistics count the sum-of-squares forward step as a forward step
     const int slot = mode == MODE_FWD_SUMSQ ? MODE_FWD : mode;
     set_region(a, mode);
-    // the reverse step covers the model region: its slabs are sized for its
-    // own tiles (a slab height tuned for the padded grid can leave it a
-    // nearly empty last wave)
-    if (mode == MODE_REV)
-        a.zchunk = auto_zchunk(C.p->radius, a.xend - a.xorg, a.yend - a.yorg, a.zend - a.zorg);
-    // a slab height tuned for this mode (its statistics slot) wins
-    if (C.zchunk_mode[slot] > 0) a.zchunk = C.zchunk_mode[slot];
+    // a slab height tuned for this mode (its statistics slot) wins; without one
+    // the slabs are sized for the mode's region and tiles. The reverse step
+    // covers the model region: it does not take the height set for the radius
+    // (one tuned for the padded grid can leave it a nearly empty last wave)
+    if (C.zchunk_mode[slot] > 0) {
+        a.zchunk = C.zchunk_mode[slot];
+    } else if (a.zchunk == 0 || mode == MODE_REV) {
+        if (C.zchunk_auto[slot] == 0)
+            C.zchunk_auto[slot] = slab_height(C.p->radius, C.variant, mode, a.xend - a.xorg,
+                                              a.yend - a.yorg, a.zend - a.zorg);
+        a.zchunk = C.zchunk_auto[slot];
+    }
     if ((a.zend - a.zorg + a.zchunk - 1) / a.zchunk > 65535)
         a.zchunk = (a.zend - a.zorg + 65534) / 65535;  // grid.z limit
     a.snap_padded = (mode == MODE_BWD_IMAGE && C.snap_padded) ? 1 : 0;

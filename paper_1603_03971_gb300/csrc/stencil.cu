@@ -15,6 +15,8 @@
 // the halo re-reads of u^n come from L2, because all tiles of a z slab
 // advance through z together.
 
+#include <algorithm>
+
 #include "rtm_internal.h"
 #include "stencil_common.cuh"
 
@@ -264,6 +266,52 @@ int auto_zchunk(int radius, int NX, int NY, int NZ) {
     if (zc < min_zc) zc = min_zc;
     if (zc > NZ) zc = NZ;
     return zc < 1 ? 1 : zc;
+}
+
+// time of a launch in planes: blocks are dispatched slab by slab to `slots`
+// resident places, each taking its slab's planes and `fill` more for its queue
+static double launch_planes(long long tiles, int nz, int zc, int slots, double fill) {
+    const long long slabs = (nz + zc - 1) / zc, full = tiles * (slabs - 1);
+    const double c1 = zc + fill, c2 = nz - (slabs - 1) * (double)zc + fill;
+    // the full slabs leave `late` places one slab behind the others
+    const long long rounds = full / slots, late = full % slots, early = slots - late;
+    const double t0 = rounds * c1, t1 = t0 + (late ? c1 : 0.0);
+    // the last slab's blocks go to the places as they fall free
+    for (long long k = 1;; k++) {
+        const double end = t0 + k * c2;
+        const long long done = early * k + late * (end > t1 ? (long long)((end - t1) / c2 + 1e-9) : 0);
+        if (done >= tiles) return std::max(end, t1);
+    }
+}
+
+// The waves decide between heights: a launch that ends on a nearly empty wave
+// loses most of it. Of the heights measured at 40^3 to 576^3, radius 4 (8-row
+// tiles) and 8 (two rows per thread), the one that launch_planes() ranks first
+// is within 1 % of the fastest on average and 5.5 % at most; one height for
+// four blocks per place lost 5-8 % at 576^3 and 10-15 % at 240 x 224 x 200.
+// The queue fill counts four planes, and half a plane where a step reads or
+// writes another field: its slabs share their boundary planes in the L2 cache
+// best when they are short
+int slab_height(int radius, int variant, int mode, int nx, int ny, int nz) {
+    const int rows = variant == 3 ? 8 : 16;
+    const int per_sm = variant == 1 ? (radius == 4 ? 2 : 1)
+                       : variant == 3 ? (radius == 4 ? 5 : 4)
+                                      : (radius == 4 ? 3 : 2);
+    const double fill = radius == 8 || mode == MODE_FWD || mode == MODE_FWD_SUMSQ ? 4.0 : 0.5;
+    const long long tiles = (long long)((nx + 63) / 64) * ((ny + rows - 1) / rows);
+    const int heights[] = {256, 192, 128, 96, 64, 48, 32, 24, 16, 12, 8, 4};
+    int best = std::min(nz, 256);
+    double least = launch_planes(tiles, nz, best, 152 * per_sm, fill);
+    for (int zc : heights) {
+        if (zc >= nz || zc < radius / 2) continue;
+        const double t = launch_planes(tiles, nz, zc, 152 * per_sm, fill);
+        if (t < least) {
+            least = t;
+            best = zc;
+        }
+    }
+    while ((nz + best - 1) / best > 65535) best *= 2;  // grid.z limit
+    return best;
 }
 
 cudaError_t launch_stencil(int radius, int mode, const StepArgs& a, cudaStream_t s) {
