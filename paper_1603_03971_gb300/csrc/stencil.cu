@@ -285,31 +285,41 @@ static double launch_planes(long long tiles, int nz, int zc, int slots, double f
 }
 
 // The waves decide between heights: a launch that ends on a nearly empty wave
-// loses most of it. Of the heights measured at 40^3 to 576^3, radius 4 (8-row
-// tiles) and 8 (two rows per thread), the one that launch_planes() ranks first
-// is within 1 % of the fastest on average and 5.5 % at most; one height for
-// four blocks per place lost 5-8 % at 576^3 and 10-15 % at 240 x 224 x 200.
-// The queue fill counts four planes, and half a plane where a step reads or
-// writes another field: its slabs share their boundary planes in the L2 cache
-// best when they are short
+// loses most of it. Of the heights measured at 15 shapes from 176 x 77 x 113 to
+// 576^3, radius 4 (8-row tiles) and 8 (two rows per thread), the one that
+// launch_planes() ranks first is within 0.6 % of the fastest on average and
+// 5.5 % at most; one height for four blocks per place lost 5-8 % at 576^3 and
+// 10-15 % at 240 x 224 x 200. The queue fill counts two planes, at radius 4
+// one where a step reads or writes another field, and next to nothing there
+// once the fields leave the L2 cache: slabs share their boundary planes in it
+// best when they are short (576^3 backward + imaging: 740 us at 12 planes, 758
+// at 48). Candidates are the even splits and a list of heights, whose short
+// last slab can fill the places that the others leave
 int slab_height(int radius, int variant, int mode, int nx, int ny, int nz) {
     const int rows = variant == 3 ? 8 : 16;
     const int per_sm = variant == 1 ? (radius == 4 ? 2 : 1)
                        : variant == 3 ? (radius == 4 ? 5 : 4)
                                       : (radius == 4 ? 3 : 2);
-    const double fill = radius == 8 || mode == MODE_FWD || mode == MODE_FWD_SUMSQ ? 4.0 : 0.5;
+    const bool plain = mode == MODE_FWD || mode == MODE_FWD_SUMSQ;
+    const double fill = radius == 8 || plain                    ? 2.0
+                        : (long long)nx * ny * nz > (16LL << 20) ? 0.25
+                                                                 : 1.0;
     const long long tiles = (long long)((nx + 63) / 64) * ((ny + rows - 1) / rows);
-    const int heights[] = {256, 192, 128, 96, 64, 48, 32, 24, 16, 12, 8, 4};
-    int best = std::min(nz, 256);
-    double least = launch_planes(tiles, nz, best, 152 * per_sm, fill);
-    for (int zc : heights) {
-        if (zc >= nz || zc < radius / 2) continue;
+    int best = nz;
+    double least = 1e300;
+    auto consider = [&](int zc) {
         const double t = launch_planes(tiles, nz, zc, 152 * per_sm, fill);
         if (t < least) {
             least = t;
             best = zc;
         }
-    }
+    };
+    const int heights[] = {256, 192, 128, 96, 64, 48, 40, 32, 28, 24, 20, 16, 12, 8, 6, 4};
+    for (int zc : heights)
+        if (zc <= nz) consider(zc);
+    // deeper grids than 64 slabs of the list's heights have no empty waves to save
+    for (int slabs = (nz + 255) / 256; slabs <= std::min(64, std::max(1, nz / 4)); slabs++)
+        consider((nz + slabs - 1) / slabs);
     while ((nz + best - 1) / best > 65535) best *= 2;  // grid.z limit
     return best;
 }
