@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "band.cuh"
+#include "pdl.cuh"
 #include "rtm_internal.h"
 
 namespace rtm {
@@ -93,6 +94,7 @@ __global__ void k_fwd_aux(Geometry G, const float* __restrict__ u_cur, float* u_
                           const float* gz, const int32_t* __restrict__ rec, int nrec,
                           float* data_row, long long src, const float* w_n, float inv_dx3,
                           int* status) {
+    pdl_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < nrec) {
         if (data_row) {
@@ -113,6 +115,7 @@ __global__ void k_bwd_aux(Geometry G, const float* __restrict__ mu_cur, float* m
                           const float* gz, const int32_t* __restrict__ rec, int nrec,
                           const float* __restrict__ r_row, long long src, float* src_adj_slot,
                           float* grad_acc, const float* w_n, float inv_dx3, int* status) {
+    pdl_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < nrec) {
         if (r_row) {
@@ -149,6 +152,7 @@ __global__ void k_image_finalize(Geometry G, const float* __restrict__ slab,
 // boundary band of the model region: gather from a padded field / scatter into it
 __global__ void k_band_copy(Geometry G, int r, float* __restrict__ field,
                             float* __restrict__ band, long long n, int to_field) {
+    pdl_wait();
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += stride) {
         int mx, my, mz;
@@ -171,6 +175,7 @@ __device__ __forceinline__ long long model_row(const Geometry& G, long long zy, 
 
 __global__ void k_illum_add(Geometry G, const float* __restrict__ slab,
                             float* __restrict__ illum, int vec, int padded) {
+    pdl_wait();
     const long long stride = (long long)gridDim.x * blockDim.x;
     if (vec) {
         const int nx4 = G.nx >> 2;
@@ -488,6 +493,7 @@ __global__ void k_finite_scan(const float* __restrict__ f, long long n, int vec,
 // (ky, kz), its threads along x
 __global__ void k_decimate(Geometry G, const float* __restrict__ u, float* __restrict__ coarse,
                            int cx, int cy, int cz) {
+    pdl_wait();
     for (int row = blockIdx.x; row < cy * cz; row += gridDim.x) {
         const int ky = row % cy, kz = row / cy;
         const float* src = u + ((long long)(G.nb + 2 * kz) * G.NY + (G.nb + 2 * ky)) * G.NX + G.nb;
@@ -513,6 +519,7 @@ __device__ __forceinline__ void lin_axis(int j, int nc, int& i0, float& w1) {
 // of the two, or a copy past the last kept column)
 __global__ void k_upsample(Geometry G, const float* __restrict__ coarse, int cx, int cy, int cz,
                            float* __restrict__ slab) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -602,9 +609,8 @@ cudaError_t launch_fwd_aux(const Geometry& G, const float* u_cur, float* u_prev,
                            const int32_t* rec, int nrec, float* data_row, long long src,
                            const float* w_n, float inv_dx3, int* status, cudaStream_t s) {
     const int n = nrec + 1;
-    k_fwd_aux<<<(n + 255) / 256, 256, 0, s>>>(G, u_cur, u_prev, c, gx, gy, gz, rec, nrec,
-                                              data_row, src, w_n, inv_dx3, status);
-    return cudaGetLastError();
+    return launch_next(k_fwd_aux, (n + 255) / 256, 256, 0, s, G, u_cur, u_prev, c, gx, gy, gz, rec,
+                       nrec, data_row, src, w_n, inv_dx3, status);
 }
 
 cudaError_t launch_bwd_aux(const Geometry& G, const float* mu_cur, float* mu_prev,
@@ -613,10 +619,8 @@ cudaError_t launch_bwd_aux(const Geometry& G, const float* mu_cur, float* mu_pre
                            float* src_adj_slot, float* grad_acc, const float* w_n,
                            float inv_dx3, int* status, cudaStream_t s) {
     const int n = nrec + 1;
-    k_bwd_aux<<<(n + 255) / 256, 256, 0, s>>>(G, mu_cur, mu_prev, c, gx, gy, gz, rec, nrec,
-                                              r_row, src, src_adj_slot, grad_acc, w_n,
-                                              inv_dx3, status);
-    return cudaGetLastError();
+    return launch_next(k_bwd_aux, (n + 255) / 256, 256, 0, s, G, mu_cur, mu_prev, c, gx, gy, gz, rec,
+                       nrec, r_row, src, src_adj_slot, grad_acc, w_n, inv_dx3, status);
 }
 
 cudaError_t launch_image_finalize(const Geometry& G, const float* slab, float* image,
@@ -630,8 +634,7 @@ cudaError_t launch_band_copy(const Geometry& G, int r, float* field, float* band
                              cudaStream_t s) {
     const long long n = band_cells(G.nx, G.ny, G.nz, r);
     if (n <= 0) return cudaSuccess;
-    k_band_copy<<<grid_for(n, 256), 256, 0, s>>>(G, r, field, band, n, to_field);
-    return cudaGetLastError();
+    return launch_next(k_band_copy, grid_for(n, 256), 256, 0, s, G, r, field, band, n, to_field);
 }
 
 cudaError_t launch_illum_add(const Geometry& G, const float* slab, float* illum, int padded,
@@ -642,8 +645,8 @@ cudaError_t launch_illum_add(const Geometry& G, const float* slab, float* illum,
     const int vec = (G.nb % 4 == 0) && (G.nx % 4 == 0) &&
                     (reinterpret_cast<uintptr_t>(illum) % 16 == 0) &&
                     (reinterpret_cast<uintptr_t>(slab) % 16 == 0);
-    k_illum_add<<<grid_for(vec ? n / 4 : n, 256), 256, 0, s>>>(G, slab, illum, vec, padded);
-    return cudaGetLastError();
+    return launch_next(k_illum_add, grid_for(vec ? n / 4 : n, 256), 256, 0, s, G, slab, illum, vec,
+                       padded);
 }
 
 cudaError_t launch_image_normalize(const float* image, const float* illum, long long n,
@@ -691,8 +694,7 @@ static int row_blocks(long long rows) { return (int)(rows < 152 * 16 ? rows : 15
 cudaError_t launch_decimate(const Geometry& G, const float* u, float* coarse, cudaStream_t s) {
     const int cx = (G.nx + 1) / 2, cy = (G.ny + 1) / 2, cz = (G.nz + 1) / 2;
     const int tb = cx > 128 ? 256 : 128;
-    k_decimate<<<row_blocks((long long)cy * cz), tb, 0, s>>>(G, u, coarse, cx, cy, cz);
-    return cudaGetLastError();
+    return launch_next(k_decimate, row_blocks((long long)cy * cz), tb, 0, s, G, u, coarse, cx, cy, cz);
 }
 
 cudaError_t launch_upsample(const Geometry& G, const float* coarse, float* slab, cudaStream_t s) {
@@ -700,8 +702,7 @@ cudaError_t launch_upsample(const Geometry& G, const float* coarse, float* slab,
     // a warp per row: 256-thread blocks, eight resident per SM
     const long long rows = (long long)G.ny * G.nz;
     const int blocks = (int)std::min<long long>((rows + 7) / 8, 152 * 8);
-    k_upsample<<<blocks, 256, 0, s>>>(G, coarse, cx, cy, cz, slab);
-    return cudaGetLastError();
+    return launch_next(k_upsample, blocks, 256, 0, s, G, coarse, cx, cy, cz, slab);
 }
 
 cudaError_t launch_misfit(const float* d, const float* obs, long long n, float* resid, double* J,

@@ -14,6 +14,7 @@
 #include <string.h>
 
 #include "../../include/rtm.h"
+#include "pdl.cuh"
 #include "rtm_internal.h"
 
 namespace rtm {
@@ -100,6 +101,7 @@ __global__ void k_fwd_aux_off(Geometry G, const float* __restrict__ u_cur, float
                               const float* __restrict__ c, const float* gx, const float* gy,
                               const float* gz, const rtm_point_taps* __restrict__ taps, int nrec,
                               float* data_row, const float* w_n, float inv_dx3, int* status) {
+    pdl_wait();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp < nrec) {
         if (!data_row) return;
@@ -143,6 +145,7 @@ __global__ void k_bwd_aux_off(Geometry G, const float* __restrict__ mu_cur, floa
                               const float* gz, const rtm_point_taps* __restrict__ taps, int nrec,
                               const float* __restrict__ r_row, float* src_adj_slot,
                               float inv_dx3, int* status) {
+    pdl_wait();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp < nrec) {
         if (!r_row) return;
@@ -182,9 +185,7 @@ cudaError_t launch_fwd_aux_off(const Geometry& G, const float* u_cur, float* u_p
                                float* data_row, const float* w_n, float inv_dx3, int* status,
                                cudaStream_t s) {
     const long long threads = 32LL * (nrec + 1);
-    k_fwd_aux_off<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
-        G, u_cur, u_prev, c, gx, gy, gz, taps, nrec, data_row, w_n, inv_dx3, status);
-    return cudaGetLastError();
+    return launch_next(k_fwd_aux_off, (unsigned)((threads + 255) / 256), 256, 0, s, G, u_cur, u_prev, c, gx, gy, gz, taps, nrec, data_row, w_n, inv_dx3, status);
 }
 
 cudaError_t launch_bwd_aux_off(const Geometry& G, const float* mu_cur, float* mu_prev,
@@ -193,9 +194,7 @@ cudaError_t launch_bwd_aux_off(const Geometry& G, const float* mu_cur, float* mu
                                const float* r_row, float* src_adj_slot, float inv_dx3,
                                int* status, cudaStream_t s) {
     const long long threads = 32LL * (nrec + 1);
-    k_bwd_aux_off<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
-        G, mu_cur, mu_prev, c, gx, gy, gz, taps, nrec, r_row, src_adj_slot, inv_dx3, status);
-    return cudaGetLastError();
+    return launch_next(k_bwd_aux_off, (unsigned)((threads + 255) / 256), 256, 0, s, G, mu_cur, mu_prev, c, gx, gy, gz, taps, nrec, r_row, src_adj_slot, inv_dx3, status);
 }
 
 }  // namespace rtm

@@ -1,0 +1,38 @@
+// Programmatic dependent launch between the kernels of a time step.
+//
+// A launch_next() kernel may be placed on the SMs while the kernel before it
+// in the stream drains: it sets up what needs no data and waits in
+// pdl_wait() until that kernel has completed and its writes are visible. On
+// short steps the launch latency between two dependent kernels is a good part
+// of the step (boundary storage runs seven kernels per time step). Every
+// thread of such a kernel calls pdl_wait() before it touches global memory, so
+// a kernel's completion implies that of all kernels before it.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace rtm {
+
+__device__ __forceinline__ void pdl_wait() {
+    // dependents may be placed from here on: they wait for this kernel anyway
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class... Params, class... Args>
+cudaError_t launch_next(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                        cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
+}  // namespace rtm

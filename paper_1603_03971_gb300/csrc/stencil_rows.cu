@@ -28,6 +28,7 @@
 
 #include "../../include/rtm.h"
 #include "packed_f32x2.cuh"
+#include "pdl.cuh"
 #include "rtm_internal.h"
 #include "stencil_common.cuh"
 #include "tma_encode.h"
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(BX* BY, 2)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();
 
     int issued = zb;  // thread 0: planes [zb, issued) are on their way
     auto issue = [&](int p) {
@@ -381,8 +383,7 @@ cudaError_t launch_t(const StepArgs& a, int* status, cudaStream_t s) {
         return cudaErrorInvalidValue;
     const dim3 grid((a.xend - a.xorg + TX - 1) / TX, (a.yend - a.yorg + TY - 1) / TY,
                     (a.zend - a.zorg + a.zchunk - 1) / a.zchunk);
-    k_stencil_rows<MODE><<<grid, dim3(BX, BY), smem, s>>>(a, M, status);
-    return cudaGetLastError();
+    return launch_next(k_stencil_rows<MODE>, grid, dim3(BX, BY), smem, s, a, M, status);
 }
 
 // encoded maps of this thread, by every encoding argument: a shot launches its

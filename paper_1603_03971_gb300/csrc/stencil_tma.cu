@@ -2,10 +2,9 @@
 //
 // The same leapfrog update and epilogues as k_stencil, with the plane loads
 // moved to the tensor memory accelerator. A block owns a tile of x-y columns
-// and marches a z slab. Variant 2: 256-thread blocks, 64 x 16 tiles at
-// radius 4 (four points per thread) and 32 x 16 at radius 8 (two points per
-// thread). Variant 3: 128-thread blocks, 64 x 8 tiles with four points per
-// thread at both radii. One thread issues
+// and marches a z slab, four points per thread. Variant 2: 256-thread blocks,
+// 64 x 16 tiles (radius 4; radius 8 has its own kernel, stencil_rows.cu).
+// Variant 3: 128-thread blocks, 64 x 8 tiles at both radii. One thread issues
 // 3D bulk tensor copies of the next planes into shared-memory rings, P
 // planes ahead of the one being computed, each slot completed on its
 // mbarrier by the copy's transaction bytes (expect-tx):
@@ -37,6 +36,7 @@
 
 #include "../../include/rtm.h"
 #include "packed_f32x2.cuh"
+#include "pdl.cuh"
 #include "rtm_internal.h"
 #include "stencil_common.cuh"
 #include "tma_encode.h"
@@ -52,16 +52,9 @@ struct TmaMaps {
     CUtensorMap u, prev, c, e1, e2, uh;  // uh: u^n without halo (queue heads)
 };
 
-// V consecutive x points per thread: 4 (16-byte vectors), except in the
-// 16-row tiles at radius 8, whose 256-thread blocks hold 2 (the 2r + G deep
-// register queue of 4-point vectors would allow one block per SM). The 8-row
-// radius-8 tiles keep 4 points per thread: 128 registers, four blocks of 128
-// threads per SM, and half the per-plane overhead and shared-memory x loads
-// per point
-template <int R, int BY = 16>
-__host__ __device__ constexpr int points_per_thread() {
-    return (R == 8 && BY == 16) ? 2 : 4;
-}
+// consecutive x points per thread: 16-byte vectors. At radius 8 the 2r + G deep
+// register queue of 4-point vectors leaves four blocks of 128 threads per SM
+constexpr int kVec = 4;
 
 // tile: 16 threads along x (V floats each) by BYT rows, one row per thread
 // (16 rows: 256 threads, the default; 8 rows: 128 threads, more blocks per SM
@@ -93,44 +86,27 @@ __device__ __forceinline__ Vec<V> vzero() {
 template <int V>
 __device__ __forceinline__ Vec<V> vlds(const float* p) {  // shared memory
     Vec<V> r;
-    if constexpr (V == 4) {
-        const float4 t = *reinterpret_cast<const float4*>(p);
-        r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
-    } else {
-        const float2 t = *reinterpret_cast<const float2*>(p);
-        r.v[0] = t.x, r.v[1] = t.y;
-    }
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
     return r;
 }
 template <int V>
 __device__ __forceinline__ Vec<V> vld_keep(const float* p) {  // read-only global, keep cached
     Vec<V> r;
-    if constexpr (V == 4) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-        r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
-    } else {
-        const float2 t = __ldg(reinterpret_cast<const float2*>(p));
-        r.v[0] = t.x, r.v[1] = t.y;
-    }
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
     return r;
 }
 template <int V>
 __device__ __forceinline__ void vst_stream(float* p, const Vec<V>& a) {
-    if constexpr (V == 4)
-        __stcs(reinterpret_cast<float4*>(p), make_float4(a.v[0], a.v[1], a.v[2], a.v[3]));
-    else
-        __stcs(reinterpret_cast<float2*>(p), make_float2(a.v[0], a.v[1]));
+    __stcs(reinterpret_cast<float4*>(p), make_float4(a.v[0], a.v[1], a.v[2], a.v[3]));
 }
 
 // the Laplacian on packed pairs of points, with half the floating-point
 // instructions. Radius 4 keeps the scalar form's order of sums (two point
-// pairs per thread already give two independent chains); radius 8 (one pair
-// per thread, eight offsets) sums even and odd offsets separately and then
-// adds, halving the dependent chain
-template <int R>
-__host__ __device__ constexpr bool packed_math() {
-    return true;
-}
+// pairs per thread already give two independent chains); radius 8 (eight
+// offsets) sums even and odd offsets separately and then adds, halving the
+// dependent chain
 template <int R>
 __host__ __device__ constexpr bool split_chains() {
     return R == 8;
@@ -161,18 +137,14 @@ __host__ __device__ constexpr int tma_prefetch() {
 
 // the register queue moves once per G planes (2r + G entries, the plane body
 // unrolled G times): 2r / G vector moves per plane instead of 2r. 576^3,
-// radius 8, 2-point vectors: G = 1 / 2 / 4 gave 204.8 / 210.6 / 215.8
-// Gpoint-updates/s; radius 4: G = 1 / 2 gave 318.4 / 320.8 (G = 3 spills
-// under the 80-register cap of three blocks per SM). Radius 8 with 4-point
-// vectors keeps G = 2 (the queue is 72 registers)
-template <int R, int V>
-__host__ __device__ constexpr int queue_group() {
-    return (R == 8 && V == 2) ? 4 : 2;
-}
+// radius 4: G = 1 / 2 gave 318.4 / 320.8 Gpoint-updates/s (G = 3 spills under
+// the 80-register cap of three blocks per SM); at radius 8 the queue is 72
+// registers and G = 4 leaves too little for the rest
+constexpr int kQueueGroup = 2;
 
 template <int R, int MODE, int BY = 16>
 struct TmaCfg {
-    using T = TmaTile<R, points_per_thread<R, BY>(), BY>;
+    using T = TmaTile<R, kVec, BY>;
     static constexpr bool SPLIT = split_ring<R, MODE>();
     static constexpr int NA = aux_planes<MODE>();
     static constexpr int NAH = NA + (SPLIT ? 1 : 0);  // aux ring entries per plane
@@ -239,9 +211,8 @@ __device__ __forceinline__ void tma3(float* dst, const CUtensorMap* map, int x, 
 }
 
 // resident blocks per SM. 16-row tiles: three 256-thread blocks, registers
-// capped at 80 per thread; at radius 4 the forward modes need 73 KB of shared
-// memory, the split-ring backward modes 54 KB; at radius 8 the split ring
-// needs 36-48 KB. 8-row tiles (128 threads): five blocks at radius 4 (102
+// capped at 80 per thread; the radius-4 forward modes need 73 KB of shared
+// memory, the split-ring backward modes 54 KB. 8-row tiles (128 threads): five blocks at radius 4 (102
 // registers, 17-29 KB), four at radius 8 (128 registers, 4-point vectors,
 // 30-53 KB)
 template <int R, int MODE, int BY = 16>
@@ -262,7 +233,7 @@ template <int R, int MODE, int BY, bool STALL = false>
 __global__ void __launch_bounds__(16 * BY, (tma_min_blocks<R, MODE, BY>()))
     k_stencil_tma(const __grid_constant__ StepArgs A, const __grid_constant__ TmaMaps M, int* status,
                   int stall) {
-    constexpr int V = points_per_thread<R, BY>();
+    constexpr int V = kVec;
     using T = TmaTile<R, V, BY>;
     using VT = Vec<V>;
     using C = TmaCfg<R, MODE, BY>;
@@ -301,6 +272,7 @@ __global__ void __launch_bounds__(16 * BY, (tma_min_blocks<R, MODE, BY>()))
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();
 
     // newest u^n plane copied with its halo: the queue head of the last step
     // (joint ring) or the last centre plane (split ring)
@@ -355,7 +327,7 @@ __global__ void __launch_bounds__(16 * BY, (tma_min_blocks<R, MODE, BY>()))
     }
     // queue planes zb - R .. zb + R - 1 straight from global memory
     // queue: plane z0 + t of a group reads entries t .. t + 2r (head 2r + t)
-    constexpr int G = queue_group<R, V>();
+    constexpr int G = kQueueGroup;
     VT q[2 * R + G];
 #pragma unroll
     for (int i = 0; i < 2 * R; i++) {
@@ -410,56 +382,44 @@ __global__ void __launch_bounds__(16 * BY, (tma_min_blocks<R, MODE, BY>()))
 #pragma unroll
             for (int i = 0; i < V; i++) v[R + i] = q[R + t].v[i];
             VT lap;
-            if constexpr (packed_math<R>()) {
-                uint64_t L2[V / 2], L2o[V / 2];
-                const uint64_t a0 = f32x2::pack(A.a[0], A.a[0]);
+            uint64_t L2[V / 2], L2o[V / 2];
+            const uint64_t a0 = f32x2::pack(A.a[0], A.a[0]);
+#pragma unroll
+            for (int j = 0; j < V / 2; j++) {
+                L2[j] = f32x2::mul(a0, f32x2::pack(q[R + t].v[2 * j], q[R + t].v[2 * j + 1]));
+                L2o[j] = 0;  // the bit pattern of two +0.0f
+            }
+#pragma unroll
+            for (int k = 1; k <= R; k++) {
+                const VT ym_ = vlds<V>(S + (R + ty - k) * T::SW + R + V * tx);
+                const VT yp_ = vlds<V>(S + (R + ty + k) * T::SW + R + V * tx);
+                const uint64_t ak = f32x2::pack(A.a[k], A.a[k]);
 #pragma unroll
                 for (int j = 0; j < V / 2; j++) {
-                    L2[j] = f32x2::mul(a0, f32x2::pack(q[R + t].v[2 * j], q[R + t].v[2 * j + 1]));
-                    L2o[j] = 0;  // the bit pattern of two +0.0f
-                }
-#pragma unroll
-                for (int k = 1; k <= R; k++) {
-                    const VT ym_ = vlds<V>(S + (R + ty - k) * T::SW + R + V * tx);
-                    const VT yp_ = vlds<V>(S + (R + ty + k) * T::SW + R + V * tx);
-                    const uint64_t ak = f32x2::pack(A.a[k], A.a[k]);
-#pragma unroll
-                    for (int j = 0; j < V / 2; j++) {
-                        const int i = 2 * j;
-                        const uint64_t px = f32x2::add(f32x2::pack(v[R + i - k], v[R + i + 1 - k]),
-                                                 f32x2::pack(v[R + i + k], v[R + i + 1 + k]));
-                        const uint64_t py = f32x2::add(f32x2::pack(ym_.v[i], ym_.v[i + 1]),
-                                                 f32x2::pack(yp_.v[i], yp_.v[i + 1]));
-                        const uint64_t pz = f32x2::add(f32x2::pack(q[R + t - k].v[i], q[R + t - k].v[i + 1]),
-                                                 f32x2::pack(q[R + t + k].v[i], q[R + t + k].v[i + 1]));
-                        if (split_chains<R>() && (k & 1))
-                            L2o[j] = f32x2::fma(ak, f32x2::add(f32x2::add(px, py), pz), L2o[j]);
-                        else
-                            L2[j] = f32x2::fma(ak, f32x2::add(f32x2::add(px, py), pz), L2[j]);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < V / 2; j++) {
-                    if constexpr (split_chains<R>())
-                        f32x2::unpack(f32x2::add(L2[j], L2o[j]), lap.v[2 * j], lap.v[2 * j + 1]);
+                    const int i = 2 * j;
+                    // at odd offsets the pairs straddle register pairs: two scalar
+                    // sums cost less than moving them together
+                    const uint64_t px =
+                        (k & 1) ? f32x2::pack(v[R + i - k] + v[R + i + k],
+                                              v[R + i + 1 - k] + v[R + i + 1 + k])
+                                : f32x2::add(f32x2::pack(v[R + i - k], v[R + i + 1 - k]),
+                                             f32x2::pack(v[R + i + k], v[R + i + 1 + k]));
+                    const uint64_t py = f32x2::add(f32x2::pack(ym_.v[i], ym_.v[i + 1]),
+                                             f32x2::pack(yp_.v[i], yp_.v[i + 1]));
+                    const uint64_t pz = f32x2::add(f32x2::pack(q[R + t - k].v[i], q[R + t - k].v[i + 1]),
+                                             f32x2::pack(q[R + t + k].v[i], q[R + t + k].v[i + 1]));
+                    if (split_chains<R>() && (k & 1))
+                        L2o[j] = f32x2::fma(ak, f32x2::add(f32x2::add(px, py), pz), L2o[j]);
                     else
-                        f32x2::unpack(L2[j], lap.v[2 * j], lap.v[2 * j + 1]);
+                        L2[j] = f32x2::fma(ak, f32x2::add(f32x2::add(px, py), pz), L2[j]);
                 }
-            } else {
+            }
 #pragma unroll
-                for (int i = 0; i < V; i++) lap.v[i] = A.a[0] * q[R + t].v[i];
-#pragma unroll
-                for (int k = 1; k <= R; k++) {
-                    const VT ym_ = vlds<V>(S + (R + ty - k) * T::SW + R + V * tx);
-                    const VT yp_ = vlds<V>(S + (R + ty + k) * T::SW + R + V * tx);
-#pragma unroll
-                    for (int i = 0; i < V; i++) {
-                        const float px = v[R + i - k] + v[R + i + k];
-                        const float py = ym_.v[i] + yp_.v[i];
-                        const float pz = q[R + t - k].v[i] + q[R + t + k].v[i];
-                        lap.v[i] = fmaf(A.a[k], (px + py) + pz, lap.v[i]);
-                    }
-                }
+            for (int j = 0; j < V / 2; j++) {
+                if constexpr (split_chains<R>())
+                    f32x2::unpack(f32x2::add(L2[j], L2o[j]), lap.v[2 * j], lap.v[2 * j + 1]);
+                else
+                    f32x2::unpack(L2[j], lap.v[2 * j], lap.v[2 * j + 1]);
             }
             const VT up = vlds<V>(aux + aux_off);
             const VT cc = vlds<V>(aux + C::APLANE + aux_off);
@@ -550,66 +510,7 @@ __global__ void __launch_bounds__(16 * BY, (tma_min_blocks<R, MODE, BY>()))
     }
 }
 
-// ---- host side: tensor maps ---------------------------------------------------
-cudaError_t encode_map(CUtensorMap* m, const float* base, int nx, int ny, int nz, int bx,
-                       int by);
-
-// A shot launches the stencil thousands of times on the same few buffers, so
-// the encoded maps are kept per thread, keyed by every encoding argument, and
-// reused (least recently encoded entry replaced)
-struct MapKey {
-    const float* base;
-    int nx, ny, nz, bx, by;
-    bool operator==(const MapKey& o) const {
-        return base == o.base && nx == o.nx && ny == o.ny && nz == o.nz && bx == o.bx &&
-               by == o.by;
-    }
-};
-constexpr int kMapCache = 64;
-struct MapCache {
-    MapKey key[kMapCache];
-    CUtensorMap map[kMapCache];
-    int n = 0, next = 0;
-};
-thread_local MapCache t_maps;
-
-cudaError_t make_map(CUtensorMap* m, const float* base, int nx, int ny, int nz, int bx, int by) {
-    const MapKey k{base, nx, ny, nz, bx, by};
-    MapCache& c = t_maps;
-    for (int i = 0; i < c.n; i++)
-        if (c.key[i] == k) {
-            *m = c.map[i];
-            return cudaSuccess;
-        }
-    cudaError_t e = encode_map(m, base, nx, ny, nz, bx, by);
-    if (e != cudaSuccess) return e;
-    int slot;
-    if (c.n < kMapCache) {
-        slot = c.n++;
-    } else {
-        slot = c.next;
-        c.next = (c.next + 1) % kMapCache;
-    }
-    c.key[slot] = k;
-    c.map[slot] = *m;
-    return cudaSuccess;
-}
-
-cudaError_t encode_map(CUtensorMap* m, const float* base, int nx, int ny, int nz, int bx,
-                       int by) {
-    EncodeTiledFn f = tma_encoder();
-    if (!f) return cudaErrorNotSupported;
-    if (((uintptr_t)base % 16) || (nx % 4)) return cudaErrorInvalidValue;
-    const cuuint64_t dims[3] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz};
-    const cuuint64_t strides[2] = {(cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
-    const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = f(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides,
-                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
+// ---- host side ---------------------------------------------------------------
 // dynamic shared memory and carveout of a TMA stencil instance
 template <class K>
 cudaError_t set_tma_attrs(K kernel, int smem) {
@@ -621,7 +522,7 @@ cudaError_t set_tma_attrs(K kernel, int smem) {
 
 template <int R, int MODE, int BY>
 cudaError_t launch_tma_t(const StepArgs& a, int* status, cudaStream_t s) {
-    using T = TmaTile<R, points_per_thread<R, BY>(), BY>;
+    using T = TmaTile<R, kVec, BY>;
     constexpr int smem = TmaCfg<R, MODE, BY>::SMEM;
     static_assert(rings_fit<R, MODE, BY>(), "rings do not fit the resident blocks");
     static bool attr = false;
@@ -633,22 +534,22 @@ cudaError_t launch_tma_t(const StepArgs& a, int* status, cudaStream_t s) {
     TmaMaps M;
     memset(&M, 0, sizeof M);
     cudaError_t e;
-    if ((e = make_map(&M.u, a.u_cur, a.NX, a.NY, a.NZ, T::TX + 2 * R, T::TY + 2 * R)) != cudaSuccess)
+    if ((e = tma_map3(&M.u, a.u_cur, a.NX, a.NY, a.NZ, T::TX + 2 * R, T::TY + 2 * R)) != cudaSuccess)
         return e;
-    if ((e = make_map(&M.prev, a.u_prev, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
+    if ((e = tma_map3(&M.prev, a.u_prev, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
     if (TmaCfg<R, MODE, BY>::SPLIT &&
-        (e = make_map(&M.uh, a.u_cur, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess)
+        (e = tma_map3(&M.uh, a.u_cur, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess)
         return e;
-    if ((e = make_map(&M.c, a.c, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
+    if ((e = tma_map3(&M.c, a.c, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
     if (MODE == MODE_BWD_IMAGE) {
-        if ((e = a.snap_padded ? make_map(&M.e1, a.snap, a.NX, a.NY, a.NZ, T::TX, T::TY)
-                               : make_map(&M.e1, a.snap, a.NX, a.ny, a.nz, T::TX, T::TY)) !=
+        if ((e = a.snap_padded ? tma_map3(&M.e1, a.snap, a.NX, a.NY, a.NZ, T::TX, T::TY)
+                               : tma_map3(&M.e1, a.snap, a.NX, a.ny, a.nz, T::TX, T::TY)) !=
             cudaSuccess)
             return e;
-        if ((e = make_map(&M.e2, a.acc, a.NX, a.ny, a.nz, T::TX, T::TY)) != cudaSuccess) return e;
+        if ((e = tma_map3(&M.e2, a.acc, a.NX, a.ny, a.nz, T::TX, T::TY)) != cudaSuccess) return e;
     } else if (MODE == MODE_BWD_GRAD) {
-        if ((e = make_map(&M.e1, a.snap, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
-        if ((e = make_map(&M.e2, a.acc, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
+        if ((e = tma_map3(&M.e1, a.snap, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
+        if ((e = tma_map3(&M.e2, a.acc, a.NX, a.NY, a.NZ, T::TX, T::TY)) != cudaSuccess) return e;
     }
     dim3 block(T::BX, T::BY);
     dim3 grid((a.xend - a.xorg + T::TX - 1) / T::TX, (a.yend - a.yorg + T::TY - 1) / T::TY,
@@ -664,12 +565,11 @@ cudaError_t launch_tma_t(const StepArgs& a, int* status, cudaStream_t s) {
                 if (e != cudaSuccess) return e;
                 attr_stall = true;
             }
-            k_stencil_tma<R, MODE, BY, true><<<grid, block, smem, s>>>(a, M, status, stall);
-            return cudaGetLastError();
+            return launch_next(k_stencil_tma<R, MODE, BY, true>, grid, block, smem, s, a, M, status,
+                               stall);
         }
     }
-    k_stencil_tma<R, MODE, BY><<<grid, block, smem, s>>>(a, M, status, -1);
-    return cudaGetLastError();
+    return launch_next(k_stencil_tma<R, MODE, BY>, grid, block, smem, s, a, M, status, -1);
 }
 
 template <int R, int BY>
@@ -716,7 +616,7 @@ cudaError_t launch_stencil_tma(int radius, int mode, const StepArgs& a, int* sta
     }
     switch (radius) {
         case 4: return launch_tma_r<4, 16>(mode, a, status, s);
-        case 8: return launch_tma_r<8, 16>(mode, a, status, s);
+        case 8: return launch_stencil_rows(mode, a, status, s);
         default: return cudaErrorInvalidValue;
     }
 }
