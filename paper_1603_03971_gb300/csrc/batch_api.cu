@@ -17,30 +17,41 @@ using namespace rtm;
 namespace {
 
 constexpr size_t kAlB = 256;
-// automatic z-slab height of a work item, per wave: the tallest slab (the
-// whole column first) that still gives every phase step at least
-// kItemsPerBlock items per resident block. Each step of a shot waits for all
-// items of its previous step, so too few items leave blocks idle at every
-// step; too short slabs repeat the 2r-plane queue warm-up. Measured with the
-// TMA kernel: 4 shots of 256 x 256 x 320 padded, whole columns / 256 / 128
-// planes: 137 / 174 / 270 Gpoint-updates/s (radius 4); the 32-shot radius-8
-// workload: whole columns 173.8, 128 planes 167.4
 constexpr int kBatchZchunk = 128;  // the workspace's sizing value
-constexpr int kItemsPerBlock = 3;
 
-int wave_zchunk(const std::vector<BatchShot>& shots, int first, int last, int grid) {
+// Automatic z-slab height of a work item, per wave of shots on `blocks`
+// resident blocks. A phase step costs its items' planes, each item four more
+// for its queue and its turn at the work queue; a shot waits for all items of
+// its previous step, which leaves blocks idle for about half an item's time,
+// shared by the shots that can run meanwhile; one shot runs in whole rounds of
+// items. Over ten batches of 1 to 6 shots of 100^3 to 280^3 (radius 4 and 8,
+// heights 8 to 300) the height ranked first is within 1 % of the fastest on
+// average, 2.7 % at most; the tallest slab with three items per block lost
+// 2 % on six shots of 170-280 cells, 40 % on five of 100-140
+int wave_zchunk(const std::vector<BatchShot>& shots, int first, int last, int blocks) {
     int nzmax = 1;
     for (int i = first; i < last; i++) nzmax = std::max(nzmax, shots[i].NZ);
-    const int cand[] = {nzmax, 512, 384, 256, 192, 128, 96, 64};
-    int best = 64;
+    const int cand[] = {nzmax, 384, 256, 192, 128, 96, 64, 48, 32, 24, 16, 12, 8};
+    constexpr double kItemPlanes = 4.0, kTail = 0.5;
+    int best = nzmax;
+    double least = 1e300;
     for (int zc : cand) {
         if (zc > nzmax) continue;
-        long long items = 0;
-        for (int i = first; i < last; i++)
-            items += (long long)shots[i].tiles_x * shots[i].tiles_y *
-                     ((shots[i].NZ + zc - 1) / zc);
-        if (items >= (long long)kItemsPerBlock * grid) return zc;
-        best = zc;
+        double work = 0.0, items = 0.0;
+        for (int i = first; i < last; i++) {
+            const double tiles = (double)shots[i].tiles_x * shots[i].tiles_y;
+            const int slabs = (shots[i].NZ + zc - 1) / zc;
+            items += tiles * slabs;
+            work += tiles * (shots[i].NZ + kItemPlanes * slabs);
+        }
+        const double item = zc + kItemPlanes;
+        const double t = last - first == 1
+                             ? ceil(items / blocks) * item
+                             : std::max(item, work / blocks + kTail * item / (last - first));
+        if (t < least) {
+            least = t;
+            best = zc;
+        }
     }
     return best;
 }
@@ -101,8 +112,10 @@ rtm_status check_batch(const rtm_params* p, int nshots, const rtm_aperture* sh) 
 // the batched kernel: TMA plane loads wherever the driver provides tensor maps
 // (unless the vector-load variant is selected for the radius)
 bool batch_uses_tma(int radius) { return tma_available() && tuning_variant(radius) != 1; }
-// tile rows of the TMA kernel: 8 when the 8-row tile (variant 3) is selected
-int batch_tile_rows(int radius) { return tuning_variant(radius) == 3 ? 8 : 16; }
+// tile rows of the TMA kernel: 8 unless the 16-row tile (variant 2) is
+// selected. Six shots of 170-280 cells: 17.8 against 20.8 ms at radius 4; at
+// radius 8 both take 23.2
+int batch_tile_rows(int radius) { return tuning_variant(radius) == 2 ? 16 : 8; }
 
 Plan make_plan(const rtm_params* p, int nshots, const rtm_aperture* sh, size_t budget,
                int zchunk) {

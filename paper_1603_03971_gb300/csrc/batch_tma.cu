@@ -2,10 +2,10 @@
 // schedule of batch.cu (phase steps of every shot in a wave, per-shot step
 // counters, bounded waits) around the plane march of the TMA stencil.
 //
-// A work item is one tile (TX columns x 16 or 8 rows x a z slab) of one shot
-// at one phase step. The block's thread 0 copies each plane with the 3D-in-4D bulk
-// tensor copy: the centre plane of u^n with its r-wide halo into a ring of
-// P + 1 slots, and, into a second ring, the tile of u^{n-1}, c, the queue head
+// A work item is one tile (64 columns x 16 or 8 rows x a z slab) of one shot
+// at one phase step. The block's thread 0 copies each plane with the 3D-in-4D
+// bulk tensor copy into a ring of P + 1 slots, one mbarrier each: the centre
+// plane of u^n with its r-wide halo, the tiles of u^{n-1}, c, the queue head
 // (u^n at z + r, no halo) and, on imaging steps, the snapshot and image tiles.
 // Each shot's padded fields (c, both field pairs, all checkpoints) sit one
 // stride apart in the workspace, and so do its slabs (snapshots, image), so
@@ -15,6 +15,13 @@
 // increment; the reading thread acquires the counter and then fences the
 // generic proxy against the asynchronous one before its copies read them.
 //
+// The march is bound by instruction issue as much as by its copies, so what a
+// plane does besides the step (source, receivers, checkpoint, snapshot, image)
+// is decided once per item and costs one branch per plane, the first step of a
+// recursion, which reads no fields, is its own instance, and plane z + P is
+// issued before the wait for plane z. Six radius-8 shots of 170-280 cells
+// (padded), 24 steps: 27.8 -> 23.2 ms; radius 4: 20.8 -> 17.8.
+//
 // The ring slots and mbarrier phases run on across items: every copy an item
 // issues is waited for within the item, so the next item reuses the slots in
 // order. Every wait is bounded and shares the abort flag of the launch.
@@ -23,7 +30,8 @@
 #include <string.h>
 
 #include "batch_internal.h"
-#include "packed_f32x2.cuh"
+#include "star_rows.cuh"
+#include "stencil_common.cuh"
 #include "tma_encode.h"
 #include "wait_clock.cuh"
 
@@ -33,71 +41,30 @@ namespace {
 
 constexpr long long kPlaneWaitLimit = 1LL << 26;
 
-// tile: 16 threads along x (V points each) by BYT rows (16: 256 threads,
-// three blocks per SM; 8: 128 threads, five blocks per SM at radius 4 and
-// four at radius 8, where the 8-row tiles keep 4-point vectors)
+// tile: 16 threads along x, four points each, by BYT rows. 16-row tiles: at
+// radius 8 two rows per thread (128 threads, two blocks per SM, see
+// stencil_rows.cu), at radius 4 one (256 threads, three blocks). 8-row tiles:
+// 128 threads, five blocks per SM at radius 4, four at radius 8
 template <int R, int BYT = 16>
 struct BT {
-    static constexpr int V = (R == 8 && BYT == 16) ? 2 : 4;  // x points per thread
-    static constexpr int BX = 16, BY = BYT;
-    static constexpr int TX = V * BX, TY = BY;
+    static constexpr int ROWS = (R == 8 && BYT == 16) ? 2 : 1;  // rows per thread
+    static constexpr int BX = 16, BY = BYT / ROWS;              // threads
+    static constexpr int TX = 4 * BX, TY = BYT;
     static constexpr int SW = TX + 2 * R, SH = TY + 2 * R;
-    static constexpr int HX = R / V;
-    static constexpr int P = R == 8 ? 2 : 1;  // planes in flight (three blocks fit per SM)
+    static constexpr int P = R == 8 ? 2 : 1;  // planes in flight
     static constexpr int NS = P + 1;
     static constexpr int UPLANE = SH * SW, APLANE = TY * TX;
     static constexpr int NAH = 5;  // u^{n-1}, c, queue head, snapshot, image
     static constexpr int SMEM = (NS * UPLANE + NS * NAH * APLANE) * 4;
-    static constexpr int G = R == 8 ? (V == 2 ? 4 : 2) : 1;  // queue moves once per G planes
-    static constexpr int MINB = BY == 16 ? 3 : (R == 8 ? 4 : 5);
-    static_assert(R % 4 == 0 && R % V == 0 && (BY == 16 || BY == 8), "tile");
+    static constexpr int G = R == 8 ? 2 : 1;  // queue moves once per G planes
+    static constexpr int MINB = ROWS == 2 ? 2 : BYT == 16 ? 3 : (R == 8 ? 4 : 5);
+    static_assert(R % 4 == 0 && (BYT == 16 || BYT == 8), "tile");
     static_assert(MINB * (SMEM + 1024 + 1024) <= 228 * 1024, "rings do not fit the resident blocks");
 };
 
-template <int V>
-struct Vec {
-    float v[V];
-};
-template <int V>
-__device__ __forceinline__ Vec<V> vzero() {
-    Vec<V> r;
-#pragma unroll
-    for (int i = 0; i < V; i++) r.v[i] = 0.f;
-    return r;
-}
-template <int V>
-__device__ __forceinline__ Vec<V> vlds(const float* p) {  // shared memory
-    Vec<V> r;
-    if constexpr (V == 4) {
-        const float4 t = *reinterpret_cast<const float4*>(p);
-        r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
-    } else {
-        const float2 t = *reinterpret_cast<const float2*>(p);
-        r.v[0] = t.x, r.v[1] = t.y;
-    }
-    return r;
-}
-template <int V>
-__device__ __forceinline__ Vec<V> vld_cg(const float* p) {  // global, coherent at L2
-    Vec<V> r;
-    if constexpr (V == 4) {
-        const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
-        r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
-    } else {
-        const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
-        r.v[0] = t.x, r.v[1] = t.y;
-    }
-    return r;
-}
 // global store, streaming (evict first): every field a step writes is read
 // again only in a later step, after the rest of the wave has gone through L2
-template <int V>
-__device__ __forceinline__ void vst(float* p, const Vec<V>& a) {
-    if constexpr (V == 4)
-        __stcs(reinterpret_cast<float4*>(p), make_float4(a.v[0], a.v[1], a.v[2], a.v[3]));
-    else
-        __stcs(reinterpret_cast<float2*>(p), make_float2(a.v[0], a.v[1]));
-}
+__device__ __forceinline__ void vst(float* p, const F4& a) { st_stream(p, a); }
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -139,9 +106,6 @@ __device__ __forceinline__ void bar_drain(uint64_t* b, uint32_t parity) {
     const unsigned long long t0 = wait_now();
     for (long long i = 0; i < kPlaneWaitLimit; i++)
         if (bar_poll(a, parity) || wait_expired(i, t0)) return;
-}
-__device__ __forceinline__ void bar_arrive(uint64_t* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_u32(b)) : "memory");
 }
 __device__ __forceinline__ void tma4(float* dst, const CUtensorMap* map, int x, int y, int z,
                                      int f, uint64_t* bar) {
@@ -185,13 +149,13 @@ struct RingPos {
 // field indices in a shot's field stack
 constexpr int F_C = 0, F_F0 = 1, F_F1 = 2, F_M0 = 3, F_M1 = 4, F_CK = 5;
 
-template <int R, int BY>
+// ZERO: the first step of a recursion, which reads no fields
+template <int R, int BY, bool ZERO>
 __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchPhase ph, int tile,
-                         int s, float* uring, float* aring, uint64_t* ubar, uint64_t* abar,
+                         int s, float* uring, float* aring, uint64_t* bar,
                          RingPos& rp) {
     using B = BT<R, BY>;
-    constexpr int V = B::V;
-    using VT = Vec<V>;
+    constexpr int ROWS = B::ROWS;
     const BatchArgs& A = T.a;
     const CUtensorMap* mU = &T.maps[s][0];
     const CUtensorMap* mP = &T.maps[s][1];
@@ -201,16 +165,20 @@ __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchP
     const int by = (tile / S.tiles_x) % S.tiles_y;
     const int bz = tile / (S.tiles_x * S.tiles_y);
     const int x0 = bx * B::TX, y0 = by * B::TY;
-    const int x = x0 + V * tx, y = y0 + ty;
+    const int x = x0 + 4 * tx, y = y0 + ROWS * ty;
     const int zb = bz * A.zchunk;
     const int ze = min(S.NZ, zb + A.zchunk);
-    const bool own = x < S.NX && y < S.NY;
+    bool own[ROWS], ym[ROWS];
+#pragma unroll
+    for (int h = 0; h < ROWS; h++) {
+        own[h] = x < S.NX && y + h < S.NY;
+        ym[h] = y + h >= S.nb && y + h < S.nb + S.ny;
+    }
     const size_t plane = (size_t)S.NX * S.NY;
     const size_t col = (size_t)y * S.NX + x;
 
     // buffers of this phase step (pointers for the stores, stack indices for the copies)
     int icur, iprev;
-    bool zero_in = false;
     float* ck_a = nullptr;  // forward: checkpoint destinations
     float* ck_b = nullptr;
     float* snap_w = nullptr;  // recompute: snapshot to write
@@ -219,7 +187,6 @@ __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchP
         const int n = ph.step;
         icur = (n & 1) ? F_F0 : F_F1;
         iprev = (n & 1) ? F_F1 : F_F0;
-        zero_in = (n == 0);
         if ((n + 1) % A.ckpt_every == 0 && n + 1 < A.nt) {
             const size_t j = (size_t)((n + 1) / A.ckpt_every);
             ck_a = S.ckpt + ((j - 1) * 2 + 0) * S.fstride;
@@ -230,7 +197,6 @@ __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchP
         if (ph.seg == 0) {
             ia = F_F0;
             ib = F_F1;
-            zero_in = (ph.local == 0);
         } else {
             ia = F_CK + (ph.seg - 1) * 2;
             ib = ia + 1;
@@ -242,45 +208,37 @@ __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchP
         const int bi = A.nt - ph.step;  // 0 for m = nt
         icur = (bi & 1) ? F_M0 : F_M1;
         iprev = (bi & 1) ? F_M1 : F_M0;
-        zero_in = (ph.step == A.nt);
         if (ph.step % A.image_every == 0) snap_r = ph.local;
     }
     const float* cur = S.c + (size_t)icur * S.fstride;
     float* prev = const_cast<float*>(S.c) + (size_t)iprev * S.fstride;
     // zero inputs: the first step of a recursion reads nothing and clears the
     // buffer that holds the step before it
-    float* clear = zero_in ? const_cast<float*>(cur) : nullptr;
-    const bool rd = own && !zero_in;
+    float* clear = ZERO ? const_cast<float*>(cur) : nullptr;
     const int img_slab = A.ckpt_every;
 
-    const bool xm = (x + V - 1 >= S.nb) && (x < S.nb + S.nx);
-    const bool ym = (y >= S.nb) && (y < S.nb + S.ny);
+    const bool xm = (x + 3 >= S.nb) && (x < S.nb + S.nx);
     const size_t slab_col = (size_t)(y - S.nb) * S.NX + x;
     const size_t slab_plane = (size_t)S.ny * S.NX;
 
     // copies of plane p: centre plane of u^n with halo; the tiles of u^{n-1},
     // c and the queue head (u^n at p + r); the snapshot and image tiles
-    const uint32_t abytes =
-        (uint32_t)((zero_in ? 1 : 3) + (snap_r >= 0 ? 2 : 0)) * B::APLANE * 4;
+    const uint32_t bytes =
+        (uint32_t)((ZERO ? 0 : B::UPLANE) + ((ZERO ? 1 : 3) + (snap_r >= 0 ? 2 : 0)) * B::APLANE) * 4;
     int nissued = 0;  // planes of this item copied (thread 0)
     auto issue = [&](int p) {
         const int sl = rp.issue;
         float* abase = aring + sl * B::NAH * B::APLANE;
-        if (!zero_in) {
-            bar_expect(&ubar[sl], B::UPLANE * 4);
-            tma4(uring + sl * B::UPLANE, mU, x0 - R, y0 - R, p, icur, &ubar[sl]);
-        } else {
-            bar_arrive(&ubar[sl]);  // no halo plane: complete the phase, keep the rings in step
-        }
-        bar_expect(&abar[sl], abytes);
-        tma4(abase + B::APLANE, mP, x0, y0, p, F_C, &abar[sl]);
-        if (!zero_in) {
-            tma4(abase, mP, x0, y0, p, iprev, &abar[sl]);
-            tma4(abase + 2 * B::APLANE, mP, x0, y0, p + R, icur, &abar[sl]);
+        bar_expect(&bar[sl], bytes);
+        tma4(abase + B::APLANE, mP, x0, y0, p, F_C, &bar[sl]);
+        if constexpr (!ZERO) {
+            tma4(uring + sl * B::UPLANE, mU, x0 - R, y0 - R, p, icur, &bar[sl]);
+            tma4(abase, mP, x0, y0, p, iprev, &bar[sl]);
+            tma4(abase + 2 * B::APLANE, mP, x0, y0, p + R, icur, &bar[sl]);
         }
         if (snap_r >= 0) {
-            tma4(abase + 3 * B::APLANE, mS, x0, y0 - S.nb, p - S.nb, snap_r, &abar[sl]);
-            tma4(abase + 4 * B::APLANE, mS, x0, y0 - S.nb, p - S.nb, img_slab, &abar[sl]);
+            tma4(abase + 3 * B::APLANE, mS, x0, y0 - S.nb, p - S.nb, snap_r, &bar[sl]);
+            tma4(abase + 4 * B::APLANE, mS, x0, y0 - S.nb, p - S.nb, img_slab, &bar[sl]);
         }
         rp.issue = sl + 1 == B::NS ? 0 : sl + 1;
         nissued++;
@@ -293,28 +251,51 @@ __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchP
         for (int p = zb; p < zb + B::P && p < ze; p++) issue(p);
     }
 
-    Vec<V> gxy = vzero<V>();
-    if (own) {
-        const float gyv = S.gy[y];
+    F4 gxy[ROWS];
 #pragma unroll
-        for (int i = 0; i < V; i++) gxy.v[i] = S.gx[x + i] * gyv;
+    for (int h = 0; h < ROWS; h++) {
+        gxy[h] = zero4();
+        if (own[h]) {
+            const float gyv = S.gy[y + h];
+#pragma unroll
+            for (int i = 0; i < 4; i++) gxy[h].v[i] = S.gx[x + i] * gyv;
+        }
     }
     // queue: plane z0 + t of a group reads entries t .. t + 2r (head 2r + t)
     constexpr int G = B::G;
-    VT q[2 * R + G];
+    F4 q[ROWS][2 * R + G];
 #pragma unroll
-    for (int i = 0; i < 2 * R; i++) {
-        const int zz = zb - R + i;
-        q[i] = (rd && zz >= 0 && zz < S.NZ) ? vld_cg<V>(cur + (size_t)zz * plane + col)
-                                            : vzero<V>();
+    for (int h = 0; h < ROWS; h++) {
+#pragma unroll
+        for (int i = 0; i < 2 * R; i++) {
+            const int zz = zb - R + i;
+            q[h][i] = (!ZERO && own[h] && zz >= 0 && zz < S.NZ)
+                          ? ld_l2(cur + (size_t)zz * plane + col + (size_t)h * S.NX)
+                          : zero4();
+        }
+#pragma unroll
+        for (int i = 2 * R; i < 2 * R + G; i++) q[h][i] = zero4();
     }
-#pragma unroll
-    for (int i = 2 * R; i < 2 * R + G; i++) q[i] = vzero<V>();
 
+    // what a plane does besides the step, decided once per item: the planes
+    // march in the block's registers and the shot record stays in shared memory
+    enum { CLEAR = 1, CKPT = 2, SNAP = 4, IMAGE = 8 };
+    const int what = (ZERO ? CLEAR : 0) | (ck_a ? CKPT : 0) | (snap_w ? SNAP : 0) |
+                     (snap_r >= 0 ? IMAGE : 0);
     const bool do_src = ph.kind != PH_BWD;
     const float w = do_src ? A.wavelet[ph.step] : 0.f;
-    const int own_off = (R + ty) * B::SW + R + V * tx;
-    const int aux_off = ty * B::TX + V * tx;
+    // the plane of the source, if one of this thread's cells holds it, and of
+    // the receivers, if they take or give data in this step (-1: none)
+    const int src_plane = do_src && S.src_x >= x && S.src_x < x + 4 && S.src_y >= y &&
+                                  S.src_y < y + ROWS
+                              ? S.src_z
+                              : -1;
+    const int rec_plane = ph.kind == PH_BWD || (ph.kind == PH_FWD && S.data) ? S.rec_z : -1;
+    const float* gz = S.gz;
+    const int row_len = S.NX, zlo = S.nb, zhi = S.nb + S.nz;
+    float* pout = prev + (size_t)zb * plane + col;  // this plane's cells of the new field
+    const int own_off = (R + ROWS * ty) * B::SW + R + 4 * tx;
+    const int aux_off = ROWS * ty * B::TX + 4 * tx;
     bool ok = true;  // the same in every thread (block-wide vote each plane)
     int nwaited = 0;
 
@@ -324,130 +305,99 @@ __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchP
             const int z = z0 + t;
             if (z >= ze || !ok) break;  // the same for every thread of the block
             const int sl = rp.slot;
-            bool got = bar_wait(&ubar[sl], (uint32_t)rp.phase, A.ctrl);
-            got = bar_wait(&abar[sl], (uint32_t)rp.phase, A.ctrl) && got;
-            // block-wide vote; also every thread is past plane z - 1, whose
-            // slots plane z + P reuses
-            ok = __syncthreads_and(got) != 0;
-            if (!ok) break;
-            nwaited++;
             if (tid == 0 && z + B::P < ze) issue(z + B::P);
-            const float* Sm = uring + sl * B::UPLANE;
-            const float* aux = aring + sl * B::NAH * B::APLANE;
-            q[2 * R + t] = zero_in ? vzero<V>() : vlds<V>(aux + 2 * B::APLANE + aux_off);
+            const bool got = bar_wait(&bar[sl], (uint32_t)rp.phase, A.ctrl);
+            const float* Sm = uring + sl * B::UPLANE + own_off;
+            const float* aux = aring + sl * B::NAH * B::APLANE + aux_off;
+#pragma unroll
+            for (int h = 0; h < ROWS; h++)
+                q[h][2 * R + t] = ZERO ? zero4() : lds4(aux + 2 * B::APLANE + h * B::TX);
 
-            if (own) {
-                VT lap = vzero<V>();
-                if (!zero_in) {
-                    float v[V + 2 * R];
+            if (own[0] && got) {
+                F4 lap[ROWS];
+                if constexpr (!ZERO) {
+                    star_rows<R, ROWS>(Sm, B::SW, q, t, A.a, lap);
+                } else {
 #pragma unroll
-                    for (int h = 0; h < B::HX; h++) {
-                        const VT l = vlds<V>(Sm + (R + ty) * B::SW + V * tx + V * h);
-                        const VT r = vlds<V>(Sm + (R + ty) * B::SW + R + V * tx + V + V * h);
+                    for (int h = 0; h < ROWS; h++) lap[h] = zero4();
+                }
+                const float gzv = __ldg(gz + z);
 #pragma unroll
-                        for (int i = 0; i < V; i++) {
-                            v[V * h + i] = l.v[i];
-                            v[R + V + V * h + i] = r.v[i];
+                for (int h = 0; h < ROWS; h++) {
+                    if (!own[h]) break;
+                    const F4 up = ZERO ? zero4() : lds4(aux + h * B::TX);
+                    const F4 cc = lds4(aux + B::APLANE + h * B::TX);
+                    const F4& qc = q[h][R + t];
+                    F4 out;
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const float g = gxy[h].v[i] * gzv;
+                        out.v[i] = g * fmaf(cc.v[i], lap[h].v[i], 2.0f * qc.v[i]) -
+                                   (g * g) * up.v[i];
+                    }
+                    // source injection: u^{n+1}[s] += c_s w^n / dx^3
+                    if (z == src_plane && y + h == S.src_y) {
+#pragma unroll
+                        for (int i = 0; i < 4; i++)
+                            if (x + i == S.src_x) out.v[i] += cc.v[i] * w * A.inv_dx3;
+                    }
+                    if (z == rec_plane && ym[h]) {
+                        const size_t row = ((size_t)(y + h - S.nb)) * S.nx;
+                        const size_t step = (size_t)S.ny * S.nx;
+                        if (ph.kind == PH_BWD) {
+                            // adjoint injection: mu^m[rec] += c g r^{m-1} / dx^3
+                            const float* d = S.dobs + (size_t)(ph.step - 1) * step + row;
+#pragma unroll
+                            for (int i = 0; i < 4; i++) {
+                                const int xi = x + i - S.nb;
+                                if (xi >= 0 && xi < S.nx)
+                                    out.v[i] += cc.v[i] * (gxy[h].v[i] * gzv) * d[xi] * A.inv_dx3;
+                            }
+                        } else {
+                            float* d = S.data + (size_t)ph.step * step + row;
+#pragma unroll
+                            for (int i = 0; i < 4; i++) {
+                                const int xi = x + i - S.nb;
+                                if (xi >= 0 && xi < S.nx) d[xi] = out.v[i];
+                            }
                         }
                     }
-#pragma unroll
-                    for (int i = 0; i < V; i++) v[R + i] = q[R + t].v[i];
-                    // the Laplacian on packed point pairs (f32x2); radius 8
-                    // sums even and odd offsets in two chains, then adds
-                    namespace P2 = f32x2;
-                    uint64_t L2[V / 2], L2o[V / 2];
-                    const uint64_t a0 = P2::pack(A.a[0], A.a[0]);
-#pragma unroll
-                    for (int j = 0; j < V / 2; j++) {
-                        L2[j] = P2::mul(a0, P2::pack(q[R + t].v[2 * j], q[R + t].v[2 * j + 1]));
-                        L2o[j] = 0;  // two +0.0f
-                    }
-#pragma unroll
-                    for (int k = 1; k <= R; k++) {
-                        const VT ym_ = vlds<V>(Sm + (R + ty - k) * B::SW + R + V * tx);
-                        const VT yp_ = vlds<V>(Sm + (R + ty + k) * B::SW + R + V * tx);
-                        const uint64_t ak = P2::pack(A.a[k], A.a[k]);
-#pragma unroll
-                        for (int j = 0; j < V / 2; j++) {
-                            const int i = 2 * j;
-                            const uint64_t px = P2::add(P2::pack(v[R + i - k], v[R + i + 1 - k]),
-                                                        P2::pack(v[R + i + k], v[R + i + 1 + k]));
-                            const uint64_t py = P2::add(P2::pack(ym_.v[i], ym_.v[i + 1]),
-                                                        P2::pack(yp_.v[i], yp_.v[i + 1]));
-                            const uint64_t pz =
-                                P2::add(P2::pack(q[R + t - k].v[i], q[R + t - k].v[i + 1]),
-                                        P2::pack(q[R + t + k].v[i], q[R + t + k].v[i + 1]));
-                            if (R == 8 && (k & 1))
-                                L2o[j] = P2::fma(ak, P2::add(P2::add(px, py), pz), L2o[j]);
-                            else
-                                L2[j] = P2::fma(ak, P2::add(P2::add(px, py), pz), L2[j]);
+                    vst(pout + h * row_len, out);
+                    if (what == 0) continue;
+                    if (what & (CLEAR | CKPT)) {
+                        const size_t o = (size_t)z * plane + col + (size_t)h * row_len;
+                        if (what & CLEAR) vst(clear + o, zero4());
+                        if (what & CKPT) {
+                            vst(ck_a + o, qc);
+                            vst(ck_b + o, out);
                         }
                     }
+                    if ((what & (SNAP | IMAGE)) && xm && ym[h] && z >= zlo && z < zhi) {
+                        const size_t so =
+                            (size_t)(z - zlo) * slab_plane + slab_col + (size_t)h * row_len;
+                        if (what & SNAP) {
+                            vst(snap_w + so, out);
+                        } else {
+                            const F4 sv = lds4(aux + 3 * B::APLANE + h * B::TX);
+                            F4 iv = lds4(aux + 4 * B::APLANE + h * B::TX);
 #pragma unroll
-                    for (int j = 0; j < V / 2; j++) {
-                        if (R == 8)
-                            P2::unpack(P2::add(L2[j], L2o[j]), lap.v[2 * j], lap.v[2 * j + 1]);
-                        else
-                            P2::unpack(L2[j], lap.v[2 * j], lap.v[2 * j + 1]);
-                    }
-                }
-                const VT up = zero_in ? vzero<V>() : vlds<V>(aux + aux_off);
-                const VT cc = vlds<V>(aux + B::APLANE + aux_off);
-                const VT& qc = q[R + t];
-                const float gzv = S.gz[z];
-                VT out;
-#pragma unroll
-                for (int i = 0; i < V; i++) {
-                    const float g = gxy.v[i] * gzv;
-                    out.v[i] = g * fmaf(cc.v[i], lap.v[i], 2.0f * qc.v[i]) - (g * g) * up.v[i];
-                }
-                // source injection: u^{n+1}[s] += c_s w^n / dx^3
-                if (do_src && z == S.src_z && y == S.src_y && S.src_x >= x && S.src_x < x + V)
-                    out.v[S.src_x - x] += cc.v[S.src_x - x] * w * A.inv_dx3;
-                const bool rplane = (z == S.rec_z) && ym;
-                if (ph.kind == PH_BWD && rplane) {
-                    // adjoint injection: mu^m[rec] += c g r^{m-1} / dx^3
-                    const float* row =
-                        S.dobs + ((size_t)(ph.step - 1) * S.ny + (y - S.nb)) * S.nx;
-#pragma unroll
-                    for (int i = 0; i < V; i++) {
-                        const int xi = x + i - S.nb;
-                        if (xi >= 0 && xi < S.nx)
-                            out.v[i] += cc.v[i] * (gxy.v[i] * gzv) * row[xi] * A.inv_dx3;
-                    }
-                }
-                const size_t o = (size_t)z * plane + col;
-                vst<V>(prev + o, out);
-                if (clear) vst<V>(clear + o, vzero<V>());
-                if (ck_a) {
-                    vst<V>(ck_a + o, qc);
-                    vst<V>(ck_b + o, out);
-                }
-                const bool inm = xm && ym && z >= S.nb && z < S.nb + S.nz;
-                if (inm) {
-                    const size_t so = (size_t)(z - S.nb) * slab_plane + slab_col;
-                    if (snap_w) vst<V>(snap_w + so, out);
-                    if (snap_r >= 0) {
-                        const VT sv = vlds<V>(aux + 3 * B::APLANE + aux_off);
-                        VT iv = vlds<V>(aux + 4 * B::APLANE + aux_off);
-#pragma unroll
-                        for (int i = 0; i < V; i++) iv.v[i] = fmaf(sv.v[i], out.v[i], iv.v[i]);
-                        vst<V>(S.img + so, iv);
-                    }
-                }
-                if (ph.kind == PH_FWD && rplane && S.data) {
-                    float* row = S.data + ((size_t)ph.step * S.ny + (y - S.nb)) * S.nx;
-#pragma unroll
-                    for (int i = 0; i < V; i++) {
-                        const int xi = x + i - S.nb;
-                        if (xi >= 0 && xi < S.nx) row[xi] = out.v[i];
+                            for (int i = 0; i < 4; i++) iv.v[i] = fmaf(sv.v[i], out.v[i], iv.v[i]);
+                            vst(S.img + so, iv);
+                        }
                     }
                 }
             }
+            pout += plane;
+            // block-wide vote; also every thread is done with this plane's
+            // slot, which plane z + P + 1 reuses
+            ok = __syncthreads_and(got) != 0;
+            if (ok) nwaited++;
             if (++rp.slot == B::NS) rp.slot = 0, rp.phase ^= 1;
         }
 #pragma unroll
-        for (int i = 0; i < 2 * R; i++) q[i] = q[i + G];
+        for (int h = 0; h < ROWS; h++)
+#pragma unroll
+            for (int i = 0; i < 2 * R; i++) q[h][i] = q[h][i + G];
     }
     if (!ok && tid == 0) {
         // copies still in flight must land before the block leaves
@@ -455,22 +405,20 @@ __device__ bool item_tma(const BatchTmaArgs& T, const BatchShot& S, const BatchP
             const int k = slot0 + j;
             const int sl = k % B::NS;
             const uint32_t ph = (uint32_t)(phase0 ^ ((k / B::NS) & 1));
-            bar_drain(&ubar[sl], ph);
-            bar_drain(&abar[sl], ph);
+            bar_drain(&bar[sl], ph);
         }
     }
     return ok;
 }
 
 template <int R, int BY>
-__global__ void __launch_bounds__(16 * BY, BT<R, BY>::MINB)
+__global__ void __launch_bounds__(BT<R, BY>::BX* BT<R, BY>::BY, BT<R, BY>::MINB)
     k_batch_tma(const __grid_constant__ BatchTmaArgs T) {
     using B = BT<R, BY>;
     extern __shared__ __align__(128) float dsm[];
     float* uring = dsm;
     float* aring = dsm + B::NS * B::UPLANE;
-    __shared__ __align__(8) uint64_t ubar[B::NS];
-    __shared__ __align__(8) uint64_t abar[B::NS];
+    __shared__ __align__(8) uint64_t bar[B::NS];
     __shared__ long long s_item;
     __shared__ int s_go, s_shot_i;
     // the item's shot, copied once per item: its fields are read again in
@@ -481,8 +429,7 @@ __global__ void __launch_bounds__(16 * BY, BT<R, BY>::MINB)
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     if (tid == 0) {
         for (int i = 0; i < B::NS; i++) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(&ubar[i])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(&abar[i])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(&bar[i])));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -512,7 +459,13 @@ __global__ void __launch_bounds__(16 * BY, BT<R, BY>::MINB)
         const int s = s_shot_i;
         const BatchShot& S = s_shot;
         const int tile = (int)(r - S.item_base);
-        const bool ok = item_tma<R, BY>(T, S, A.phases[t], tile, s, uring, aring, ubar, abar, rp);
+        const BatchPhase ph = A.phases[t];
+        const bool first = ph.kind == PH_FWD   ? ph.step == 0
+                           : ph.kind == PH_REC ? ph.seg == 0 && ph.local == 0
+                                               : ph.step == A.nt;
+        const bool ok =
+            first ? item_tma<R, BY, true>(T, S, ph, tile, s, uring, aring, bar, rp)
+                  : item_tma<R, BY, false>(T, S, ph, tile, s, uring, aring, bar, rp);
         __threadfence();
         __syncthreads();
         if (!ok) {
@@ -551,7 +504,7 @@ int batch_tma_blocks_per_sm(int radius, int tile_rows) {
         cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              B::SMEM);
         if (r != cudaSuccess) return r;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, 16 * B::BY, B::SMEM);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, B::BX * B::BY, B::SMEM);
     });
     return e == cudaSuccess ? n : 0;
 }
@@ -597,7 +550,7 @@ cudaError_t launch_batch_tma(int radius, int tile_rows, const BatchTmaArgs& a, i
         using B = decltype(b);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(16, B::BY);
+        cfg.blockDim = dim3(B::BX, B::BY);
         cfg.dynamicSmemBytes = B::SMEM;
         cfg.stream = s;
         cudaLaunchAttribute attr[1];

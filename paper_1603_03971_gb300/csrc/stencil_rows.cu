@@ -27,9 +27,9 @@
 #include <string.h>
 
 #include "../../include/rtm.h"
-#include "packed_f32x2.cuh"
 #include "pdl.cuh"
 #include "rtm_internal.h"
+#include "star_rows.cuh"
 #include "stencil_common.cuh"
 #include "tma_encode.h"
 #include "wait_clock.cuh"
@@ -212,73 +212,7 @@ __global__ void __launch_bounds__(BX* BY, 2)
             for (int h = 0; h < 2; h++) q[h][2 * R + t] = lds4(aux + (C::NA - 1) * APLANE + h * TX);
             if (own[0] && ok) {
                 F4 lap[2];
-                {
-                    float v[2][4 + 2 * R];
-                    uint64_t L[2][2], Lo[2][2];
-                    const uint64_t a0 = f32x2::pack(A.a[0], A.a[0]);
-#pragma unroll
-                    for (int h = 0; h < 2; h++) {
-#pragma unroll
-                        for (int g = 0; g < R / 4; g++) {
-                            const F4 l = lds4(S + h * SW - R + 4 * g);
-                            const F4 r = lds4(S + h * SW + 4 + 4 * g);
-#pragma unroll
-                            for (int i = 0; i < 4; i++) {
-                                v[h][4 * g + i] = l.v[i];
-                                v[h][R + 4 + 4 * g + i] = r.v[i];
-                            }
-                        }
-                        const F4& qc = q[h][R + t];
-#pragma unroll
-                        for (int i = 0; i < 4; i++) v[h][R + i] = qc.v[i];
-#pragma unroll
-                        for (int j = 0; j < 2; j++) {
-                            L[h][j] = f32x2::mul(a0, f32x2::pack(qc.v[2 * j], qc.v[2 * j + 1]));
-                            Lo[h][j] = 0;
-                        }
-                    }
-                    // rows 1 - k and k serve both rows: read for the one at offset k - 1,
-                    // kept for the other at offset k
-                    F4 up_ = q[0][R + t], dn_ = q[1][R + t];
-#pragma unroll
-                    for (int k = 1; k <= R; k++) {
-                        const F4 lo = lds4(S - k * SW), hi = lds4(S + (k + 1) * SW);
-                        const uint64_t ak = f32x2::pack(A.a[k], A.a[k]);
-#pragma unroll
-                        for (int h = 0; h < 2; h++) {
-                            const F4& ylo = h == 0 ? lo : up_;
-                            const F4& yhi = h == 0 ? dn_ : hi;
-                            const F4 &zm = q[h][R + t - k], &zp = q[h][R + t + k];
-#pragma unroll
-                            for (int j = 0; j < 2; j++) {
-                                const int i = 2 * j;
-                                const float* w = v[h];
-                                const uint64_t px =
-                                    (k & 1) ? f32x2::pack(w[R + i - k] + w[R + i + k],
-                                                          w[R + i + 1 - k] + w[R + i + 1 + k])
-                                            : f32x2::add(f32x2::pack(w[R + i - k], w[R + i + 1 - k]),
-                                                         f32x2::pack(w[R + i + k], w[R + i + 1 + k]));
-                                const uint64_t py = f32x2::add(f32x2::pack(ylo.v[i], ylo.v[i + 1]),
-                                                               f32x2::pack(yhi.v[i], yhi.v[i + 1]));
-                                const uint64_t pz = f32x2::add(f32x2::pack(zm.v[i], zm.v[i + 1]),
-                                                               f32x2::pack(zp.v[i], zp.v[i + 1]));
-                                const uint64_t s = f32x2::add(f32x2::add(px, py), pz);
-                                if (k & 1)
-                                    Lo[h][j] = f32x2::fma(ak, s, Lo[h][j]);
-                                else
-                                    L[h][j] = f32x2::fma(ak, s, L[h][j]);
-                            }
-                        }
-                        up_ = lo;
-                        dn_ = hi;
-                    }
-#pragma unroll
-                    for (int h = 0; h < 2; h++)
-#pragma unroll
-                        for (int j = 0; j < 2; j++)
-                            f32x2::unpack(f32x2::add(L[h][j], Lo[h][j]), lap[h].v[2 * j],
-                                          lap[h].v[2 * j + 1]);
-                }
+                star_rows<R, 2>(S, SW, q, t, A.a, lap);
                 const float gzv = A.gz[z];
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
