@@ -11,8 +11,9 @@
 //   s_hat = rms(s) * y
 // A float32 snapshot becomes 16 bfloat16 channels per 4^3 voxels: 8x fewer
 // bytes. Every convolution (forward, data gradient, weight gradient) is an
-// implicit GEMM on the tcgen05 engine of tc_gemm.cuh; the rank-8 patch-conv
-// weight gradients, bias gradients, loss and Adam run on the CUDA cores.
+// implicit GEMM on the tcgen05 engine of tc_gemm.cuh; the training layers
+// whose operands are plain copies are in ae_train.cu. Loss and Adam run on the
+// CUDA cores.
 //
 // Parameters: one float32 vector, in order W1[32][2][2][2], b1[32],
 // W2[16][3][3][3][32], b2[16], W3[32][4][4][4][16], b3[32], W4[2][2][2][32],
@@ -21,7 +22,10 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "ae_internal.h"
+#include "ae_train.h"
 #include "tc_gemm.cuh"
 
 namespace rtm {
@@ -31,11 +35,12 @@ using bf16 = __nv_bfloat16;
 
 __device__ __forceinline__ float leaky(float a) { return a > 0.f ? a : kSlope * a; }
 
+// voxel v < 2^31 (half- and quarter-resolution grids of at most 2^34 samples)
 __device__ __forceinline__ void decode3(long long v, int nx, int ny, int& x, int& y, int& z) {
-    x = (int)(v % nx);
-    const long long t = v / nx;
-    y = (int)(t % ny);
-    z = (int)(t / ny);
+    const unsigned u = (unsigned)v, t = u / (unsigned)nx;
+    x = (int)(u - t * (unsigned)nx);
+    z = (int)(t / (unsigned)ny);
+    y = (int)(t - (unsigned)z * (unsigned)ny);
 }
 
 __device__ __forceinline__ uint4 zero4u() { return make_uint4(0, 0, 0, 0); }
@@ -476,252 +481,6 @@ struct OpD2d {  // gy (bf16, full grid) -> ga3 = (W4^T gy) * leaky'(a3)
     }
 };
 
-struct OpD1d {  // ga3 -> glat: dlat[j] = sum_k W3[.,k,.]^T ga3[2j + k - 1]
-    using Args = D1dArgs;
-    static constexpr int N = 16;
-    __device__ static void tile(const Args&, int& m0, int& c0, int& c1) {
-        m0 = blockIdx.x * 128;
-        c0 = 0;
-        c1 = 64;
-    }
-    __device__ static void load(const Args& a, int m0, int ktap, uint8_t* sA, uint8_t* sB, int tid) {
-        const long long v = m0 + tid;
-        const long long total = (long long)a.l.nx * a.l.ny * a.l.nz;
-        const int kz = ktap >> 4, ky = (ktap >> 2) & 3, kx = ktap & 3;
-        uint4 r[4] = {zero4u(), zero4u(), zero4u(), zero4u()};
-        if (v < total) {
-            int x, y, z;
-            decode3(v, a.l.nx, a.l.ny, x, y, z);
-            const int ox = 2 * x + kx - 1, oy = 2 * y + ky - 1, oz = 2 * z + kz - 1;
-            if (ox >= 0 && ox < a.h.nx && oy >= 0 && oy < a.h.ny && oz >= 0 && oz < a.h.nz) {
-                const uint4* src = reinterpret_cast<const uint4*>(
-                    a.ga3 + (((long long)oz * a.h.ny + oy) * a.h.nx + ox) * 32);
-#pragma unroll
-                for (int j = 0; j < 4; j++) r[j] = src[j];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++) tc::st_vec8(sA, tid, 8 * j, r[j]);
-        load_b(a, ktap, sB, tid);
-    }
-    __device__ static void load_b(const Args& a, int ktap, uint8_t* sB, int tid) {
-        if (tid < 64) {
-            const int i = tid >> 2, j = tid & 3;
-            float w[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++) w[e] = a.P[kOW3 + (8 * j + e) * 1024 + ktap * 16 + i];
-            tc::st_vec8(sB, i, 8 * j, tc::pack8(w));
-        }
-    }
-    __device__ static void load_async(const Args& a, int m0, int ktap, uint8_t* sA, uint8_t* sB,
-                                      int tid) {
-        const long long v = m0 + tid;
-        const long long total = (long long)a.l.nx * a.l.ny * a.l.nz;
-        const int kz = ktap >> 4, ky = (ktap >> 2) & 3, kx = ktap & 3;
-        const bf16* src = a.ga3;
-        bool ok = false;
-        if (v < total) {
-            int x, y, z;
-            decode3(v, a.l.nx, a.l.ny, x, y, z);
-            const int ox = 2 * x + kx - 1, oy = 2 * y + ky - 1, oz = 2 * z + kz - 1;
-            if (ox >= 0 && ox < a.h.nx && oy >= 0 && oy < a.h.ny && oz >= 0 && oz < a.h.nz) {
-                ok = true;
-                src = a.ga3 + (((long long)oz * a.h.ny + oy) * a.h.nx + ox) * 32;
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++) tc::cp_async16(sA, tid, 8 * j, src + 8 * j, ok);
-        load_b(a, ktap, sB, tid);
-    }
-    __device__ static void epilogue(const Args& a, int m0, int row, const float* acc) {
-        const long long v = m0 + row;
-        if (v >= (long long)a.l.nx * a.l.ny * a.l.nz) return;
-        store_bf16_row(a.glat + v * 16, acc, 16);
-    }
-};
-
-struct OpE2d {  // glat -> ga1 = (sum over taps of W2^T glat) * leaky'(a1)
-    using Args = E2dArgs;
-    static constexpr int N = 32;
-    __device__ static void tile(const Args&, int& m0, int& c0, int& c1) {
-        m0 = blockIdx.x * 128;
-        c0 = 0;
-        c1 = 14;  // 27 taps, two per slab, the last one padded
-    }
-    __device__ static void load(const Args& a, int m0, int ch, uint8_t* sA, uint8_t* sB, int tid) {
-        const long long p = m0 + tid;
-        const long long total = (long long)a.h.nx * a.h.ny * a.h.nz;
-        int px = 0, py = 0, pz = 0;
-        if (p < total) decode3(p, a.h.nx, a.h.ny, px, py, pz);
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int tap = 2 * ch + h;
-            uint4 r0 = zero4u(), r1 = zero4u();
-            if (p < total && tap < 27) {
-                const int kz = tap / 9, ky = (tap / 3) % 3, kx = tap % 3;
-                const int nz = pz + 1 - kz, ny = py + 1 - ky, nx = px + 1 - kx;
-                if (nx >= 0 && ny >= 0 && nz >= 0 && !(nx & 1) && !(ny & 1) && !(nz & 1)) {
-                    const int vx = nx >> 1, vy = ny >> 1, vz = nz >> 1;
-                    if (vx < a.l.nx && vy < a.l.ny && vz < a.l.nz) {
-                        const uint4* src = reinterpret_cast<const uint4*>(
-                            a.glat + (((long long)vz * a.l.ny + vy) * a.l.nx + vx) * 16);
-                        r0 = src[0];
-                        r1 = src[1];
-                    }
-                }
-            }
-            tc::st_vec8(sA, tid, 16 * h, r0);
-            tc::st_vec8(sA, tid, 16 * h + 8, r1);
-        }
-        {
-            const int i = tid >> 2, j = tid & 3, h = j >> 1, o0 = (j & 1) * 8;
-            const int tap = 2 * ch + h;
-            float w[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++)
-                w[e] = tap < 27 ? a.P[kOW2 + (o0 + e) * 864 + tap * 32 + i] : 0.f;
-            tc::st_vec8(sB, i, 8 * j, tc::pack8(w));
-        }
-    }
-    __device__ static void epilogue(const Args& a, int m0, int row, const float* acc) {
-        const long long p = m0 + row;
-        if (p >= (long long)a.h.nx * a.h.ny * a.h.nz) return;
-        float f[32], g[8];
-        for (int j = 0; j < 32; j += 8) {
-            bf16x8_to_f(reinterpret_cast<const uint4*>(a.h1 + p * 32)[j / 8], g);
-            for (int e = 0; e < 8; e++) f[j + e] = acc[j + e] * (g[e] > 0.f ? 1.0f : kSlope);
-        }
-        store_bf16_row(a.ga1 + p * 32, f, 32);
-    }
-};
-
-// ============================================================================
-// weight gradients on the tensor cores (reduction over voxels, split over CTAs)
-// ============================================================================
-struct OpE2w {  // dW2[o][tap][i] += sum_v glat[v][o] h1[2v + tap - 1][i]
-    using Args = E2wArgs;
-    static constexpr int N = 16;
-    __device__ static void tile(const Args& a, int& m0, int& c0, int& c1) {
-        m0 = blockIdx.x * 128;  // rows r = tap * 32 + i
-        const long long nv = (long long)a.l.nx * a.l.ny * a.l.nz;
-        const int nch = (int)((nv + 31) / 32);
-        c0 = blockIdx.y * a.chunks_per_cta;
-        c1 = min(nch, c0 + a.chunks_per_cta);
-        if (c1 < c0) c1 = c0;
-    }
-    __device__ static void load(const Args& a, int m0, int ch, uint8_t* sA, uint8_t* sB, int tid) {
-        const long long nv = (long long)a.l.nx * a.l.ny * a.l.nz;
-        const int vv = tid & 31, tt = tid >> 5;
-        const int tap = m0 / 32 + tt;
-        const long long v = (long long)ch * 32 + vv;
-        float f[32];
-#pragma unroll
-        for (int i = 0; i < 32; i++) f[i] = 0.f;
-        if (tap < 27 && v < nv) {
-            int x, y, z;
-            decode3(v, a.l.nx, a.l.ny, x, y, z);
-            const int kz = tap / 9, ky = (tap / 3) % 3, kx = tap % 3;
-            const int sx = 2 * x + kx - 1, sy = 2 * y + ky - 1, sz = 2 * z + kz - 1;
-            if (sx >= 0 && sx < a.h.nx && sy >= 0 && sy < a.h.ny && sz >= 0 && sz < a.h.nz) {
-                const uint4* src = reinterpret_cast<const uint4*>(
-                    a.h1 + (((long long)sz * a.h.ny + sy) * a.h.nx + sx) * 32);
-#pragma unroll
-                for (int j = 0; j < 4; j++) bf16x8_to_f(src[j], f + 8 * j);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 32; i++) tc::st_one(sA, tt * 32 + i, vv, __float2bfloat16_rn(f[i]));
-        if (tid < 32) {
-            const long long w = (long long)ch * 32 + tid;
-            float g[16];
-#pragma unroll
-            for (int o = 0; o < 16; o++) g[o] = 0.f;
-            if (w < nv) {
-                const uint4* src = reinterpret_cast<const uint4*>(a.glat + w * 16);
-                bf16x8_to_f(src[0], g);
-                bf16x8_to_f(src[1], g + 8);
-            }
-#pragma unroll
-            for (int o = 0; o < 16; o++) tc::st_one(sB, o, tid, __float2bfloat16_rn(g[o]));
-        }
-    }
-    __device__ static void epilogue(const Args& a, int m0, int row, const float* acc) {
-        const int r = m0 + row;
-        if (r >= 27 * 32) return;
-        for (int o = 0; o < 16; o++) atomicAdd(&a.grad[kOW2 + o * 864 + r], acc[o]);
-    }
-};
-
-struct OpD1w {  // dW3[o][k][i] += sum_j ga3[2j + q][o] lat[j + t][i], class q = blockIdx.x
-    using Args = D1wArgs;
-    static constexpr int N = 32;
-    __device__ static void tile(const Args& a, int& m0, int& c0, int& c1) {
-        m0 = 0;  // rows r = tau * 16 + i, tau the class's 8 taps
-        const long long nv = (long long)a.l.nx * a.l.ny * a.l.nz;
-        const int nch = (int)((nv + 31) / 32);
-        c0 = blockIdx.y * a.chunks_per_cta;
-        c1 = min(nch, c0 + a.chunks_per_cta);
-        if (c1 < c0) c1 = c0;
-    }
-    __device__ static void load(const Args& a, int, int ch, uint8_t* sA, uint8_t* sB, int tid) {
-        const int q = blockIdx.x, qz = q >> 2, qy = (q >> 1) & 1, qx = q & 1;
-        const long long nv = (long long)a.l.nx * a.l.ny * a.l.nz;
-#pragma unroll
-        for (int rep = 0; rep < 2; rep++) {
-            const int idx = tid + rep * 128;
-            const int vv = idx & 31, tau = idx >> 5;
-            const long long j = (long long)ch * 32 + vv;
-            float f[16];
-#pragma unroll
-            for (int i = 0; i < 16; i++) f[i] = 0.f;
-            if (j < nv) {
-                int x, y, z;
-                decode3(j, a.l.nx, a.l.ny, x, y, z);
-                int tz, kz, ty, ky, tx, kx;
-                convt_tap(qz, tau >> 2, tz, kz);
-                convt_tap(qy, (tau >> 1) & 1, ty, ky);
-                convt_tap(qx, tau & 1, tx, kx);
-                const int sx = x + tx, sy = y + ty, sz = z + tz;
-                if (sx >= 0 && sx < a.l.nx && sy >= 0 && sy < a.l.ny && sz >= 0 && sz < a.l.nz) {
-                    const uint4* src = reinterpret_cast<const uint4*>(
-                        a.lat + (((long long)sz * a.l.ny + sy) * a.l.nx + sx) * 16);
-                    bf16x8_to_f(src[0], f);
-                    bf16x8_to_f(src[1], f + 8);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 16; i++) tc::st_one(sA, tau * 16 + i, vv, __float2bfloat16_rn(f[i]));
-        }
-        if (tid < 32) {
-            const long long j = (long long)ch * 32 + tid;
-            float g[32];
-#pragma unroll
-            for (int o = 0; o < 32; o++) g[o] = 0.f;
-            if (j < nv) {
-                int x, y, z;
-                decode3(j, a.l.nx, a.l.ny, x, y, z);
-                const long long o = (((long long)(2 * z + qz) * a.h.ny + (2 * y + qy)) * a.h.nx +
-                                     2 * x + qx);
-                const uint4* src = reinterpret_cast<const uint4*>(a.ga3 + o * 32);
-#pragma unroll
-                for (int k = 0; k < 4; k++) bf16x8_to_f(src[k], g + 8 * k);
-            }
-#pragma unroll
-            for (int o = 0; o < 32; o++) tc::st_one(sB, o, tid, __float2bfloat16_rn(g[o]));
-        }
-    }
-    __device__ static void epilogue(const Args& a, int, int row, const float* acc) {
-        const int q = blockIdx.x, qz = q >> 2, qy = (q >> 1) & 1, qx = q & 1;
-        const int tau = row >> 4, i = row & 15;
-        int tz, kz, ty, ky, tx, kx;
-        convt_tap(qz, tau >> 2, tz, kz);
-        convt_tap(qy, (tau >> 1) & 1, ty, ky);
-        convt_tap(qx, tau & 1, tx, kx);
-        const int ktap = (kz * 4 + ky) * 4 + kx;
-        for (int o = 0; o < 32; o++) atomicAdd(&a.grad[kOW3 + o * 1024 + ktap * 16 + i], acc[o]);
-    }
-};
-
 // ============================================================================
 // CUDA-core kernels
 // ============================================================================
@@ -801,108 +560,69 @@ __global__ void k_scale(const double* acc, long long n, float* sigma, float* inv
     *inv_sigma = (float)(1.0 / r);
 }
 
-// loss += mean((y - x0)^2) * scale; gy = bf16(scale * 2 (y - x0) / n); grad[b4] += sum gy
-__global__ void k_loss(const float* __restrict__ y, Vol in, const float* inv_sigma, float scale,
-                       bf16* gy, double* loss, float* grad) {
+// loss += mean((y - x0)^2) * scale; gy = bf16(scale * 2 (y - x0) / n); grad[b4] += sum gy.
+// y and gy are dense; in is read as one array where it is dense too, four
+// values at a time where `vec` says so. The squares are summed as pairs of
+// floats (exact products, about 48 bits): GB300 has few float64 lanes, and two
+// float64 operations per sample took half of the kernel's 54 us at 192^3
+__global__ void __launch_bounds__(256) k_loss(const float* __restrict__ y, Vol in,
+                                              const float* inv_sigma, float scale, int vec, bf16* gy,
+                                              double* loss, float* grad) {
     const long long n = (long long)in.nx * in.ny * in.nz;
+    const bool dense = in.sy == in.nx && in.sz == (long long)in.nx * in.ny;
     const float s = *inv_sigma;
-    double l = 0.0;
-    float gsum = 0.f;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        int x, yy, z;
-        decode3(i, in.nx, in.ny, x, yy, z);
-        const float x0 = in.p[(long long)z * in.sz + (long long)yy * in.sy + x] * s;
-        const float d = y[i] - x0;
-        l += (double)d * d;
+    float hi = 0.f, lo = 0.f, gsum = 0.f;
+    auto one = [&](float yv, float xv) {
+        const float d = yv - xv * s;
+        const float p = d * d, t = hi + p, bb = t - hi;
+        lo += ((hi - (t - bb)) + (p - bb)) + fmaf(d, d, -p);
+        hi = t;
         const bf16 g = __float2bfloat16_rn(scale * 2.0f * d / (float)n);
-        gy[i] = g;
         gsum += __bfloat162float(g);
+        return g;
+    };
+    const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    if (vec) {
+        for (long long i = first; i < n / 4; i += step) {
+            const float4 a = __ldcs(reinterpret_cast<const float4*>(y) + i);
+            const float4 x = __ldg(reinterpret_cast<const float4*>(in.p) + i);
+            __nv_bfloat162 g[2];
+            g[0].x = one(a.x, x.x);
+            g[0].y = one(a.y, x.y);
+            g[1].x = one(a.z, x.z);
+            g[1].y = one(a.w, x.w);
+            reinterpret_cast<uint2*>(gy)[i] = *reinterpret_cast<uint2*>(g);
+        }
+    } else {
+        for (long long i = first; i < n; i += step) {
+            long long at = i;
+            if (!dense) {
+                const long long zy = i / in.nx;
+                at = zy / in.ny * in.sz + zy % in.ny * in.sy + i % in.nx;
+            }
+            gy[i] = one(y[i], in.p[at]);
+        }
     }
+    double l = (double)hi + (double)lo;
     for (int o = 16; o > 0; o >>= 1) {
         l += __shfl_xor_sync(0xffffffffu, l, o);
         gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
     }
+    __shared__ double lpart[8];
+    __shared__ float gpart[8];
     if ((threadIdx.x & 31) == 0) {
+        lpart[threadIdx.x >> 5] = l;
+        gpart[threadIdx.x >> 5] = gsum;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; w++) {
+            l += lpart[w];
+            gsum += gpart[w];
+        }
         atomicAdd(loss, l * scale / (double)n);
         atomicAdd(&grad[kOB4], gsum);
-    }
-}
-
-// patch-conv weight gradients (rank 8) and the bias gradients:
-//   dW1[c][d] += sum_v ga1[v][c] xq[2v + d],   dW4[d][i] += sum_v gy[2v + d] g1[v][i]
-//   db1 += sum ga1, db2 += sum glat, db3 += sum ga3
-// a warp per voxel, lane = channel: lanes 0..7 load the voxel's 8 patch
-// inputs and lanes 8..15 its 8 output gradients, shared by shuffles; each
-// lane accumulates its row of the two outer products; the 8 warps of a block
-// are summed in shared memory and the block adds its sums with one atomic per
-// output
-__global__ void __launch_bounds__(256) k_small_grads(Vol in, const float* inv_sigma,
-                                                     const bf16* __restrict__ ga1,
-                                                     const bf16* __restrict__ gy,
-                                                     const bf16* __restrict__ g1,
-                                                     const bf16* __restrict__ ga3,
-                                                     const bf16* __restrict__ glat, Dims3 h,
-                                                     Dims3 l, float* grad) {
-    constexpr int kVals = 19;  // per lane: dW1 row (8), dW4 column (8), db1, db3, db2
-    __shared__ float red[8][kVals][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const long long nh = (long long)h.nx * h.ny * h.nz;
-    const long long nl = (long long)l.nx * l.ny * l.nz;
-    const long long gw = (long long)blockIdx.x * 8 + wid, nw = (long long)gridDim.x * 8;
-    const float s = *inv_sigma;
-    const int NX = 2 * h.nx, NY = 2 * h.ny;
-    const int e = lane & 7, ez = e >> 2, ey = (e >> 1) & 1, ex = e & 1;
-    float w1[8], w4[8], b1 = 0.f, b3 = 0.f, b2 = 0.f;
-#pragma unroll
-    for (int d = 0; d < 8; d++) w1[d] = w4[d] = 0.f;
-    for (long long v = gw; v < nh; v += nw) {
-        int x, y, z;
-        decode3(v, h.nx, h.ny, x, y, z);
-        float mine = 0.f;
-        if (lane < 8)
-            mine = __bfloat162float(__float2bfloat16_rn(
-                in.p[(long long)(2 * z + ez) * in.sz + (long long)(2 * y + ey) * in.sy + 2 * x + ex] *
-                s));
-        else if (lane < 16)
-            mine = __bfloat162float(
-                gy[((long long)(2 * z + ez) * NY + (2 * y + ey)) * NX + 2 * x + ex]);
-        const float a = __bfloat162float(ga1[v * 32 + lane]);
-        const float gg = __bfloat162float(g1[v * 32 + lane]);
-        b1 += a;
-        b3 += __bfloat162float(ga3[v * 32 + lane]);
-#pragma unroll
-        for (int d = 0; d < 8; d++) {
-            w1[d] = fmaf(a, __shfl_sync(0xffffffffu, mine, d), w1[d]);
-            w4[d] = fmaf(__shfl_sync(0xffffffffu, mine, 8 + d), gg, w4[d]);
-        }
-    }
-    if (lane < 16)
-        for (long long v = gw; v < nl; v += nw) b2 += __bfloat162float(glat[v * 16 + lane]);
-#pragma unroll
-    for (int d = 0; d < 8; d++) {
-        red[wid][d][lane] = w1[d];
-        red[wid][8 + d][lane] = w4[d];
-    }
-    red[wid][16][lane] = b1;
-    red[wid][17][lane] = b3;
-    red[wid][18][lane] = b2;
-    __syncthreads();
-    for (int k = threadIdx.x; k < kVals * 32; k += blockDim.x) {
-        const int val = k >> 5, ln = k & 31;
-        float t = 0.f;
-#pragma unroll
-        for (int w = 0; w < 8; w++) t += red[w][val][ln];
-        if (val < 8)
-            atomicAdd(&grad[kOW1 + ln * 8 + val], t);
-        else if (val < 16)
-            atomicAdd(&grad[kOW4 + (val - 8) * 32 + ln], t);
-        else if (val == 16)
-            atomicAdd(&grad[kOB1 + ln], t);
-        else if (val == 17)
-            atomicAdd(&grad[kOB3 + ln], t);
-        else if (ln < 16)
-            atomicAdd(&grad[kOB2 + ln], t);
     }
 }
 
@@ -969,8 +689,7 @@ cudaError_t ae_rms(const Vol& in, AeScalars* sc, cudaStream_t s) {
 }
 
 cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScalars* sc,
-                      float* sigma_out, int* status, cudaStream_t s, bool keep_h1,
-                      bool sumsq_ready) {
+                      float* sigma_out, int* status, cudaStream_t s, bool sumsq_ready) {
     cudaError_t e = cudaSuccess;
     if (sumsq_ready) {
         k_scale<<<1, 1, 0, s>>>(&sc->sumsq, (long long)in.nx * in.ny * in.nz, &sc->sigma,
@@ -981,7 +700,7 @@ cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScal
     }
     if (e != cudaSuccess) return e;
     const Dims3 h{in.nx / 2, in.ny / 2, in.nz / 2}, l{in.nx / 4, in.ny / 4, in.nz / 4};
-    e = keep_h1 ? cudaErrorNotSupported : ae_encode_march(P, in, &sc->inv_sigma, lat, status, s);
+    e = ae_encode_march(P, in, &sc->inv_sigma, lat, status, s);
     if (e == cudaErrorNotSupported) {
         cudaGetLastError();
         E1Args a1{in, &sc->inv_sigma, P, h1, h};
@@ -996,17 +715,9 @@ cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScal
     return e;
 }
 
-cudaError_t ae_decode(const float* P, const bf16* lat, const float* sigma, const Vol& out, bf16* g1,
+cudaError_t ae_decode(const float* P, const bf16* lat, const float* sigma, const Vol& out,
                       int* status, cudaStream_t s) {
     const Dims3 h{out.nx / 2, out.ny / 2, out.nz / 2}, l{out.nx / 4, out.ny / 4, out.nz / 4};
-    if (g1) {  // two passes through g1 (training keeps g1 for the backward pass)
-        D1Args a1{lat, l, P, g1, h};
-        cudaError_t e =
-            run_async<OpD1>(a1, dim3(tiles((long long)l.nx * l.ny * l.nz), 8), status, s);
-        if (e != cudaSuccess) return e;
-        D2Args a2{g1, h, P, sigma, out};
-        return run<OpD2>(a2, dim3(tiles((long long)h.nx * h.ny * h.nz)), status, s);
-    }
     D12Args a{D1Args{lat, l, P, nullptr, h}, sigma, out};
     const cudaError_t e = ae_decode_march(a, status, s);
     if (e != cudaErrorNotSupported) return e;
@@ -1018,37 +729,32 @@ cudaError_t ae_decode(const float* P, const bf16* lat, const float* sigma, const
 cudaError_t ae_sample_grad(const float* P, const Vol& in, float scale, const AeTrainBufs& b,
                            AeScalars* sc, double* loss, float* grad, int* status, cudaStream_t s) {
     const Dims3 h{in.nx / 2, in.ny / 2, in.nz / 2}, l{in.nx / 4, in.ny / 4, in.nz / 4};
-    const long long nh = (long long)h.nx * h.ny * h.nz, nl = (long long)l.nx * l.ny * l.nz;
+    const unsigned tiles_h = tiles((long long)h.nx * h.ny * h.nz);
     const long long n = (long long)in.nx * in.ny * in.nz;
-    cudaError_t e = ae_encode(P, in, b.h1, b.lat, sc, nullptr, status, s, true);
-    if (e != cudaSuccess) return e;
+#define RUN(call)                                \
+    do {                                         \
+        const cudaError_t e_ = (call);           \
+        if (e_ != cudaSuccess) return e_;        \
+    } while (0)
+    RUN(ae_rms(in, sc, s));
+    RUN(run<OpE1>(E1Args{in, &sc->inv_sigma, P, b.h1, h}, dim3(tiles_h), status, s));
+    RUN(ae_train_e2(P, b.W, b.h1, b.lat, h, l, status, s));
+    RUN(ae_train_d1(P, b.W, b.lat, b.g1, h, l, status, s));
     const Vol yv{b.y, (long long)in.nx, (long long)in.nx * in.ny, in.nx, in.ny, in.nz};
-    e = ae_decode(P, b.lat, nullptr, yv, b.g1, status, s);
-    if (e != cudaSuccess) return e;
-    long long blocks = (n + 255) / 256;
-    if (blocks > 152 * 8) blocks = 152 * 8;
-    k_loss<<<(unsigned)blocks, 256, 0, s>>>(b.y, in, &sc->inv_sigma, scale, b.gy, loss, grad);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    D2dArgs d2{b.gy, h, b.g1, P, b.ga3};
-    if ((e = run<OpD2d>(d2, dim3(tiles(nh)), status, s)) != cudaSuccess) return e;
-    const int nch_l = (int)((nl + 31) / 32);
-    const int cpc_l = max(1, (nch_l + 151) / 152);
-    D1wArgs w3{b.lat, l, b.ga3, h, grad, cpc_l};
-    if ((e = run<OpD1w>(w3, dim3(8, (nch_l + cpc_l - 1) / cpc_l), status, s)) != cudaSuccess)
-        return e;
-    D1dArgs d1{b.ga3, h, l, P, b.glat};
-    if ((e = run_async<OpD1d>(d1, dim3(tiles(nl)), status, s)) != cudaSuccess) return e;
-    E2wArgs w2{b.h1, h, b.glat, l, grad, cpc_l};
-    if ((e = run<OpE2w>(w2, dim3(7, (nch_l + cpc_l - 1) / cpc_l), status, s)) != cudaSuccess)
-        return e;
-    E2dArgs d0{b.glat, l, b.h1, h, P, b.ga1};
-    if ((e = run<OpE2d>(d0, dim3(tiles(nh)), status, s)) != cudaSuccess) return e;
-    long long sb = (nh + 8 * 64 - 1) / (8 * 64);  // at least 64 voxels per warp
-    if (sb < 1) sb = 1;
-    if (sb > 152 * 4) sb = 152 * 4;
-    k_small_grads<<<(unsigned)sb, 256, 0, s>>>(in, &sc->inv_sigma, b.ga1, b.gy, b.g1, b.ga3,
-                                               b.glat, h, l, grad);
-    return cudaGetLastError();
+    RUN(run<OpD2>(D2Args{b.g1, h, P, nullptr, yv}, dim3(tiles_h), status, s));
+    const int vec = reinterpret_cast<uintptr_t>(in.p) % 16 == 0 && in.sy == in.nx &&
+                    in.sz == (long long)in.nx * in.ny;  // every side is a multiple of 4
+    const long long blocks = std::min<long long>((n + 1023) / 1024, 152 * 8);
+    k_loss<<<(unsigned)blocks, 256, 0, s>>>(b.y, in, &sc->inv_sigma, scale, vec, b.gy, loss, grad);
+    RUN(cudaGetLastError());
+    RUN(run<OpD2d>(D2dArgs{b.gy, h, b.g1, P, b.ga3}, dim3(tiles_h), status, s));
+    RUN(ae_train_d1_weights(b.lat, b.ga3, grad, h, l, status, s));
+    RUN(ae_train_d1_grad(b.W, b.ga3, b.glat, h, l, status, s));
+    RUN(ae_train_e2_weights(b.h1, b.glat, grad, h, l, status, s));
+    RUN(ae_train_e2_grad(b.W, b.glat, b.h1, b.ga1, h, l, status, s));
+    RUN(ae_train_patch_weights(in, &sc->inv_sigma, b.ga1, b.gy, b.g1, b.ga3, grad, h, l, status, s));
+#undef RUN
+    return cudaSuccess;
 }
 
 cudaError_t ae_adam(float* P, float* m, float* v, const float* g, int step, float lr, float clip,

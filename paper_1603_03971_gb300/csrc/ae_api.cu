@@ -7,6 +7,7 @@
 
 #include "../../include/rtm.h"
 #include "ae_internal.h"
+#include "ae_train.h"
 #include "rtm_internal.h"
 
 using namespace rtm;
@@ -20,7 +21,7 @@ size_t upa(size_t v) { return (v + kAl - 1) / kAl * kAl; }
 
 struct AeLayout {
     size_t status = 0, scalars = 64;
-    size_t h1, lat, g1, y, gy, ga3, glat, ga1, grad, total;
+    size_t h1, lat, g1, y, gy, ga3, glat, ga1, grad, packed, total;
 };
 
 AeLayout ae_layout(int nx, int ny, int nz) {
@@ -41,6 +42,7 @@ AeLayout ae_layout(int nx, int ny, int nz) {
     L.glat = take(nl * 16 * 2);
     L.ga1 = take(nh * 32 * 2);
     L.grad = take((size_t)kNParams * 4);
+    L.packed = take(kAePackedBytes);
     L.total = o;
     return L;
 }
@@ -122,7 +124,7 @@ rtm_status rtm_ae_decode(const float* d_params, const uint16_t* d_latent, const 
     cudaGetLastError();
     const Vol out{d_out, sy, sz, nx, ny, nz};
     CUA(cudaMemsetAsync(w, 0, sizeof(int), s));
-    CUA(ae_decode(d_params, reinterpret_cast<const bf16*>(d_latent), d_scale, out, nullptr,
+    CUA(ae_decode(d_params, reinterpret_cast<const bf16*>(d_latent), d_scale, out,
                   reinterpret_cast<int*>(w + L.status), s));
     return RTM_OK;
 }
@@ -146,10 +148,12 @@ rtm_status rtm_ae_train_step(float* d_params, float* d_adam_m, float* d_adam_v, 
     AeTrainBufs b{reinterpret_cast<bf16*>(w + L.h1),  reinterpret_cast<bf16*>(w + L.lat),
                   reinterpret_cast<bf16*>(w + L.g1),  reinterpret_cast<bf16*>(w + L.gy),
                   reinterpret_cast<bf16*>(w + L.ga3), reinterpret_cast<bf16*>(w + L.glat),
-                  reinterpret_cast<bf16*>(w + L.ga1), reinterpret_cast<float*>(w + L.y)};
+                  reinterpret_cast<bf16*>(w + L.ga1), reinterpret_cast<float*>(w + L.y),
+                  w + L.packed};
     CUA(cudaMemsetAsync(w, 0, sizeof(int), s));
     CUA(cudaMemsetAsync(grad, 0, sizeof(float) * kNParams, s));
     CUA(cudaMemsetAsync(d_loss, 0, sizeof(double), s));
+    CUA(ae_pack_weights(d_params, w + L.packed, s));
     const size_t n = (size_t)nx * ny * nz;
     for (int i = 0; i < batch; i++) {
         const Vol in{const_cast<float*>(d_batch) + i * n, (long long)nx, (long long)nx * ny, nx,

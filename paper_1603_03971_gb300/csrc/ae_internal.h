@@ -39,10 +39,6 @@ struct D1Args { const bf16* lat; Dims3 l; const float* P; bf16* g1; Dims3 h; };
 struct D2Args { const bf16* g1; Dims3 h; const float* P; const float* sigma; Vol out; };
 struct D12Args { D1Args d1; const float* sigma; Vol out; };
 struct D2dArgs { const bf16* gy; Dims3 h; const bf16* g1; const float* P; bf16* ga3; };
-struct D1dArgs { const bf16* ga3; Dims3 h; Dims3 l; const float* P; bf16* glat; };
-struct E2dArgs { const bf16* glat; Dims3 l; const bf16* h1; Dims3 h; const float* P; bf16* ga1; };
-struct E2wArgs { const bf16* h1; Dims3 h; const bf16* glat; Dims3 l; float* grad; int chunks_per_cta; };
-struct D1wArgs { const bf16* lat; Dims3 l; const bf16* ga3; Dims3 h; float* grad; int chunks_per_cta; };
 
 // device-resident scalars of one codec call
 struct AeScalars {
@@ -55,26 +51,25 @@ struct AeScalars {
 struct AeTrainBufs {
     bf16 *h1, *lat, *g1, *gy, *ga3, *glat, *ga1;
     float* y;
+    const void* W;  // packed weights (ae_train.h)
 };
 
 }  // namespace ae
 
 cudaError_t ae_gemm_test(const ae::GemmArgs& a, int N, int* status, cudaStream_t s);
 cudaError_t ae_rms(const ae::Vol& in, ae::AeScalars* sc, cudaStream_t s);
-// snapshot -> latent; the snapshot's rms goes to sigma_out if given. With
-// keep_h1 the GEMM-engine layers run and leave E1's output in h1 (training
-// reads it); otherwise the z-marching kernel runs where it can and h1 is
-// untouched scratch. With sumsq_ready, sc->sumsq already holds the
+// snapshot -> latent; the snapshot's rms goes to sigma_out if given. The
+// z-marching kernel runs where it can, otherwise the GEMM-engine layers through
+// h1. With sumsq_ready, sc->sumsq already holds the
 // snapshot's sum of squares (accumulated by the stencil step that wrote it)
 // and only the scale is derived from it.
 cudaError_t ae_encode(const float* P, const ae::Vol& in, ae::bf16* h1, ae::bf16* lat,
                       ae::AeScalars* sc, float* sigma_out, int* status, cudaStream_t s,
-                      bool keep_h1 = false, bool sumsq_ready = false);
-// latent -> snapshot scaled by *sigma (1 if NULL); with g1 NULL the two
-// decoder layers run fused (inference), otherwise g1 keeps the D1 output
+                      bool sumsq_ready = false);
+// latent -> snapshot scaled by *sigma (1 if NULL), the two decoder layers fused
 cudaError_t ae_decode(const float* P, const ae::bf16* lat, const float* sigma, const ae::Vol& out,
-                      ae::bf16* g1, int* status, cudaStream_t s);
-// the fused inference decoder as one z-marching persistent kernel (TMA plane
+                      int* status, cudaStream_t s);
+// the fused decoder as one z-marching persistent kernel (TMA plane
 // loads read in place by the tensor cores); cudaErrorNotSupported when it
 // cannot run or is not selected
 cudaError_t ae_decode_march(const ae::D12Args& a, int* status, cudaStream_t s);

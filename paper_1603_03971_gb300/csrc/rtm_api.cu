@@ -652,7 +652,7 @@ rtm_status run_forward(Ctx& C, const int32_t* rec, float* data, float* u_last) {
             const size_t k = (size_t)((n + 1) / ie - 1);
             CU(ae_encode(C.ae, C.field_view(prev), reinterpret_cast<ae::bf16*>(C.at(C.L.ae_h)),
                          C.latent_slot(k), scal, C.at(C.L.scales) + k, C.status(), C.s,
-                         false, true));
+                         true));
             count_launch(2);  // scale, encoder
         }
         float* t = prev;
@@ -840,7 +840,7 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
                     CU(launch_upsample(C.G, C.coarse_slot(k), slab, C.s));
                 else
                     CU(ae_decode(C.ae, C.latent_slot(k), C.at(C.L.scales) + k,
-                                 C.model_view(slab), nullptr, C.status(), C.s));
+                                 C.model_view(slab), C.status(), C.s));
                 count_launch(1);
             }
             // down to the state after the next coded one
