@@ -818,6 +818,10 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
             a.off = off;
             a.acc = acc;
             a.illum = C.illum;
+            // the source's field pair is scratch while the receivers propagate,
+            // except where its states are still to be recomputed from it
+            if (C.taps && p->storage != RTM_STORE_REVOLVE)
+                for (int i = 0; i < 2; i++) a.scatter[i] = C.at(C.L.f[i]);
             return run_span(C, a, snap ? (grad ? MODE_BWD_GRAD : MODE_BWD_IMAGE) : MODE_FWD, mprev,
                             mcur);
         }

@@ -23,9 +23,14 @@
 //   104^3, r = 4:             6.5 / 7.1 / 8.6     18.5 / 18.5 / 18.6
 //   132 x 120 x 110, r = 4:   9.4 / 10.1 / 13.1   18.6 / 20.6 / 20.6
 //   104^3, r = 8 (forward):   10.9 / 11.5         20.5 / 20.5
+//   104^3, r = 4, off grid:   12.1 / - / 14.7     42 / - / 34     (1024 receivers)
 // A brick has to fit one SM's shared memory, which is also where a launch per
 // step catches up: several bricks per SM (192 x 173 x 159, five each) took
 // 21 / 23 / 32 us against 25 / 26 / 27.
+// Off the grid a receiver is up to 8^3 taps and its neighbours share bricks:
+// taken by the bricks that they reach, 1024 receivers made a step 13.2 / 39.4
+// us (3969: 17.2 / 120). So the blocks share the receivers out evenly and the
+// data go through one of two padded fields, a step ahead (3969: 15.7 / 19.8).
 // What is left at 104^3: about 4 us of shared-memory reads and instructions,
 // the rest barrier, copy and store latency (3.1 us on the smallest grid).
 //
@@ -52,6 +57,7 @@ namespace {
 // leave a block few columns spread them over four times the threads
 constexpr int kColumn = 4;
 constexpr int kListCap = 2048;                           // receivers of a block kept in shared memory
+constexpr int kTapCap = 32;                              // tap tables of a block kept in shared memory
 constexpr unsigned long long kBarrierNs = 20000000000ull;  // bound of a grid barrier: 20 s
 constexpr int kSmemMax = 227 * 1024;
 
@@ -61,6 +67,8 @@ template <int R, bool BWD, int PZ>
 __host__ __device__ constexpr int span_threads() {
     return PZ == 1 || R == 4 ? 512 : 384;
 }
+
+static_assert(sizeof(rtm_point_taps) * kTapCap <= 4 * kListCap, "tap tables share the list's room");
 
 struct SpanMaps {
     CUtensorMap u[2];
@@ -171,14 +179,20 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
     k_span(const __grid_constant__ SpanArgs A, const __grid_constant__ SpanMaps M) {
     extern __shared__ __align__(128) float dsm[];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ int s_ok, s_count;
+    __shared__ int s_ok, s_count, s_zlo, s_zhi;
+    __shared__ rtm_point_taps s_src;  // OFF: the source
     const SpanPlan& P = A.P;
     const int tid = threadIdx.x, T = blockDim.x;
     const int SW = 4 * P.bxv + 2 * R, SH = P.by + 2 * R, SD = P.bz + 2 * R;
     const int box = SW * SH * SD;
     const int bx = 4 * P.bxv, cells = bx * P.by * P.bz;
     float* inj = dsm + ((box + 31) & ~31);                 // BWD: receiver data by cell of the brick
-    int* list = reinterpret_cast<int*>(inj + cells);       // BWD: receivers that reach the brick
+    // BWD: receivers that reach the brick; OFF: tap tables of the receivers
+    // that this block gathers or scatters (every gridDim.x-th)
+    int* list = reinterpret_cast<int*>(inj + (BWD ? cells : 0));
+    rtm_point_taps* tables = reinterpret_cast<rtm_point_taps*>(list);
+    const bool scatter = OFF && BWD && A.scatter[0] != nullptr;
+    const int my_recs = (A.nrec - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     const size_t plane = (size_t)A.NX * A.NY;
     const int ix = blockIdx.x % P.nbx, iyz = blockIdx.x / P.nbx;
     const int x0 = ix * bx, y0 = iyz % P.nby * P.by, z0 = iyz / P.nby * P.bz;  // the brick
@@ -187,6 +201,9 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&bar)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_count = 0;
+        s_zlo = A.NZ;
+        s_zhi = -1;
+        if (OFF && !BWD) s_src = A.taps[0];
         s_ok = *reinterpret_cast<volatile int*>(&A.ctrl->abort) == 0;
     }
     __syncthreads();
@@ -205,7 +222,18 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
     int nlist = 0;
     if constexpr (BWD) {
         for (int i = tid; i < cells; i += T) inj[i] = 0.f;
-        if (A.rdata) {
+        if (scatter) {
+            // the planes that any receiver's taps reach
+            int lo = A.NZ, hi = -1;
+            for (int j = tid; j < A.nrec; j += T) {
+                const rtm_point_taps& t = A.taps[1 + j];
+                if (taps_outside(t, A) && taps_of(t) == 0) continue;
+                lo = min(lo, max(t.k0, 0));
+                hi = max(hi, min(t.k0 + t.nz, A.NZ) - 1);
+            }
+            atomicMin(&s_zlo, lo);
+            atomicMax(&s_zhi, hi);
+        } else if (A.rdata) {
             for (int j = tid; j < A.nrec; j += T) {
                 bool hit;
                 if constexpr (OFF) {
@@ -228,6 +256,29 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
         __syncthreads();
         nlist = s_count;
     }
+    if constexpr (OFF) {
+        if (!BWD || scatter)
+            for (int k = tid; k < min(my_recs, kTapCap); k += T)
+                tables[k] = A.taps[1 + blockIdx.x + k * gridDim.x];
+        __syncthreads();
+    }
+    // receiver blockIdx.x + k gridDim.x
+    auto table = [&](int k) -> const rtm_point_taps& {
+        return k < kTapCap ? tables[k] : A.taps[1 + blockIdx.x + k * gridDim.x];
+    };
+    // OFF: many receivers' taps meet in few bricks, so all blocks take a share
+    // of them and add the data of step m into a padded field, which the cells'
+    // owners read (and clear) one barrier later
+    auto scatter_taps = [&](int m, float* field) {
+        const float* row = A.rdata + (size_t)(m - 1) * A.nrec;
+        for (int k = tid >> 5; k < my_recs; k += T >> 5) {
+            const float r = row[blockIdx.x + k * gridDim.x];
+            for_taps(table(k), tid & 31, [&](int x, int y, int z, float w) {
+                if (x >= 0 && x < A.NX && y >= 0 && y < A.NY && z >= 0 && z < A.NZ)
+                    atomicAdd(field + (size_t)z * plane + (size_t)y * A.NX + x, w * r);
+            });
+        }
+    };
     // the data of step m at the brick's receivers, summed per cell (times the
     // tap weights). They need no other block's work, so they are formed while
     // the grid barrier is under way
@@ -339,6 +390,22 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
                 for (int v = 0; v < 4; v++) gxy.v[v] = gxv.v[v] * gyv;
             }
             wait_here();
+            bool hit = nlist > 0;  // receivers' data may lie in these cells
+            float* given = BWD ? &inj[(PZ * zg * P.by + ty) * bx + 4 * tx] : nullptr;
+            if constexpr (OFF && BWD) {
+                if (scatter && z <= s_zhi && z + PZ > s_zlo) {
+                    hit = true;
+                    float* src = A.scatter[i & 1] + o;
+#pragma unroll
+                    for (int p = 0; p < PZ; p++)
+                        if (z + p < A.NZ)
+                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                             su32(given + p * P.by * bx)),
+                                         "l"(src + p * plane)
+                                         : "memory");
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                }
+            }
             // the z column of the vector: planes z - R .. z + PZ - 1 + R
             const float* colp = dsm + (PZ * zg * SH + R + ty) * SW + R + 4 * tx;
             F4 zc[PZ + 2 * R];
@@ -403,7 +470,7 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
                 if constexpr (!BWD) {
                     // the source: lower u^{n-1} by c w / (dx^3 g^2)
                     if constexpr (OFF) {
-                        const rtm_point_taps& t = A.taps[0];
+                        const rtm_point_taps& t = s_src;
                         const int dz = z + p - t.k0, dy = y - t.j0;
                         if (dz >= 0 && dz < t.nz && dy >= 0 && dy < t.ny && taps_of(t) > 0) {
 #pragma unroll
@@ -424,9 +491,9 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
                                 up[p & 1].v[e] -= cc[p & 1].v[e] * w * A.inv_dx3 / (g * g);
                             }
                     }
-                } else if (nlist > 0) {
-                    float4* ip = reinterpret_cast<float4*>(
-                        &inj[((PZ * zg + p) * P.by + ty) * (4 * P.bxv) + 4 * tx]);
+                } else if (hit) {
+                    if (OFF && p == 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    float4* ip = reinterpret_cast<float4*>(given + p * P.by * bx);
                     const float4 t = *ip;
                     if (t.x != 0.f || t.y != 0.f || t.z != 0.f || t.w != 0.f) {
                         // lower u^{m+1} by c r / (dx^3 g): the step adds c g r / dx^3
@@ -436,7 +503,10 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
                             if (r[e] != 0.f)
                                 up[p & 1].v[e] +=
                                     -cc[p & 1].v[e] * r[e] * A.inv_dx3 / (gxy.v[e] * gzv);
-                        *ip = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (OFF && scatter)
+                            st_plain4(A.scatter[i & 1] + o + p * plane, zero4());
+                        else
+                            *ip = make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                 }
                 F4 out;
@@ -514,14 +584,31 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
                 float* row = A.data + (size_t)(n - 1) * A.nrec;
                 if constexpr (OFF) {
                     const int lane = tid & 31;
-                    for (int j = (blockIdx.x * T + tid) >> 5; j < A.nrec; j += (gridDim.x * T) >> 5) {
+                    for (int k = tid >> 5; k < my_recs; k += T >> 5) {
+                        // a lane's columns of the box, their z taps in flight together
+                        const rtm_point_taps& t = table(k);
+                        const int n0 = t.nx, nxy = taps_of(t) ? t.nx * t.ny : 0;
                         float sum = 0.f;
-                        for_taps(A.taps[1 + j], lane, [&](int x, int y, int z, float wt) {
-                            if (x >= 0 && x < A.NX && y >= 0 && y < A.NY && z >= 0 && z < A.NZ)
-                                sum += wt * __ldcg(cur + (size_t)z * plane + (size_t)y * A.NX + x);
-                        });
+#pragma unroll 2
+                        for (int q = lane; q < nxy; q += 32) {
+                            const int tb = q / n0, ta = q - tb * n0;
+                            const int x = t.i0 + ta, y = t.j0 + tb;
+                            const bool in = x >= 0 && x < A.NX && y >= 0 && y < A.NY;
+                            const float* src =
+                                cur + (long long)t.k0 * (long long)plane + (long long)y * A.NX + x;
+                            float u[8];
+#pragma unroll
+                            for (int c = 0; c < 8; c++)
+                                u[c] = in && c < t.nz && t.k0 + c >= 0 && t.k0 + c < A.NZ
+                                           ? __ldcg(src + c * plane)
+                                           : 0.f;
+                            const float wxy = t.wx[ta] * t.wy[tb];
+#pragma unroll
+                            for (int c = 0; c < 8; c++)
+                                if (c < t.nz) sum += wxy * t.wz[c] * u[c];
+                        }
                         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                        if (lane == 0) row[j] = sum;
+                        if (lane == 0) row[blockIdx.x + k * gridDim.x] = sum;
                     }
                 } else {
                     if (j0 < A.nrec) row[j0] = d0;
@@ -538,12 +625,26 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
             if (A.src_adj && n < A.nt && blockIdx.x == 0 && tid == 0)
                 A.src_adj[n] = __ldcg(cur + A.src) / (A.gx[srx] * A.gy[sry] * A.gz[srz]);
         }
+        if constexpr (OFF && BWD) {
+            if (scatter && i + 1 < A.nsteps) scatter_taps(n - 1, A.scatter[(i + 1) & 1]);
+        }
         if (i + 1 < A.nsteps) {
             __syncthreads();  // the box, the receiver terms and the block's writes are done with
             if (tid == 0) grid_arrive(A.ctrl);
             if constexpr (BWD) inject(n - 1);
         }
     }
+}
+
+// the data of a span's first step, as scatter_taps does for the others
+__global__ void k_scatter_first(const __grid_constant__ SpanArgs A) {
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (j >= A.nrec) return;
+    const float r = A.rdata[(size_t)(A.first - 1) * A.nrec + j];
+    for_taps(A.taps[1 + j], threadIdx.x & 31, [&](int x, int y, int z, float w) {
+        if (x >= 0 && x < A.NX && y >= 0 && y < A.NY && z >= 0 && z < A.NZ)
+            atomicAdd(A.scatter[0] + ((size_t)z * A.NY + y) * A.NX + x, w * r);
+    });
 }
 
 cudaError_t encode_box(CUtensorMap* m, const float* base, const SpanArgs& a, int R) {
@@ -566,6 +667,13 @@ cudaError_t launch_span_t(const SpanArgs& a, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kSmemMax - 1024);
     if (e != cudaSuccess) return e;
+    if (OFF && BWD && a.scatter[0] && a.nrec > 0) {
+        const size_t bytes = sizeof(float) * a.NX * a.NY * a.NZ;
+        for (int i = 0; i < 2; i++)
+            if ((e = cudaMemsetAsync(a.scatter[i], 0, bytes, s)) != cudaSuccess) return e;
+        k_scatter_first<<<(a.nrec + 7) / 8, 256, 0, s>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     SpanMaps M;
     memset(&M, 0, sizeof M);
     for (int i = 0; i < 2; i++)
@@ -660,7 +768,9 @@ SpanPlan span_plan(int R, int NX, int NY, int NZ, int backward) {
                     if (nbricks > sms) break;  // one brick per SM
                     const long long box = (long long)(4 * bxv + 2 * R) * (by + 2 * R) * (bz + 2 * R);
                     const long long smem = (box + 31) / 32 * 128 +
-                                           (backward ? 16LL * bxv * by * bz + 4 * kListCap : 0) + 128;
+                                           (backward ? 16LL * bxv * by * bz + 4 * kListCap
+                                                     : (long long)sizeof(rtm_point_taps) * kTapCap) +
+                                           128;
                     if (smem > kSmemMax - 1024) continue;
                     const int items = bxv * by * (bz / pz);
                     const int rounds = (items + T - 1) / T;

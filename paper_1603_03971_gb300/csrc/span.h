@@ -45,6 +45,7 @@ struct SpanArgs {
     float inv_dx3;
     float* data;         // forward: d[n-1] = u^n at the receivers (n >= 1), or NULL
     const float* rdata;  // backward: rows injected at the receivers
+    float* scatter[2];   // backward, tap table: padded fields of scratch, or NULL
     float* src_adj;      // backward: trace at the source, or NULL
     // snapshot of state k (k = n + 1 forward, m backward): written or imaged
     // with where k % every == 0, at snap + (k / div - off) * stride; NULL: none

@@ -148,6 +148,38 @@ def test_off_grid_shot_matches_the_launches(r):
     assert rel_l2(img, img_ref) <= 7e-6
 
 
+@pytest.mark.parametrize("r,storage,ckpt,nrec", [
+    (4, "all", 0, 1), (4, "ckpt", 9, 6000), (4, "revolve", 3, 700), (8, "revolve", 3, 6000),
+    (4, "boundary", 0, 700)])
+def test_off_grid_receivers_beyond_a_blocks_tables(r, storage, ckpt, nrec):
+    """One receiver, a few per block and more than a block keeps tap tables
+    for (32), also where no padded fields are left to scatter into."""
+    import torch
+
+    import paper_1603_03971_gb300 as rtm
+
+    case = Case(r=r, nt=23, storage=storage, ckpt_every=ckpt, nx=46, ny=43, nz=37, nb=9)
+    rng = np.random.default_rng(5)
+    pts = rng.uniform((0, 0, 1), (45, 42, 4.5), (nrec, 3))
+    g = DeviceShot(case)
+    p = g.p.copy(nrec=nrec)
+    ws = rtm.alloc_workspace(p)
+    taps = rtm.offgrid_taps(p, (20.3, 20.6, 3.5), pts, "cuda")
+    dobs = torch.from_numpy(case.d_obs(nrec).astype(np.float32)).cuda()
+
+    def run():
+        img = torch.zeros(rtm.model_shape(p), device="cuda")
+        data = torch.empty((p.nt, nrec), device="cuda")
+        rtm.shot_offgrid(p, g.c, taps, dobs, ws, img, data=data)
+        rtm.check(ws)
+        return img.cpu().numpy(), data.cpu().numpy()
+    (img, data), (img_ref, data_ref) = _both(r, run)
+    # as above, with the terms of a cell: each of its 8^3 neighbours' receivers
+    # (6000 over 45 x 42 x 3.5: about 0.9 per cell, 512 taps each way)
+    assert rel_l2(data, data_ref) <= 7e-6
+    assert rel_l2(img, img_ref) <= 7e-6
+
+
 def test_receivers_outside_are_reported_and_skipped():
     import paper_1603_03971_gb300 as rtm
 
