@@ -26,6 +26,7 @@
 
 #include "ae_internal.h"
 #include "ae_train.h"
+#include "pdl.cuh"
 #include "tc_gemm.cuh"
 
 namespace rtm {
@@ -484,13 +485,15 @@ struct OpD2d {  // gy (bf16, full grid) -> ga3 = (W4^T gy) * leaky'(a3)
 // ============================================================================
 // CUDA-core kernels
 // ============================================================================
+constexpr int kSumsqBlocks = 6;  // resident blocks per SM
+
 // sum of squares of a strided volume: float partials per thread (four
 // accumulators over at most a few hundred values), a block reduction in
 // double, one atomic per block. A contiguous 16-byte aligned volume is read
 // as one flat float4 array, four loads in flight per thread; otherwise a
 // warp per row of x (float4 loads when rows are 16-byte aligned), 8 rows per
 // block
-__global__ void __launch_bounds__(256) k_sumsq(Vol in, double* acc) {
+__global__ void __launch_bounds__(256, kSumsqBlocks) k_sumsq(Vol in, double* acc) {
     const long long rows = (long long)in.ny * in.nz;
     const int lane = threadIdx.x, nx4 = in.nx >> 2;
     const bool vec = ((reinterpret_cast<uintptr_t>(in.p) & 15) == 0) && (in.sy % 4 == 0) &&
@@ -553,11 +556,15 @@ __global__ void __launch_bounds__(256) k_sumsq(Vol in, double* acc) {
     }
 }
 
-__global__ void k_scale(const double* acc, long long n, float* sigma, float* inv_sigma) {
+// sigma_out: the caller's copy of the scale, or NULL
+__global__ void k_scale(const double* acc, long long n, float* sigma, float* inv_sigma,
+                        float* sigma_out) {
+    pdl_wait();
     double r = sqrt(*acc / (double)n);
     if (!(r > 0.0)) r = 1.0;
     *sigma = (float)r;
     *inv_sigma = (float)(1.0 / r);
+    if (sigma_out) *sigma_out = (float)r;
 }
 
 // loss += mean((y - x0)^2) * scale; gy = bf16(scale * 2 (y - x0) / n); grad[b4] += sum gy.
@@ -677,15 +684,17 @@ cudaError_t ae_gemm_test(const GemmArgs& a, int N, int* status, cudaStream_t s) 
     return cudaErrorInvalidValue;
 }
 
-cudaError_t ae_rms(const Vol& in, AeScalars* sc, cudaStream_t s) {
+cudaError_t ae_rms(const Vol& in, AeScalars* sc, cudaStream_t s, float* sigma_out) {
     cudaError_t e = cudaMemsetAsync(&sc->sumsq, 0, sizeof(double), s);
     if (e != cudaSuccess) return e;
     const long long n = (long long)in.nx * in.ny * in.nz;
     long long blocks = ((long long)in.ny * in.nz + 7) / 8;
-    if (blocks > 152 * 8) blocks = 152 * 8;
+    // one wave of resident blocks
+    if (blocks > 152 * kSumsqBlocks) blocks = 152 * kSumsqBlocks;
     k_sumsq<<<(unsigned)blocks, dim3(32, 8), 0, s>>>(in, &sc->sumsq);
-    k_scale<<<1, 1, 0, s>>>(&sc->sumsq, n, &sc->sigma, &sc->inv_sigma);
-    return cudaGetLastError();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_next(k_scale, dim3(1), dim3(1), 0, s, &sc->sumsq, n, &sc->sigma, &sc->inv_sigma,
+                       sigma_out);
 }
 
 cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScalars* sc,
@@ -693,10 +702,10 @@ cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScal
     cudaError_t e = cudaSuccess;
     if (sumsq_ready) {
         k_scale<<<1, 1, 0, s>>>(&sc->sumsq, (long long)in.nx * in.ny * in.nz, &sc->sigma,
-                                &sc->inv_sigma);
+                                &sc->inv_sigma, sigma_out);
         e = cudaGetLastError();
     } else {
-        e = ae_rms(in, sc, s);
+        e = ae_rms(in, sc, s, sigma_out);
     }
     if (e != cudaSuccess) return e;
     const Dims3 h{in.nx / 2, in.ny / 2, in.nz / 2}, l{in.nx / 4, in.ny / 4, in.nz / 4};
@@ -709,9 +718,6 @@ cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScal
         E2Args a2{h1, h, P, lat, l};
         e = run_async<OpE2>(a2, dim3(tiles((long long)l.nx * l.ny * l.nz)), status, s);
     }
-    if (e != cudaSuccess) return e;
-    if (sigma_out) e = cudaMemcpyAsync(sigma_out, &sc->sigma, sizeof(float),
-                                       cudaMemcpyDeviceToDevice, s);
     return e;
 }
 

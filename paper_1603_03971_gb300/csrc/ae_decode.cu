@@ -57,12 +57,14 @@ constexpr int kPlaneBytes = 2 * kHalfBytes;
 constexpr int kTmaBytes = 2 * HX * HY * 16;    // bytes one plane load delivers
 constexpr int kSlots = 9;                      // plane ring
 constexpr int kW3Bytes = 64 * 1024;            // 64 B operands (parity, tap): 32 x 16, 1 KB each
-constexpr int kA2Bytes = 128 * 32 * 2;          // D2 A operand: 128 rows x 32 channels, bf16
 // W3 operands, plane ring, b3 (128 B), the D2 B operand W4 (16 x 32 bf16,
-// 1 KB), four D2 A operands per epilogue warpgroup: > half an SM, 1 CTA
-constexpr int kSmem = 128 + kW3Bytes + kSlots * kPlaneBytes + 128 + 1024 + 2 * 4 * kA2Bytes;
+// 1 KB): > half an SM, 1 CTA
+constexpr int kGroups = 4;                     // epilogue warpgroups
+constexpr int kSmem = 128 + kW3Bytes + kSlots * kPlaneBytes + 128 + 1024;
+static_assert(2 * kSmem > 228 * 1024, "one CTA per SM: all of its tensor memory is taken");
 constexpr int kTmemCols = 512;
-constexpr int kThreads = 320;
+constexpr int kMmaWarp = 4 * kGroups, kLoadWarp = kMmaWarp + 1;
+constexpr int kThreads = (kLoadWarp + 1) * 32;
 constexpr long long kLimit = 1LL << 24;
 constexpr uint32_t kSuspendNs = 20000;  // longest sleep of one poll (woken by the phase)
 
@@ -168,6 +170,29 @@ __device__ __forceinline__ bool wg_all(bool v, int id) {
         : "memory");
     return r != 0;
 }
+// r into 16 columns of this warp's lanes; tmem_wait_st before anyone reads them
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]),
+        "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+// as tc::mma_bf16 with A in tensor memory: row r in lane r, two K values per column
+__device__ __forceinline__ void mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc,
+                                            uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
 // 8 columns of this warp's lanes into r, without waiting (as tmem_ld16_nw)
 __device__ __forceinline__ void tmem_ld8_nw(uint32_t taddr, uint32_t* r) {
     asm volatile(
@@ -187,8 +212,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     k_decode_march(const __grid_constant__ D12Args A, const __grid_constant__ CUtensorMap map,
                    const Sched S, int* status) {
     extern __shared__ uint8_t dsm_raw[];
-    __shared__ __align__(8) uint64_t full[kSlots], freed[kSlots], acc_full[2], acc_free[2], fin,
-        d2_full[2];
+    __shared__ __align__(8) uint64_t full[kSlots], freed[kSlots], acc_full[kGroups],
+        acc_free[kGroups], fin, d2_full[kGroups];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
@@ -198,7 +223,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* ring = base + kW3Bytes;
     float* b3s = reinterpret_cast<float*>(ring + kSlots * kPlaneBytes);  // b3[32]
     uint8_t* b4t = ring + kSlots * kPlaneBytes + 128;  // W4 as a 16 x 32 K-major operand
-    uint8_t* a2 = b4t + 1024;                          // D2 A operands
 
     const D1Args& d = A.d1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -209,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc::mbar_init(&full[s], 1);
             tc::mbar_init(&freed[s], 1);
         }
-        for (int b = 0; b < 2; b++) {
+        for (int b = 0; b < kGroups; b++) {
             tc::mbar_init(&acc_full[b], 1);
             tc::mbar_init(&acc_free[b], 128);
             tc::mbar_init(&d2_full[b], 1);
@@ -220,26 +244,40 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (warp == 0) tc::tmem_alloc(&tmem_slot, kTmemCols);
     // B operands: (parity q, tap tau) -> W3[o][kz][ky][kx][i] as a 32 x 16 K-major tile
-    for (int idx = tid; idx < 64 * 32 * 2; idx += kThreads) {
-        const int j = idx & 1, o = (idx >> 1) & 31, t = idx >> 6, q = t >> 3, tau = t & 7;
-        int tz, kz, ty, ky, tx, kx;
-        taps(q >> 2, tau >> 2, tz, kz);
-        taps((q >> 1) & 1, (tau >> 1) & 1, ty, ky);
-        taps(q & 1, tau & 1, tx, kx);
-        const int ktap = (kz * 4 + ky) * 4 + kx;
-        float w[8];
+    const bool wvec = (reinterpret_cast<uintptr_t>(d.P) & 15) == 0;
+    static_assert(kOW3 % 4 == 0 && kOW4 % 4 == 0, "16-byte weight loads");
+    constexpr int kStage = 4;  // operand rows in flight per thread
+    for (int i0 = tid; i0 < 64 * 32 * 2; i0 += kStage * kThreads) {
+        float w[kStage][8];
 #pragma unroll
-        for (int e = 0; e < 8; e++) w[e] = d.P[kOW3 + o * 1024 + ktap * 16 + 8 * j + e];
-        *reinterpret_cast<uint4*>(w3 + w3_block(q, tau) * 1024 + b_off(o, 8 * j)) =
-            tc::pack8(w);
+        for (int k = 0; k < kStage; k++) {
+            const int idx = min(i0 + k * kThreads, 64 * 32 * 2 - 1);
+            const int j = idx & 1, o = (idx >> 1) & 31, t = idx >> 6, q = t >> 3, tau = t & 7;
+            int tz, kz, ty, ky, tx, kx;
+            taps(q >> 2, tau >> 2, tz, kz);
+            taps((q >> 1) & 1, (tau >> 1) & 1, ty, ky);
+            taps(q & 1, tau & 1, tx, kx);
+            load8(d.P + kOW3 + o * 1024 + ((kz * 4 + ky) * 4 + kx) * 16 + 8 * j, wvec, w[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kStage; k++) {
+            const int idx = i0 + k * kThreads;
+            if (idx >= 64 * 32 * 2) break;
+            const int j = idx & 1, o = (idx >> 1) & 31, t = idx >> 6;
+            *reinterpret_cast<uint4*>(w3 + w3_block(t >> 3, t & 7) * 1024 + b_off(o, 8 * j)) =
+                tc::pack8(w[k]);
+        }
     }
     // W4[e][c] (e = (ez, ey, ex), c = channel) as rows e of a 16 x 32 K-major
     // bf16 operand, rows 8..15 zero
     for (int idx = tid; idx < 16 * 4; idx += kThreads) {
         const int e = idx >> 2, c8 = (idx & 3) * 8;
         float w[8];
+        load8(d.P + kOW4 + (e & 7) * 32 + c8, wvec, w);
+        if (e >= 8) {
 #pragma unroll
-        for (int i = 0; i < 8; i++) w[i] = e < 8 ? d.P[kOW4 + e * 32 + c8 + i] : 0.f;
+            for (int i = 0; i < 8; i++) w[i] = 0.f;
+        }
         tc::st_vec8(b4t, e, c8, tc::pack8(w));
     }
     if (tid < 32) b3s[tid] = d.P[kOB3 + tid];
@@ -250,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = tmem_slot;
     const int lnx = d.l.nx, lny = d.l.ny, lnz = d.l.nz;
 
-    if (warp == 8) {
+    if (warp == kMmaWarp) {
         if (lane == 0) {
             // ---------------- MMA issuer ----------------
             constexpr uint32_t idesc = tc::idesc_bf16(128, 32), idesc64 = tc::idesc_bf16(128, 64);
@@ -265,7 +303,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int s = base_seq + zi; s <= base_seq + zi + 2 && ok; s++)
                         ok = wait_bar(&full[s % kSlots], (uint32_t)((s / kSlots) & 1), abrt);
                     const int b = out & 1, u = out >> 1;
-                    if (ok && u >= 1) ok = wait_bar(&acc_free[b], (uint32_t)((u - 1) & 1), abrt);
                     if (!ok) break;
                     tc::tc_fence_after();
                     // descriptors: the start-address field is address >> 4 and no
@@ -289,6 +326,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // parity overwriting its accumulator. 52 MMAs per plane
 #pragma unroll
                     for (int m = 0; m < 4; m++) {
+                        // a half plane (z parity) is one epilogue warpgroup's
+                        if ((m & 1) == 0) {
+                            if (u >= 1)
+                                ok = wait_bar(&acc_free[2 * b + (m >> 1)], (uint32_t)((u - 1) & 1),
+                                              abrt);
+                            if (!ok) break;
+                            tc::tc_fence_after();
+                        }
                         const uint32_t c0 = tmem + b * 256 + (2 * m) * 32, c1 = c0 + 32;
 #pragma unroll
                         for (int g = 0; g < 4; g++) {
@@ -308,8 +353,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 tc::mma_bf16(c0, a + 0, bg + 3 * 64, idesc, 1u);   // q0, x tap 1
                             }
                         }
+                        if (m & 1) tc::mma_commit(&acc_full[2 * b + (m >> 1)]);
                     }
-                    tc::mma_commit(&acc_full[b]);
+                    if (!ok) break;
                     // plane z - 1 is read by no later output of this item
                     tc::mma_commit(&freed[(base_seq + zi) % kSlots]);
                     if (zi == nz - 1) {
@@ -324,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc::mma_commit(&fin);
             if (!wait_bar(&fin, 0, nullptr)) *abrt = 1;
         }
-    } else if (warp == 9) {
+    } else if (warp == kLoadWarp) {
         if (lane == 0) {
             // ---------------- plane loader ----------------
             // every latent plane of every item (with its z halo) into the next
@@ -354,19 +400,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else {
         // ---------------- epilogue warpgroups ----------------
-        const int g = warp >> 2, row = tid & 127, ly = row >> 3, lx = row & 7;
+        const int g = warp >> 2, qz = g & 1, row = tid & 127, ly = row >> 3, lx = row & 7;
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const float b4 = d.P[kOB4];
         const float sc = A.sigma ? *A.sigma : 1.0f;
         const bool vec = ((reinterpret_cast<uintptr_t>(A.out.p) & 15) == 0) &&
                          (A.out.sy % 4 == 0) && (A.out.sz % 4 == 0);
-        // b3 as packed pairs and the slope as a pair (f32x2 arithmetic, IEEE
-        // single precision per lane)
-        uint64_t b3p[16];
-#pragma unroll
-        for (int c = 0; c < 16; c++) b3p[c] = f32x2::pack(b3s[2 * c], b3s[2 * c + 1]);
+        // the slope as a pair (f32x2 arithmetic, IEEE single precision per lane)
         const uint64_t slope2 = f32x2::pack(kSlope, kSlope);
-        uint8_t* atile = a2 + g * 4 * kA2Bytes;  // this warpgroup's four D2 A operands
         constexpr uint32_t idesc2 = tc::idesc_bf16(128, 16);
         int out = 0, d2_phase = 0;
         bool ok = true, d2_pending = false;
@@ -376,66 +417,54 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int X = cx * TX + lx, Y = cy * TY + ly;
             const bool valid = X < lnx && Y < lny;
             for (int zi = 0; zi < nz; zi++, out++) {
-                if ((out & 1) != g) continue;
+                if ((out & 1) != g >> 1) continue;
                 const int u = out >> 1;
                 ok = wg_all(wait_bar(&acc_full[g], (uint32_t)(u & 1), abrt), 1 + g);
                 if (!ok) break;
                 tc::tc_fence_after();
                 const int Z = z0 + zi;
-                const uint32_t tb = lane_base + g * 256;
-#pragma unroll 1
-                for (int qz = 0; qz < 2 && ok; qz++) {
+                const uint32_t tb = lane_base + g * 128;
+                {
                     // g1 = bf16(LeakyReLU(acc + b3)) of the four parities (qz, qy, qx)
                     // into the A operands (row = latent voxel, K = channel), one
                     // parity's TMEM load in flight while the one before it is
                     // processed; LeakyReLU as max(h, slope h) on packed pairs (the
                     // same bits as the select form for 0 < slope < 1)
-                    auto tile = [&](int p4, const uint32_t* r) {
-                        uint8_t* t = atile + p4 * kA2Bytes;
+                    auto half_row = [&](int half, const uint32_t* r, uint32_t* w) {
+                        // b3 from shared memory (pairs, one address for all
+                        // lanes): the registers hold two accumulator halves
+                        const ulonglong2* b3p =
+                            reinterpret_cast<const ulonglong2*>(b3s + 16 * half);
 #pragma unroll
-                        for (int k8 = 0; k8 < 4; k8++) {
-                            uint32_t w[4];
-#pragma unroll
-                            for (int c = 0; c < 4; c++) {
-                                const int i = 8 * k8 + 2 * c;
-                                const uint64_t h = f32x2::add(
-                                    f32x2::pack(__uint_as_float(r[i]), __uint_as_float(r[i + 1])),
-                                    b3p[i >> 1]);
-                                const uint64_t sh = f32x2::mul(h, slope2);
-                                float h0, h1, s0, s1;
-                                f32x2::unpack(h, h0, h1);
-                                f32x2::unpack(sh, s0, s1);
-                                w[c] = tc::pack2(fmaxf(h0, s0), fmaxf(h1, s1));
-                            }
-                            tc::st_vec8(t, row, 8 * k8, make_uint4(w[0], w[1], w[2], w[3]));
+                        for (int c = 0; c < 8; c++) {
+                            const uint64_t h = f32x2::add(
+                                f32x2::pack(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])),
+                                c & 1 ? b3p[c >> 1].y : b3p[c >> 1].x);
+                            const uint64_t sh = f32x2::mul(h, slope2);
+                            float h0, h1, s0, s1;
+                            f32x2::unpack(h, h0, h1);
+                            f32x2::unpack(sh, s0, s1);
+                            w[c] = tc::pack2(fmaxf(h0, s0), fmaxf(h1, s1));
                         }
                     };
-                    const uint32_t cq = tb + qz * 4 * 32;
-                    uint32_t x0[32], x1[32];
-                    tmem_ld16_nw(cq, x0);
-                    tmem_ld16_nw(cq + 16, x0 + 16);
-                    tmem_wait_regs16(x0);
-                    tmem_wait_regs16(x0 + 16);
-                    tmem_ld16_nw(cq + 32, x1);
-                    tmem_ld16_nw(cq + 48, x1 + 16);
-                    tile(0, x0);
-                    tmem_wait_regs16(x1);
-                    tmem_wait_regs16(x1 + 16);
-                    tmem_ld16_nw(cq + 64, x0);
-                    tmem_ld16_nw(cq + 80, x0 + 16);
-                    tile(1, x1);
-                    tmem_wait_regs16(x0);
-                    tmem_wait_regs16(x0 + 16);
-                    tmem_ld16_nw(cq + 96, x1);
-                    tmem_ld16_nw(cq + 112, x1 + 16);
-                    tile(2, x0);
-                    tmem_wait_regs16(x1);
-                    tmem_wait_regs16(x1 + 16);
-                    tile(3, x1);
-                    // the generic-proxy tile writes and the drained accumulator
-                    // columns, then one thread issues the D2 products into those
-                    // columns: [128 x 32] g1 x [32 x 16] W4 (rows 8..15 zero)
-                    tc::fence_proxy_async();
+                    uint32_t x0[16], x1[16];
+                    tmem_ld16_nw(tb, x0);
+#pragma unroll
+                    for (int p = 0; p < 4; p++) {
+                        tmem_wait_regs16(x0);
+                        tmem_ld16_nw(tb + p * 32 + 16, x1);
+                        uint32_t w[16];
+                        half_row(0, x0, w);
+                        tmem_wait_regs16(x1);
+                        if (p < 3) tmem_ld16_nw(tb + p * 32 + 32, x0);
+                        half_row(1, x1, w + 8);
+                        tmem_st16(tb + p * 32 + 16, w);
+                    }
+                    // the operands and the drained accumulator columns, then one
+                    // thread issues the D2 products: [128 x 32] g1 (columns 16-31
+                    // of the parity's 32) x [32 x 16] W4 (rows 8..15 zero) into
+                    // columns 0-15
+                    tmem_wait_st();
                     tc::tc_fence_before();
                     asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
                     if (row == 0) {
@@ -443,11 +472,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint64_t dB = tc::sdesc(tc::smem_u32(b4t), 128, 512);
 #pragma unroll
                         for (int p = 0; p < 4; p++) {
-                            const uint64_t dA =
-                                tc::sdesc(tc::smem_u32(atile + p * kA2Bytes), 128, 512);
-                            const uint32_t dcol = tmem + g * 256 + (qz * 4 + p) * 32;
-                            tc::mma_bf16(dcol, dA, dB, idesc2, 0u);
-                            tc::mma_bf16(dcol, dA + 16, dB + 16, idesc2, 1u);  // K 16..31
+                            const uint32_t dcol = tmem + g * 128 + p * 32;
+                            mma_bf16_ta(dcol, dcol + 16, dB, idesc2, 0u);
+                            mma_bf16_ta(dcol, dcol + 24, dB + 16, idesc2, 1u);  // K 16..31
                         }
                         tc::mma_commit(&d2_full[g]);
                         d2_pending = true;
@@ -461,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tc::tc_fence_after();
                     uint32_t ry[32];
 #pragma unroll
-                    for (int p = 0; p < 4; p++) tmem_ld8_nw(tb + (qz * 4 + p) * 32, ry + 8 * p);
+                    for (int p = 0; p < 4; p++) tmem_ld8_nw(tb + p * 32, ry + 8 * p);
                     tmem_wait_regs16(ry);
                     tmem_wait_regs16(ry + 16);
                     float y[4][8];

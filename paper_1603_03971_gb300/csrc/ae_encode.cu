@@ -65,6 +65,7 @@
 #include "../../include/rtm.h"
 #include "ae_internal.h"
 #include "packed_f32x2.cuh"
+#include "pdl.cuh"
 #include "rtm_internal.h"
 #include "tc_gemm.cuh"
 #include "tma_encode.h"
@@ -305,12 +306,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) tc::tmem_alloc(&tmem_slot, kTmemCols);
     // E2 B operands: (tap, half) -> W2[o][tap][16 half + i], 16-row K-major
     // blocks in region C (kz 0 and 2) or K1 (kz 1)
-    for (int idx = tid; idx < 54 * 16 * 2; idx += kThreads) {
-        const int j = idx & 1, o = (idx >> 1) & 15, t = idx >> 5, tap = t >> 1, hh = t & 1;
-        float w[8];
+    const bool wvec = (reinterpret_cast<uintptr_t>(A.P) & 15) == 0;
+    static_assert(kOW1 % 4 == 0 && kOW2 % 4 == 0, "16-byte weight loads");
+    constexpr int kStage = 4;  // operand rows of a thread, all in flight
+    static_assert(kStage * kThreads >= 54 * 16 * 2, "one pass over the operand rows");
+    float w2r[kStage][8];
 #pragma unroll
-        for (int e = 0; e < 8; e++) w[e] = A.P[kOW2 + o * 864 + tap * 32 + 16 * hh + 8 * j + e];
-        const uint4 v = tc::pack8(w);
+    for (int k = 0; k < kStage; k++) {
+        const int idx = min(tid + k * kThreads, 54 * 16 * 2 - 1);
+        const int j = idx & 1, o = (idx >> 1) & 15, t = idx >> 5;
+        load8(A.P + kOW2 + o * 864 + (t >> 1) * 32 + 16 * (t & 1) + 8 * j, wvec, w2r[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < kStage; k++) {
+        const int idx = tid + k * kThreads;
+        if (idx >= 54 * 16 * 2) break;
+        const int j = idx & 1, o = (idx >> 1) & 15, t = idx >> 5, tap = t >> 1, hh = t & 1;
+        const uint4 v = tc::pack8(w2r[k]);
         const int kz = tap / 9, blk = (tap % 9) * 2 + hh, bo = b_off(o, 8 * j);
         if (kz == 1) {
             *reinterpret_cast<uint4*>(w2 + kW2CBytes + blk * 512 + bo) = v;
@@ -325,8 +337,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (tid < 64) {
         const int o = tid >> 1, j = tid & 1;
         float w[8];
+        load8(A.P + kOW1 + o * 8, wvec, w);
+        if (j) {
 #pragma unroll
-        for (int e = 0; e < 8; e++) w[e] = j ? 0.f : A.P[kOW1 + o * 8 + e];
+            for (int e = 0; e < 8; e++) w[e] = 0.f;
+        }
         *reinterpret_cast<uint4*>(w1 + (o >> 3) * 256 + j * 128 + (o & 7) * 16) = tc::pack8(w);
     }
     // E1 A tiles: rows past the 561 voxels stay zero (the second K half of
@@ -335,6 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int g = i / (kARows - NVOX), r = NVOX + i % (kARows - NVOX);
         *reinterpret_cast<uint4*>(atile + g * kATileBytes + r * 16) = make_uint4(0u, 0u, 0u, 0u);
     }
+    pdl_wait();  // the weights are staged while the kernels of the scale drain
     tc::fence_proxy_async();
     tc::tc_fence_before();
     __syncthreads();
@@ -698,8 +714,7 @@ cudaError_t ae_encode_march(const float* P, const ae::Vol& in, const float* inv_
     S.nitems = (int)(ncol * ((l.nz + S.zc - 1) / S.zc));
     EncArgs a{P, inv_sigma, lat, l, h, take_test_stall(RTM_STALL_ENCODER)};
     const int grid = std::min(nsm, S.nitems);
-    k_encode_march<<<grid, kThreads, kSmem, s>>>(a, map, S, status);
-    return cudaGetLastError();
+    return launch_next(k_encode_march, dim3(grid), dim3(kThreads), kSmem, s, a, map, S, status);
 }
 
 }  // namespace rtm

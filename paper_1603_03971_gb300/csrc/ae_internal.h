@@ -19,6 +19,19 @@ constexpr int kOB4 = 47184;   // b4[1]
 constexpr int kNParams = 47185;
 constexpr float kSlope = 0.1f;  // LeakyReLU
 
+// 8 consecutive float32 weights; vec: p is 16-byte aligned
+__device__ __forceinline__ void load8(const float* __restrict__ p, bool vec, float* w) {
+    if (vec) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+        const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+        w[0] = a.x, w[1] = a.y, w[2] = a.z, w[3] = a.w;
+        w[4] = b.x, w[5] = b.y, w[6] = b.z, w[7] = b.w;
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; e++) w[e] = __ldg(p + e);
+    }
+}
+
 struct Dims3 {
     int nx, ny, nz;
 };
@@ -57,7 +70,8 @@ struct AeTrainBufs {
 }  // namespace ae
 
 cudaError_t ae_gemm_test(const ae::GemmArgs& a, int N, int* status, cudaStream_t s);
-cudaError_t ae_rms(const ae::Vol& in, ae::AeScalars* sc, cudaStream_t s);
+cudaError_t ae_rms(const ae::Vol& in, ae::AeScalars* sc, cudaStream_t s,
+                   float* sigma_out = nullptr);
 // snapshot -> latent; the snapshot's rms goes to sigma_out if given. The
 // z-marching kernel runs where it can, otherwise the GEMM-engine layers through
 // h1. With sumsq_ready, sc->sumsq already holds the
