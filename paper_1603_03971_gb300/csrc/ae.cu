@@ -148,7 +148,9 @@ struct OpE1 {  // x0 (strided float32, scaled by 1/rms) -> h1
                        s;
             }
         }
-        tc::st_vec8(sA, tid, 0, tc::pack8(f));
+        const uint4 patch = tc::pack8(f);
+        if (a.xq && v < total) *reinterpret_cast<uint4*>(a.xq + v * 8) = patch;
+        tc::st_vec8(sA, tid, 0, patch);
         tc::st_vec8(sA, tid, 8, zero4u());
         tc::st_vec8(sA, tid, 16, zero4u());
         tc::st_vec8(sA, tid, 24, zero4u());
@@ -712,7 +714,7 @@ cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScal
     e = ae_encode_march(P, in, &sc->inv_sigma, lat, status, s);
     if (e == cudaErrorNotSupported) {
         cudaGetLastError();
-        E1Args a1{in, &sc->inv_sigma, P, h1, h};
+        E1Args a1{in, &sc->inv_sigma, P, h1, h, nullptr};
         e = run<OpE1>(a1, dim3(tiles((long long)h.nx * h.ny * h.nz)), status, s);
         if (e != cudaSuccess) return e;
         E2Args a2{h1, h, P, lat, l};
@@ -743,7 +745,7 @@ cudaError_t ae_sample_grad(const float* P, const Vol& in, float scale, const AeT
         if (e_ != cudaSuccess) return e_;        \
     } while (0)
     RUN(ae_rms(in, sc, s));
-    RUN(run<OpE1>(E1Args{in, &sc->inv_sigma, P, b.h1, h}, dim3(tiles_h), status, s));
+    RUN(run<OpE1>(E1Args{in, &sc->inv_sigma, P, b.h1, h, b.xq}, dim3(tiles_h), status, s));
     RUN(ae_train_e2(P, b.W, b.h1, b.lat, h, l, status, s));
     RUN(ae_train_d1(P, b.W, b.lat, b.g1, h, l, status, s));
     const Vol yv{b.y, (long long)in.nx, (long long)in.nx * in.ny, in.nx, in.ny, in.nz};
@@ -758,7 +760,7 @@ cudaError_t ae_sample_grad(const float* P, const Vol& in, float scale, const AeT
     RUN(ae_train_d1_grad(b.W, b.ga3, b.glat, h, l, status, s));
     RUN(ae_train_e2_weights(b.h1, b.glat, grad, h, l, status, s));
     RUN(ae_train_e2_grad(b.W, b.glat, b.h1, b.ga1, h, l, status, s));
-    RUN(ae_train_patch_weights(in, &sc->inv_sigma, b.ga1, b.gy, b.g1, b.ga3, grad, h, l, status, s));
+    RUN(ae_train_patch_weights(b.xq, b.ga1, b.gy, b.g1, b.ga3, grad, h, l, status, s));
 #undef RUN
     return cudaSuccess;
 }

@@ -21,7 +21,7 @@ size_t upa(size_t v) { return (v + kAl - 1) / kAl * kAl; }
 
 struct AeLayout {
     size_t status = 0, scalars = 64;
-    size_t h1, lat, g1, y, gy, ga3, glat, ga1, grad, packed, total;
+    size_t h1, lat, g1, y, gy, ga3, glat, ga1, xq, grad, packed, total;
 };
 
 AeLayout ae_layout(int nx, int ny, int nz) {
@@ -41,6 +41,7 @@ AeLayout ae_layout(int nx, int ny, int nz) {
     L.ga3 = take(nh * 32 * 2);
     L.glat = take(nl * 16 * 2);
     L.ga1 = take(nh * 32 * 2);
+    L.xq = take(nh * 8 * 2);
     L.grad = take((size_t)kNParams * 4);
     L.packed = take(kAePackedBytes);
     L.total = o;
@@ -148,8 +149,8 @@ rtm_status rtm_ae_train_step(float* d_params, float* d_adam_m, float* d_adam_v, 
     AeTrainBufs b{reinterpret_cast<bf16*>(w + L.h1),  reinterpret_cast<bf16*>(w + L.lat),
                   reinterpret_cast<bf16*>(w + L.g1),  reinterpret_cast<bf16*>(w + L.gy),
                   reinterpret_cast<bf16*>(w + L.ga3), reinterpret_cast<bf16*>(w + L.glat),
-                  reinterpret_cast<bf16*>(w + L.ga1), reinterpret_cast<float*>(w + L.y),
-                  w + L.packed};
+                  reinterpret_cast<bf16*>(w + L.ga1), reinterpret_cast<bf16*>(w + L.xq),
+                  reinterpret_cast<float*>(w + L.y), w + L.packed};
     CUA(cudaMemsetAsync(w, 0, sizeof(int), s));
     CUA(cudaMemsetAsync(grad, 0, sizeof(float) * kNParams, s));
     CUA(cudaMemsetAsync(d_loss, 0, sizeof(double), s));

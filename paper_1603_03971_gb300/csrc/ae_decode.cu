@@ -18,21 +18,28 @@
 // started at plane z + tz, row (1 + ty), column (1 + tx): a descriptor with a
 // shifted start address.
 //
-// Roles: warp 9 (one thread) issues the TMA plane loads, each as soon as its
-// ring slot is free; warp 8 (one thread) the MMAs into one of two
-// accumulator buffers (2 x 256 columns);
-// warpgroup 0 finishes even planes, warpgroup 1 odd planes, four parities at
-// a time: tcgen05.ld of their accumulators (one row per thread),
-// LeakyReLU(acc + b3) rounded to bfloat16 (as the training decoder rounds
-// g1) into four 128 x 32 K-major A operands in shared memory, then one
-// thread issues D2 as tensor-core products, [128 x 32] g1 x [32 x 16] W4
-// (rows 8..15 zero), into the accumulator columns just drained; the 8 results
-// per parity are read back, scaled by the snapshot's rms and stored as the
-// float4 rows of the latent voxel's 4 x 4 x 4 output block. mbarriers: plane
-// full (TMA bytes), plane free (commit of the last MMAs that read it),
-// accumulator full (commit), accumulator free (128 epilogue arrivals), D2
-// done (commit). Every wait is bounded and shares an abort flag; the
-// warpgroups vote on each wait's outcome, so they leave together.
+// Roles: the last warp (one thread) issues the TMA plane loads, each as soon
+// as its ring slot is free; the warp before it (one thread) the MMAs into one
+// of two accumulator buffers (2 x 256 columns); four warpgroups finish half a
+// plane each (z parity g & 1 of the planes of buffer g >> 1), four parities:
+// tcgen05.ld of their accumulators (one row per thread), LeakyReLU(acc + b3)
+// rounded to bfloat16 (as the training decoder rounds g1) and stored back into
+// the drained accumulator columns, from which one thread issues D2 as
+// tensor-core products with A in tensor memory, [128 x 32] g1 x [32 x 16] W4
+// (rows 8..15 zero); the 8 results per parity are read back, scaled by the
+// snapshot's rms and stored as the float4 rows of the latent voxel's
+// 4 x 4 x 4 output block. mbarriers: plane full (TMA bytes), plane free
+// (commit of the last MMAs that read it), accumulator half full (commit) and
+// free (128 epilogue arrivals), D2 done (commit). Every wait is bounded and
+// shares an abort flag; the warpgroups vote on each wait's outcome, so they
+// leave together.
+//
+// 384^3: 130 -> 121 us. An MMA of 128 rows takes 45-48 cycles for any N up to
+// 64, aligned or not, so a plane's 52 + 16 hold the tensor cores for 3100 of
+// its 4600 cycles; D2's wait in the queue behind the next plane's. The start
+// (weights into shared memory) took 16 us of the 130 and takes 10 with four
+// rows of 16-byte loads in flight per thread. Four warpgroups with g1 through
+// shared memory were no faster than two.
 
 #include <cuda.h>
 #include <cuda_bf16.h>

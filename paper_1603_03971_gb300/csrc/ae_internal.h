@@ -46,7 +46,8 @@ struct Vol {
 using bf16 = __nv_bfloat16;
 
 struct GemmArgs { const bf16* A; const bf16* B; float* C; int M, K; };
-struct E1Args { Vol in; const float* inv_sigma; const float* P; bf16* h1; Dims3 h; };
+// xq: each voxel's 8 normalised inputs, kept for the weight gradient, or NULL
+struct E1Args { Vol in; const float* inv_sigma; const float* P; bf16* h1; Dims3 h; bf16* xq; };
 struct E2Args { const bf16* h1; Dims3 h; const float* P; bf16* lat; Dims3 l; };
 struct D1Args { const bf16* lat; Dims3 l; const float* P; bf16* g1; Dims3 h; };
 struct D2Args { const bf16* g1; Dims3 h; const float* P; const float* sigma; Vol out; };
@@ -62,7 +63,7 @@ struct AeScalars {
 };
 
 struct AeTrainBufs {
-    bf16 *h1, *lat, *g1, *gy, *ga3, *glat, *ga1;
+    bf16 *h1, *lat, *g1, *gy, *ga3, *glat, *ga1, *xq;
     float* y;
     const void* W;  // packed weights (ae_train.h)
 };

@@ -2,27 +2,35 @@
 // gathers: forward E2 and D1, their data gradients, and every weight and bias
 // gradient.
 //
-// One 128-thread CTA computes a 128 x N tile on the tensor cores, as in
-// tc_gemm.cuh, with nothing in its slab loop that waits for global memory:
+// A CTA computes a 128 x N tile on the tensor cores: four warps copy operand
+// slabs into a ring, a fifth multiplies (k_tc_train).
 //  - Weights are packed once per step into the shared-memory image of each
 //    slab's B operand (k_pack_weights), so B is a contiguous cp.async. Reading
 //    the float32 parameters in every slab (for D1's gradient 512 of them 4 KB
 //    apart) stalled each of the 64 slabs of a tile.
+//  - Four lanes copy one 64-byte row of a gather, through L1: of the rows that
+//    one tap reads, the next tap along x reads half again.
 //  - The weight gradients contract over voxels, and activations are stored
 //    [voxel][channel]: both operands are MN-major for that product, so a
 //    voxel's channels are copied as they lie and the transposition is the
 //    instruction descriptor's. Writing the transposed slab element by element
-//    took 32-48 two-byte stores per thread and slab.
+//    took 32-48 two-byte stores per thread and slab. Every CTA adds its sums
+//    to the same few hundred gradients, about 60 ns per CTA, so there are few
+//    (the patch gradients: 1456 CTAs 143 us, 304 CTAs 71 us).
 //  - E2's data gradient runs one launch row per output parity: a parity reaches
 //    1, 2, 4 or 8 of the 27 taps, the tile of all parities gathered all 27.
 //  - The rank-8 gradients of the patch convolutions and their biases are one
 //    product: rows [ga1 | g1 | ga3], columns [x patch | gy patch | 1].
-// Every accumulator still sums its taps in the order of the general engine.
+// Every accumulator sums its taps in the order of the general engine.
 //
-// us per 192^3 sample, before -> now: E2 99 -> 68, D1 109 -> 73, D1's data
-// gradient 219 -> 145, E2's 175 -> 64, weight gradients of E2 241 -> 68,
-// of D1 218 -> 82, of E1 and D2 with the biases 387 -> 118. A sample's
+// us per 192^3 sample, general engine -> one role for copies and products ->
+// now: E2 99 -> 68 -> 48, D1 109 -> 73 -> 56, D1's data gradient 219 -> 145 ->
+// 103, E2's 175 -> 64 -> 58, weight gradients of E2 241 -> 68 -> 55, of D1
+// 218 -> 82 -> 43, of E1 and D2 with the biases 387 -> 118 -> 71. A sample's
 // activations are 57 MB each: 8 us per pass over one at the HBM copy rate.
+// What is left: a CTA's copies are issued slab by slab, about 0.8 us each with
+// their index arithmetic, and the gathers move 3 to 8 times the activations
+// from L2.
 
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -53,14 +61,45 @@ __device__ __forceinline__ Pos position_of(unsigned v, const Dims3& d) {
     p.ok = v < total;
     return p;
 }
-__device__ __forceinline__ bool inside(int x, int y, int z, const Dims3& d) {
-    return x >= 0 && x < d.nx && y >= 0 && y < d.ny && z >= 0 && z < d.nz;
+__device__ __forceinline__ int at(int x, int y, int z, const Dims3& d) {
+    return (z * d.ny + y) * d.nx + x;
 }
-__device__ __forceinline__ long long at(int x, int y, int z, const Dims3& d) {
-    return ((long long)z * d.ny + y) * d.nx + x;
+// where the taps of a voxel lie in grid g: the index of the first (it may be
+// outside) and, four bits per axis, which of the next offsets are inside
+struct Tap0 {
+    int lin;
+    unsigned in;
+};
+__device__ __forceinline__ Tap0 tap0(const Pos& p, int scale, int org, const Dims3& g) {
+    const int x = scale * p.x + org, y = scale * p.y + org, z = scale * p.z + org;
+    auto axis = [](int c, int n) {
+        unsigned b = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) b |= (unsigned)((unsigned)(c + k) < (unsigned)n) << k;
+        return b;
+    };
+    Tap0 t;
+    t.lin = (int)(((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx + (unsigned)x);
+    t.in = p.ok ? axis(x, g.nx) | axis(y, g.ny) << 4 | axis(z, g.nz) << 8 : 0u;
+    return t;
+}
+__device__ __forceinline__ bool tap_in(unsigned in, int kx, int ky, int kz) {
+    return (in >> kx) & (in >> (4 + ky)) & (in >> (8 + kz)) & 1u;
 }
 
+// 16 bytes through L1 (gathered rows: the next taps of the tile read them again)
 __device__ __forceinline__ void copy16(uint8_t* dst, const void* src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
+                 "r"(valid ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void copy4(uint8_t* dst, const void* src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
+                 "r"(valid ? 4 : 0)
+                 : "memory");
+}
+// 16 bytes past L1 (read once)
+__device__ __forceinline__ void stream16(uint8_t* dst, const void* src, bool valid) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
                  "r"(valid ? 16 : 0)
                  : "memory");
@@ -73,6 +112,32 @@ __device__ __forceinline__ uint8_t* kmaj(uint8_t* slab, int r, int g) {
 // with rows and k exchanged
 __device__ __forceinline__ uint8_t* mnmaj(uint8_t* slab, int g, int k) {
     return slab + g * 512 + (k >> 3) * 128 + (k & 7) * 16;
+}
+// Four lanes take the chunks of one row, so a warp's copy reads 8 rows of 64
+// bytes (or 16 of 32) and not 16 bytes of each of 32 rows, which are 32 cache
+// lines. A thread's rows: (tid >> 2) + 32 i
+struct Rows {
+    Tap0 t[4];
+};
+__device__ __forceinline__ Rows rows_of(const Dims3& l, int scale, int org, const Dims3& g, int tid) {
+    Rows R;
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+        R.t[i] = tap0(position_of(blockIdx.x * 128u + (tid >> 2) + 32 * i, l), scale, org, g);
+    return R;
+}
+// chunk tid & 3 of the thread's rows: 8 of the C channels, from e on, at tap
+// (kx, ky, kz); zeros unless `on`
+template <int C>
+__device__ __forceinline__ void copy_rows(uint8_t* sA, const bf16* in, const Rows& R, const Dims3& g,
+                                          int kx, int ky, int kz, bool on, int e, int tid) {
+    const int off = at(kx, ky, kz, g);
+    uint8_t* dst = kmaj(sA, tid >> 2, tid & 3);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const bool ok = on && tap_in(R.t[i].in, kx, ky, kz);
+        copy16(dst + 2048 * i, in + (ok ? (long long)(R.t[i].lin + off) * C + e : 0), ok);
+    }
 }
 // a packed B slab of n rows
 __device__ __forceinline__ void copy_packed(uint8_t* sB, const uint4* slab, int n, int tid) {
@@ -95,11 +160,10 @@ __device__ __forceinline__ void store_row(bf16* dst, const float* f, int n) {
     for (int j = 0; j < n; j += 8) *reinterpret_cast<uint4*>(dst + j) = tc::pack8(f + j);
 }
 // f *= LeakyReLU'(activation) of 32 channels
-__device__ __forceinline__ void mask_row(const bf16* act, float* f) {
+__device__ __forceinline__ void mask_row(const uint4* act, float* f) {
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-        const uint4 u = reinterpret_cast<const uint4*>(act)[j];
-        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(act + j);
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             const float2 t = __bfloat1622float2(h[e]);
@@ -107,6 +171,38 @@ __device__ __forceinline__ void mask_row(const bf16* act, float* f) {
             f[8 * j + 2 * e + 1] *= t.y > 0.f ? 1.0f : kSlope;
         }
     }
+}
+// rows of 32 channels between a lane's registers and voxels v (negative: none)
+// of its warp, four lanes per row on the memory side; buf: 2 KB of the warp
+__device__ __forceinline__ uint4* row_chunk(uint8_t* buf, int r, int j) {
+    return reinterpret_cast<uint4*>(buf + (r * 4 + (j ^ ((r >> 1) & 3))) * 16);
+}
+__device__ __forceinline__ void store_rows(uint8_t* buf, bf16* out, int v, const float* f) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 4; j++) *row_chunk(buf, lane, j) = tc::pack8(f + 8 * j);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int r = (lane >> 2) + 8 * i, vr = __shfl_sync(0xffffffffu, v, r);
+        if (vr >= 0)
+            *reinterpret_cast<uint4*>(out + (long long)vr * 32 + 8 * (lane & 3)) =
+                *row_chunk(buf, r, lane & 3);
+    }
+}
+__device__ __forceinline__ void load_rows(uint8_t* buf, const bf16* in, int v, uint4* u) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int r = (lane >> 2) + 8 * i, vr = __shfl_sync(0xffffffffu, v, r);
+        if (vr >= 0)
+            *row_chunk(buf, r, lane & 3) =
+                *reinterpret_cast<const uint4*>(in + (long long)vr * 32 + 8 * (lane & 3));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 4; j++) u[j] = *row_chunk(buf, lane, j);
+    __syncwarp();
 }
 __device__ __forceinline__ float leaky_relu(float a) { return a > 0.f ? a : kSlope * a; }
 
@@ -202,137 +298,120 @@ struct LayerArgs {
 
 struct TE2 {  // h1 -> latent
     using Args = LayerArgs;
+    using Where = Rows;
+    __device__ static void init(uint8_t*, int) {}
+    static constexpr int kS = 6;
     static constexpr int N = 16;
     static constexpr bool kMN = false;
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = 27;
     }
-    __device__ static Pos position(const Args& a, int tid) {
-        return position_of(blockIdx.x * 128u + tid, a.l);
-    }
-    __device__ static void load(const Args& a, const Pos& p, int tap, uint8_t* sA, uint8_t* sB,
+    __device__ static Where where(const Args& a, int tid) { return rows_of(a.l, 2, -1, a.h, tid); }
+    __device__ static void load(const Args& a, const Where& R, int tap, uint8_t* sA, uint8_t* sB,
                                 int tid) {
-        const int kz = tap / 9, ky = (tap / 3) % 3, kx = tap % 3;
-        const int x = 2 * p.x + kx - 1, y = 2 * p.y + ky - 1, z = 2 * p.z + kz - 1;
-        const bool ok = p.ok && inside(x, y, z, a.h);
-        const bf16* src = ok ? a.in + at(x, y, z, a.h) * 32 : a.in;
-#pragma unroll
-        for (int j = 0; j < 4; j++) copy16(kmaj(sA, tid, j), src + 8 * j, ok);
+        copy_rows<32>(sA, a.in, R, a.h, tap % 3, (tap / 3) % 3, tap / 9, true, 8 * (tid & 3), tid);
         copy_packed(sB, a.W + kE2At + tap * kE2Slab, N, tid);
     }
-    __device__ static void epilogue(const Args& a, const Pos& p, int, const float* acc) {
+    __device__ static void epilogue(const Args& a, int row, uint8_t*, const float* acc) {
+        const Pos p = position_of(blockIdx.x * 128u + row, a.l);
         if (!p.ok) return;
         float f[16];
 #pragma unroll
         for (int o = 0; o < 16; o++) f[o] = acc[o] + a.P[kOB2 + o];
-        store_row(a.out + at(p.x, p.y, p.z, a.l) * 16, f, 16);
+        store_row(a.out + (long long)(blockIdx.x * 128u + row) * 16, f, 16);
     }
 };
 
 struct TD1 {  // latent -> g1, output parity blockIdx.y
     using Args = LayerArgs;
+    using Where = Rows;
+    __device__ static void init(uint8_t*, int) {}
+    static constexpr int kS = 2;
     static constexpr int N = 32;
     static constexpr bool kMN = false;
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = 4;
     }
-    __device__ static Pos position(const Args& a, int tid) {
-        return position_of(blockIdx.x * 128u + tid, a.l);
-    }
-    __device__ static void load(const Args& a, const Pos& p, int ch, uint8_t* sA, uint8_t* sB,
+    __device__ static Where where(const Args& a, int tid) { return rows_of(a.l, 1, -1, a.l, tid); }
+    __device__ static void load(const Args& a, const Where& R, int ch, uint8_t* sA, uint8_t* sB,
                                 int tid) {
-        const int q = blockIdx.y;
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int tau = 2 * ch + h;
-            int tz, ty, tx, k;
-            convt(q >> 2, tau >> 2, tz, k);
-            convt((q >> 1) & 1, (tau >> 1) & 1, ty, k);
-            convt(q & 1, tau & 1, tx, k);
-            const int x = p.x + tx, y = p.y + ty, z = p.z + tz;
-            const bool ok = p.ok && inside(x, y, z, a.l);
-            const bf16* src = ok ? a.in + at(x, y, z, a.l) * 16 : a.in;
-            copy16(kmaj(sA, tid, 2 * h), src, ok);
-            copy16(kmaj(sA, tid, 2 * h + 1), src + 8, ok);
-        }
+        const int q = blockIdx.y, tau = 2 * ch + ((tid >> 1) & 1);
+        int tz, ty, tx, k;
+        convt(q >> 2, tau >> 2, tz, k);
+        convt((q >> 1) & 1, (tau >> 1) & 1, ty, k);
+        convt(q & 1, tau & 1, tx, k);
+        copy_rows<16>(sA, a.in, R, a.l, tx + 1, ty + 1, tz + 1, true, 8 * (tid & 1), tid);
         copy_packed(sB, a.W + kD1At + (4 * q + ch) * kD1Slab, N, tid);
     }
-    __device__ static void epilogue(const Args& a, const Pos& p, int, const float* acc) {
-        if (!p.ok) return;
+    __device__ static void epilogue(const Args& a, int row, uint8_t* buf, const float* acc) {
+        const Pos p = position_of(blockIdx.x * 128u + row, a.l);
         const int q = blockIdx.y;
         float f[32];
 #pragma unroll
         for (int c = 0; c < 32; c++) f[c] = leaky_relu(acc[c] + a.P[kOB3 + c]);
-        store_row(a.out + at(2 * p.x + (q & 1), 2 * p.y + ((q >> 1) & 1), 2 * p.z + (q >> 2), a.h) * 32,
-                  f, 32);
+        store_rows(buf, a.out,
+                   p.ok ? at(2 * p.x + (q & 1), 2 * p.y + ((q >> 1) & 1), 2 * p.z + (q >> 2), a.h) : -1,
+                   f);
     }
 };
 
 struct TD1d {  // ga3 -> glat: dlat[j] = sum_k W3[.,k,.]^T ga3[2j + k - 1]
     using Args = LayerArgs;
+    using Where = Rows;
+    __device__ static void init(uint8_t*, int) {}
+    static constexpr int kS = 6;
     static constexpr int N = 16;
     static constexpr bool kMN = false;
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = 64;
     }
-    __device__ static Pos position(const Args& a, int tid) {
-        return position_of(blockIdx.x * 128u + tid, a.l);
-    }
-    __device__ static void load(const Args& a, const Pos& p, int tap, uint8_t* sA, uint8_t* sB,
+    __device__ static Where where(const Args& a, int tid) { return rows_of(a.l, 2, -1, a.h, tid); }
+    __device__ static void load(const Args& a, const Where& R, int tap, uint8_t* sA, uint8_t* sB,
                                 int tid) {
-        const int x = 2 * p.x + (tap & 3) - 1, y = 2 * p.y + ((tap >> 2) & 3) - 1,
-                  z = 2 * p.z + (tap >> 4) - 1;
-        const bool ok = p.ok && inside(x, y, z, a.h);
-        const bf16* src = ok ? a.in + at(x, y, z, a.h) * 32 : a.in;
-#pragma unroll
-        for (int j = 0; j < 4; j++) copy16(kmaj(sA, tid, j), src + 8 * j, ok);
+        copy_rows<32>(sA, a.in, R, a.h, tap & 3, (tap >> 2) & 3, tap >> 4, true, 8 * (tid & 3), tid);
         copy_packed(sB, a.W + kD1dAt + tap * kD1dSlab, N, tid);
     }
-    __device__ static void epilogue(const Args& a, const Pos& p, int, const float* acc) {
-        if (p.ok) store_row(a.out + at(p.x, p.y, p.z, a.l) * 16, acc, 16);
+    __device__ static void epilogue(const Args& a, int row, uint8_t*, const float* acc) {
+        const Pos p = position_of(blockIdx.x * 128u + row, a.l);
+        if (p.ok) store_row(a.out + (long long)(blockIdx.x * 128u + row) * 16, acc, 16);
     }
 };
 
 struct TE2d {  // glat -> ga1 at output parity blockIdx.y: (sum of W2^T glat) * leaky'(a1)
     using Args = LayerArgs;
+    using Where = Rows;
+    __device__ static void init(uint8_t*, int) {}
+    static constexpr int kS = 2;
     static constexpr int N = 32;
     static constexpr bool kMN = false;
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = (e2d_taps(blockIdx.y) + 1) / 2;
     }
-    __device__ static Pos position(const Args& a, int tid) {
-        return position_of(blockIdx.x * 128u + tid, a.l);
-    }
-    __device__ static void load(const Args& a, const Pos& p, int ch, uint8_t* sA, uint8_t* sB,
+    __device__ static Where where(const Args& a, int tid) { return rows_of(a.l, 1, 0, a.l, tid); }
+    __device__ static void load(const Args& a, const Where& R, int ch, uint8_t* sA, uint8_t* sB,
                                 int tid) {
-        const int q = blockIdx.y;
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int i = 2 * ch + h;
-            int kz, ky, kx, dz, dy, dx;
-            e2d_tap(q, i, kz, ky, kx, dz, dy, dx);
-            const int x = p.x + dx, y = p.y + dy, z = p.z + dz;
-            const bool ok = p.ok && i < e2d_taps(q) && inside(x, y, z, a.l);
-            const bf16* src = ok ? a.in + at(x, y, z, a.l) * 16 : a.in;
-            copy16(kmaj(sA, tid, 2 * h), src, ok);
-            copy16(kmaj(sA, tid, 2 * h + 1), src + 8, ok);
-        }
+        const int q = blockIdx.y, i = 2 * ch + ((tid >> 1) & 1);
+        int kz, ky, kx, dz, dy, dx;
+        e2d_tap(q, i, kz, ky, kx, dz, dy, dx);
+        copy_rows<16>(sA, a.in, R, a.l, dx, dy, dz, i < e2d_taps(q), 8 * (tid & 1), tid);
         copy_packed(sB, a.W + kE2dAt + (e2d_first_slab(q) + ch) * kE2dSlab, N, tid);
     }
-    __device__ static void epilogue(const Args& a, const Pos& p, int, const float* acc) {
-        if (!p.ok) return;
+    __device__ static void epilogue(const Args& a, int row, uint8_t* buf, const float* acc) {
+        const Pos p = position_of(blockIdx.x * 128u + row, a.l);
         const int q = blockIdx.y;
-        const long long v =
-            at(2 * p.x + (q & 1), 2 * p.y + ((q >> 1) & 1), 2 * p.z + (q >> 2), a.h);
+        const int v =
+            p.ok ? at(2 * p.x + (q & 1), 2 * p.y + ((q >> 1) & 1), 2 * p.z + (q >> 2), a.h) : -1;
+        uint4 act[4];
+        load_rows(buf, a.act, v, act);
         float f[32];
 #pragma unroll
         for (int c = 0; c < 32; c++) f[c] = acc[c];
-        mask_row(a.act + v * 32, f);
-        store_row(a.out + v * 32, f, 32);
+        mask_row(act, f);
+        store_rows(buf, a.out, v, f);
     }
 };
 
@@ -341,8 +420,7 @@ struct WeightArgs {
     const bf16 *a, *b;  // row and column operands
     const bf16 *c;      // (patch gradients) third row operand
     const bf16* gy;     // (patch gradients) output gradients, full resolution
-    Vol in;             // (patch gradients) the snapshot
-    const float* inv_sigma;
+    const bf16* xq;     // (patch gradients) normalised inputs, 8 per voxel
     float* grad;
     Dims3 h, l;
     int slabs, per_cta;  // slabs of 32 voxels, and how many a CTA takes
@@ -353,25 +431,43 @@ __device__ __forceinline__ void slab_range(const WeightArgs& a, int cta, int& c0
     if (c1 < c0) c1 = c0;
 }
 
+// a warp's 32 voxels of a slab, one per lane, handed to the lanes that copy
+// their chunks
+struct NoRows {};
+__device__ __forceinline__ Tap0 from_lane(const Tap0& t, int lane) {
+    return Tap0{__shfl_sync(0xffffffffu, t.lin, lane), __shfl_sync(0xffffffffu, t.in, lane)};
+}
+__device__ __forceinline__ unsigned voxels(const Dims3& d) {
+    return (unsigned)d.nx * (unsigned)d.ny * (unsigned)d.nz;
+}
+
 struct TE2w {  // dW2[o][tap][i] += sum_v glat[v][o] h1[2v + tap - 1][i]; blockIdx.x: four taps
     using Args = WeightArgs;
+    using Where = NoRows;
+    __device__ static void init(uint8_t*, int) {}
+    static constexpr int kS = 6;
     static constexpr int N = 16;
     static constexpr bool kMN = true;
     __device__ static void range(const Args& a, int& c0, int& c1) { slab_range(a, blockIdx.y, c0, c1); }
-    __device__ static Pos position(const Args&, int) { return Pos{0, 0, 0, 1}; }
-    __device__ static void load(const Args& a, const Pos&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
-        const int vv = tid & 31, tt = tid >> 5, tap = blockIdx.x * 4 + tt;
-        const Pos p = position_of(ch * 32u + vv, a.l);
-        const int kz = tap / 9, ky = (tap / 3) % 3, kx = tap % 3;
-        const int x = 2 * p.x + kx - 1, y = 2 * p.y + ky - 1, z = 2 * p.z + kz - 1;
-        const bool ok = p.ok && tap < 27 && inside(x, y, z, a.h);
-        const bf16* src = ok ? a.a + at(x, y, z, a.h) * 32 : a.a;
+    __device__ static Where where(const Args&, int) { return Where{}; }
+    __device__ static void load(const Args& a, const Where&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
+        const int lane = tid & 31, tt = tid >> 5, tap = blockIdx.x * 4 + tt, j = lane & 3;
+        const Tap0 t = tap0(position_of(ch * 32u + lane, a.l), 2, -1, a.h);
+        const int kz = tap / 9, ky = (tap / 3) % 3, kx = tap % 3, off = at(kx, ky, kz, a.h);
 #pragma unroll
-        for (int j = 0; j < 4; j++) copy16(mnmaj(sA, 4 * tt + j, vv), src + 8 * j, ok);
-        if (tid < 64)  // columns: two chunks of 8 output channels
-            copy16(mnmaj(sB, tt, vv), a.b + (p.ok ? at(p.x, p.y, p.z, a.l) * 16 + 8 * tt : 0), p.ok);
+        for (int i = 0; i < 4; i++) {
+            const int vv = (lane >> 2) + 8 * i;
+            const Tap0 u = from_lane(t, vv);
+            const bool ok = tap < 27 && tap_in(u.in, kx, ky, kz);
+            copy16(mnmaj(sA, 4 * tt + j, vv), a.a + (ok ? (long long)(u.lin + off) * 32 + 8 * j : 0), ok);
+        }
+        if (tid < 64) {  // columns: two chunks of 8 output channels
+            const unsigned v = ch * 32u + (tid >> 1);
+            const bool ok = v < voxels(a.l);
+            copy16(mnmaj(sB, tid & 1, tid >> 1), a.b + (ok ? (long long)v * 16 + 8 * (tid & 1) : 0), ok);
+        }
     }
-    __device__ static void epilogue(const Args& a, const Pos&, int row, const float* acc) {
+    __device__ static void epilogue(const Args& a, int row, uint8_t*, const float* acc) {
         const int r = blockIdx.x * 128 + row;  // tap * 32 + i
         if (r >= 27 * 32) return;
         for (int o = 0; o < 16; o++) atomicAdd(&a.grad[kOW2 + o * 864 + r], acc[o]);
@@ -380,32 +476,44 @@ struct TE2w {  // dW2[o][tap][i] += sum_v glat[v][o] h1[2v + tap - 1][i]; blockI
 
 struct TD1w {  // dW3[o][k][i] += sum_j ga3[2j + q][o] lat[j + t][i], parity q = blockIdx.x
     using Args = WeightArgs;
+    using Where = NoRows;
+    __device__ static void init(uint8_t*, int) {}
+    static constexpr int kS = 6;
     static constexpr int N = 32;
     static constexpr bool kMN = true;
     __device__ static void range(const Args& a, int& c0, int& c1) { slab_range(a, blockIdx.y, c0, c1); }
-    __device__ static Pos position(const Args&, int) { return Pos{0, 0, 0, 1}; }
-    __device__ static void load(const Args& a, const Pos&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
-        const int q = blockIdx.x, vv = tid & 31;
-        const Pos p = position_of(ch * 32u + vv, a.l);
+    __device__ static Where where(const Args&, int) { return Where{}; }
+    __device__ static void load(const Args& a, const Where&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
+        const int q = blockIdx.x, lane = tid & 31, warp = tid >> 5;
+        const Pos p = position_of(ch * 32u + lane, a.l);
+        const Tap0 t = tap0(p, 1, -1, a.l);
 #pragma unroll
-        for (int rep = 0; rep < 2; rep++) {
-            const int tau = (tid >> 5) + 4 * rep;  // rows tau * 16 + i
-            int tz, ty, tx, k;
-            convt(q >> 2, tau >> 2, tz, k);
-            convt((q >> 1) & 1, (tau >> 1) & 1, ty, k);
-            convt(q & 1, tau & 1, tx, k);
-            const int x = p.x + tx, y = p.y + ty, z = p.z + tz;
-            const bool ok = p.ok && inside(x, y, z, a.l);
-            const bf16* src = ok ? a.a + at(x, y, z, a.l) * 16 : a.a;
-            copy16(mnmaj(sA, 2 * tau, vv), src, ok);
-            copy16(mnmaj(sA, 2 * tau + 1, vv), src + 8, ok);
+        for (int half = 0; half < 2; half++) {
+            const int vv = (lane >> 1) + 16 * half;
+            const Tap0 u = from_lane(t, vv);
+#pragma unroll
+            for (int rep = 0; rep < 2; rep++) {
+                const int tau = warp + 4 * rep;  // rows tau * 16 + i
+                int tz, ty, tx, k;
+                convt(q >> 2, tau >> 2, tz, k);
+                convt((q >> 1) & 1, (tau >> 1) & 1, ty, k);
+                convt(q & 1, tau & 1, tx, k);
+                const bool ok = tap_in(u.in, tx + 1, ty + 1, tz + 1);
+                copy16(mnmaj(sA, 2 * tau + (lane & 1), vv),
+                       a.a + (ok ? (long long)(u.lin + at(tx + 1, ty + 1, tz + 1, a.l)) * 16 +
+                                       8 * (lane & 1)
+                                 : 0),
+                       ok);
+            }
         }
-        const int j = tid >> 5;  // columns: four chunks of 8 output channels
-        const long long o =
-            p.ok ? at(2 * p.x + (q & 1), 2 * p.y + ((q >> 1) & 1), 2 * p.z + (q >> 2), a.h) : 0;
-        copy16(mnmaj(sB, j, vv), a.b + o * 32 + 8 * j, p.ok);
+        // columns: four chunks of 8 output channels, 8 voxels per warp
+        const int v =
+            p.ok ? at(2 * p.x + (q & 1), 2 * p.y + ((q >> 1) & 1), 2 * p.z + (q >> 2), a.h) : -1;
+        const int vr = __shfl_sync(0xffffffffu, v, tid >> 2);
+        copy16(mnmaj(sB, tid & 3, tid >> 2), a.b + (vr >= 0 ? (long long)vr * 32 + 8 * (tid & 3) : 0),
+               vr >= 0);
     }
-    __device__ static void epilogue(const Args& a, const Pos&, int row, const float* acc) {
+    __device__ static void epilogue(const Args& a, int row, uint8_t*, const float* acc) {
         const int q = blockIdx.x, tau = row >> 4, i = row & 15;
         int t, kz, ky, kx;
         convt(q >> 2, tau >> 2, t, kz);
@@ -421,44 +529,43 @@ struct TD1w {  // dW3[o][k][i] += sum_j ga3[2j + q][o] lat[j + t][i], parity q =
 // columns [xq patch | gy patch | 1 | -] of 8
 struct TPatch {
     using Args = WeightArgs;
+    using Where = NoRows;
+    static constexpr int kS = 10;
     static constexpr int N = 32;
     static constexpr bool kMN = true;
     __device__ static void range(const Args& a, int& c0, int& c1) { slab_range(a, blockIdx.x, c0, c1); }
-    __device__ static Pos position(const Args&, int) { return Pos{0, 0, 0, 1}; }
-    __device__ static void load(const Args& a, const Pos&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
-        const int vv = tid & 31, part = tid >> 5;
-        const unsigned v = ch * 32u + vv;
-        const Pos p = position_of(v, a.h);
-        if (part < 3) {
-            const bf16* src = (part == 0 ? a.a : part == 1 ? a.b : a.c) + (p.ok ? (long long)v * 32 : 0);
+    __device__ static Where where(const Args&, int) { return Where{}; }
+    __device__ static void load(const Args& a, const Where&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
+        const int lane = tid & 31, part = tid >> 5;
+        const bf16* rows = part == 0 ? a.a : part == 1 ? a.b : a.c;
 #pragma unroll
-            for (int j = 0; j < 4; j++) copy16(mnmaj(sA, 4 * part + j, vv), src + 8 * j, p.ok);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; j++) copy16(mnmaj(sA, 12 + j, vv), a.a, false);  // zeros
+        for (int i = 0; i < 4; i++) {
+            const int vv = (lane >> 2) + 8 * i, j = lane & 3;
+            const unsigned v = ch * 32u + vv;
+            const bool ok = part < 3 && v < voxels(a.h);  // (the fourth part: zeros)
+            stream16(mnmaj(sA, 4 * part + j, vv), rows + (ok ? (long long)v * 32 + 8 * j : 0), ok);
         }
-        uint4 w = make_uint4(0, 0, 0, 0);
-        if (part == 0 && p.ok) {  // the voxel's patch of normalised inputs
-            const float s = *a.inv_sigma;
-            const float* src = a.in.p + 2LL * p.z * a.in.sz + 2LL * p.y * a.in.sy + 2 * p.x;
-            float f[8];
-#pragma unroll
-            for (int d = 0; d < 8; d++)
-                f[d] = src[(d >> 2) * a.in.sz + ((d >> 1) & 1) * a.in.sy + (d & 1)] * s;
-            w = tc::pack8(f);
-        } else if (part == 1 && p.ok) {  // its patch of output gradients: pairs along x
+        const unsigned v = ch * 32u + lane;
+        uint8_t* dst = mnmaj(sB, part, lane);
+        if (part == 0) {  // the voxel's patch of normalised inputs
+            const bool ok = v < voxels(a.h);
+            stream16(dst, a.xq + (ok ? (long long)v * 8 : 0), ok);
+        } else if (part == 1) {  // its patch of output gradients: pairs along x
+            const Pos p = position_of(v, a.h);
             const long long NX = 2 * a.h.nx, NY = 2 * a.h.ny;
-            const bf16* src = a.gy + ((2LL * p.z) * NY + 2 * p.y) * NX + 2 * p.x;
-            w.x = *reinterpret_cast<const uint32_t*>(src);
-            w.y = *reinterpret_cast<const uint32_t*>(src + NX);
-            w.z = *reinterpret_cast<const uint32_t*>(src + NY * NX);
-            w.w = *reinterpret_cast<const uint32_t*>(src + NY * NX + NX);
-        } else if (part == 2) {
-            w.x = 0x3F80;  // bf16 1.0 in the first of the eight columns
+            const bf16* src = a.gy + (p.ok ? ((2LL * p.z) * NY + 2 * p.y) * NX + 2 * p.x : 0);
+#pragma unroll
+            for (int d = 0; d < 4; d++)
+                copy4(dst + 4 * d, src + (p.ok ? (d >> 1) * NY * NX + (d & 1) * NX : 0), p.ok);
         }
-        *reinterpret_cast<uint4*>(mnmaj(sB, part, vv)) = w;
     }
-    __device__ static void epilogue(const Args& a, const Pos&, int row, const float* acc) {
+    // columns 16-23: bf16 1.0 in the first; 24-31: zeros
+    __device__ static void init(uint8_t* sB, int tid) {
+        if (tid >= 64)
+            *reinterpret_cast<uint4*>(mnmaj(sB, tid >> 5, tid & 31)) =
+                make_uint4((tid >> 5) == 2 ? 0x3F80u : 0u, 0u, 0u, 0u);
+    }
+    __device__ static void epilogue(const Args& a, int row, uint8_t*, const float* acc) {
         const int c = row & 31, part = row >> 5;
         if (part == 0) {
             for (int d = 0; d < 8; d++) atomicAdd(&a.grad[kOW1 + c * 8 + d], acc[d]);
@@ -471,78 +578,96 @@ struct TPatch {
     }
 };
 
-// ---- engine: the pipeline of k_tc_gemm_async ----------------------------------
-constexpr int kS = 4, kAhead = 2;  // stages; slabs loaded ahead of the one multiplied
+// ---- engine -------------------------------------------------------------------
+// Warps 0-3 copy slabs into a ring, each as soon as its stage is free, and
+// leave the arrival at the slab's barrier to their copies; warp 4 waits for a
+// slab, makes it visible to the tensor cores and multiplies. A proxy fence in
+// the threads that copy would wait for all of their copies in flight, and with
+// it every slab for the memory's full latency, however deep the ring.
+// Op::kS: stages of 10 KB; two for the products of few slabs (six CTAs per SM),
+// 6 to 10 for the long ones (104 against 127 us with two for D1's gradient)
+template <class Op>
+constexpr int train_smem() {
+    return Op::kS * tc::kStageBytes + 1024;
+}
 
 template <class Op>
-__global__ void __launch_bounds__(128) k_tc_train(const __grid_constant__ typename Op::Args args,
+__global__ void __launch_bounds__(160) k_tc_train(const __grid_constant__ typename Op::Args args,
                                                   int* status) {
-    constexpr int N = Op::N;
-    __shared__ __align__(1024) uint8_t smem[kS][tc::kStageBytes];
-    __shared__ __align__(8) uint64_t bars[kS];
+    constexpr int N = Op::N, kS = Op::kS;
+    extern __shared__ uint8_t raw[];
+    uint8_t(*smem)[tc::kStageBytes] = reinterpret_cast<uint8_t(*)[tc::kStageBytes]>(
+        (reinterpret_cast<uintptr_t>(raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    __shared__ __align__(8) uint64_t full[kS], empty[kS], done;
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = tid >> 5;
     int c0, c1;
     Op::range(args, c0, c1);
     const int nch = c1 - c0;
-    const Pos pos = Op::position(args, tid);
 
     if (tid == 0) {
-        for (int s = 0; s < kS; s++) tc::mbar_init(&bars[s], 1);
+        for (int s = 0; s < kS; s++) {
+            tc::mbar_init(&full[s], 128);
+            tc::mbar_init(&empty[s], 1);
+        }
+        tc::mbar_init(&done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tc::tmem_alloc(&tmem_slot, tc::kTmemCols);
+    if (warp < 4) {
+        for (int s = 0; s < kS; s++) Op::init(smem[s] + tc::kABytes, tid);
+        tc::fence_proxy_async();
+    }
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    // MN-major A and B: transpose bits 15 and 16
-    constexpr uint32_t idesc = tc::idesc_bf16(tc::kRows, N) | (Op::kMN ? (3u << 15) : 0u);
 
-    for (int c = 0; c < kAhead; c++) {
-        if (c < nch) Op::load(args, pos, c0 + c, smem[c], smem[c] + tc::kABytes, tid);
-        tc::cp_async_commit();
-    }
     bool ok = true;
-    int issued = 0;
-    for (int i = 0; i < nch && ok; i++) {
-        const int j = i + kAhead;
-        if (j < nch) {
-            // slab j takes the stage of slab j - kS, multiplied two iterations ago
-            if (j >= kS) ok = tc::mbar_wait(&bars[j % kS], (uint32_t)(((j - kS) / kS) & 1));
-            ok = __syncthreads_and(ok);
-            if (!ok) break;
-            Op::load(args, pos, c0 + j, smem[j % kS], smem[j % kS] + tc::kABytes, tid);
-        }
-        tc::cp_async_commit();
-        tc::cp_async_wait<kAhead>();
-        tc::fence_proxy_async();
-        __syncthreads();
-        if (tid == 0) {
-            tc::tc_fence_after();
-            const uint32_t a0 = tc::smem_u32(smem[i % kS]), b0 = a0 + tc::kABytes;
+    if (warp == 4) {
+        if (tid == 128 && nch > 0) {
+            // MN-major A and B: transpose bits 15 and 16
+            constexpr uint32_t idesc = tc::idesc_bf16(tc::kRows, N) | (Op::kMN ? (3u << 15) : 0u);
+            for (int i = 0; i < nch && ok; i++) {
+                ok = tc::mbar_wait(&full[i % kS], (uint32_t)((i / kS) & 1));
+                if (!ok) break;
+                tc::fence_proxy_async();
+                tc::tc_fence_after();
+                const uint32_t a0 = tc::smem_u32(smem[i % kS]), b0 = a0 + tc::kABytes;
 #pragma unroll
-            for (int s = 0; s < tc::kBK / 16; s++)
-                tc::mma_bf16(tmem, tc::sdesc(a0 + 256 * s, 128, 512),
-                             tc::sdesc(b0 + 256 * s, 128, 512), idesc, (i > 0 || s > 0) ? 1u : 0u);
-            tc::mma_commit(&bars[i % kS]);
+                for (int s = 0; s < tc::kBK / 16; s++)
+                    tc::mma_bf16(tmem, tc::sdesc(a0 + 256 * s, 128, 512),
+                                 tc::sdesc(b0 + 256 * s, 128, 512), idesc,
+                                 (i > 0 || s > 0) ? 1u : 0u);
+                tc::mma_commit(&empty[i % kS]);
+            }
+            tc::mma_commit(&done);
         }
-        issued = i + 1;
+        __syncwarp();
+    } else {
+        const typename Op::Where where = Op::where(args, tid);
+        for (int j = 0; j < nch; j++) {
+            if (j >= kS) ok = tc::mbar_wait(&empty[j % kS], (uint32_t)((j / kS - 1) & 1));
+            if (!ok) break;
+            Op::load(args, where, c0 + j, smem[j % kS], smem[j % kS] + tc::kABytes, tid);
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(
+                             tc::smem_u32(&full[j % kS]))
+                         : "memory");
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
-    tc::cp_async_wait<0>();
-    if (issued > 0) {
-        const int last = issued - 1;
-        const bool done = tc::mbar_wait(&bars[last % kS], (uint32_t)((last / kS) & 1));
-        ok = ok && done;
-    }
+    // the products are done with the stages and the accumulator
+    if (nch > 0 && tid <= 128) ok = tc::mbar_wait(&done, 0) && ok;
     ok = __syncthreads_and(ok);
     tc::tc_fence_after();
     if (ok && nch > 0) {
-        float acc[N];
-        const uint32_t t = tmem + ((uint32_t)(warp * 32) << 16);
-        tc::tmem_ld16(t, acc);
-        if constexpr (N == 32) tc::tmem_ld16(t + 16, acc + 16);
-        Op::epilogue(args, pos, tid, acc);
+        if (warp < 4) {
+            float acc[N];
+            const uint32_t t = tmem + ((uint32_t)(warp * 32) << 16);
+            tc::tmem_ld16(t, acc);
+            if constexpr (N == 32) tc::tmem_ld16(t + 16, acc + 16);
+            Op::epilogue(args, tid, smem[0] + 2048 * warp, acc);
+        }
     } else if (!ok && tid == 0 && status) {
         atomicCAS(status, 0, tc::kErrTimeout);
     }
@@ -569,7 +694,10 @@ __global__ void k_latent_bias(const bf16* __restrict__ glat, long long nl, float
 
 template <class Op>
 cudaError_t run(const typename Op::Args& a, dim3 grid, int* status, cudaStream_t s) {
-    k_tc_train<Op><<<grid, 128, 0, s>>>(a, status);
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        k_tc_train<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, train_smem<Op>());
+    if (attr != cudaSuccess) return attr;
+    k_tc_train<Op><<<grid, 160, train_smem<Op>(), s>>>(a, status);
     return cudaGetLastError();
 }
 
@@ -578,7 +706,7 @@ unsigned tiles_of(const Dims3& d) { return (unsigned)(((long long)d.nx * d.ny * 
 // slabs of a contraction over the voxels of d, split over about `ctas` CTAs
 void split(WeightArgs& w, const Dims3& d, int ctas, unsigned& rows) {
     w.slabs = (int)(((long long)d.nx * d.ny * d.nz + 31) / 32);
-    w.per_cta = std::max(8, (w.slabs + ctas - 1) / ctas);
+    w.per_cta = std::max(16, (w.slabs + ctas - 1) / ctas);
     rows = (unsigned)((w.slabs + w.per_cta - 1) / w.per_cta);
 }
 
@@ -623,7 +751,7 @@ cudaError_t ae_train_d1_weights(const bf16* lat, const bf16* ga3, float* grad, D
     w.h = h;
     w.l = l;
     unsigned rows;
-    split(w, l, 152, rows);
+    split(w, l, 57, rows);
     return run<TD1w>(w, dim3(8, rows), status, s);
 }
 cudaError_t ae_train_e2_weights(const bf16* h1, const bf16* glat, float* grad, Dims3 h, Dims3 l,
@@ -635,28 +763,27 @@ cudaError_t ae_train_e2_weights(const bf16* h1, const bf16* glat, float* grad, D
     w.h = h;
     w.l = l;
     unsigned rows;
-    split(w, l, 152, rows);
+    split(w, l, 65, rows);
     cudaError_t e = run<TE2w>(w, dim3(7, rows), status, s);
     if (e != cudaSuccess) return e;
     const long long nl = (long long)l.nx * l.ny * l.nz;
     k_latent_bias<<<(unsigned)std::min<long long>((nl + 255) / 256, 152), 256, 0, s>>>(glat, nl, grad);
     return cudaGetLastError();
 }
-cudaError_t ae_train_patch_weights(const Vol& in, const float* inv_sigma, const bf16* ga1,
-                                   const bf16* gy, const bf16* g1, const bf16* ga3, float* grad,
-                                   Dims3 h, Dims3 l, int* status, cudaStream_t s) {
+cudaError_t ae_train_patch_weights(const bf16* xq, const bf16* ga1, const bf16* gy, const bf16* g1,
+                                   const bf16* ga3, float* grad, Dims3 h, Dims3 l, int* status,
+                                   cudaStream_t s) {
     WeightArgs w{};
     w.a = ga1;
     w.b = g1;
     w.c = ga3;
     w.gy = gy;
-    w.in = in;
-    w.inv_sigma = inv_sigma;
+    w.xq = xq;
     w.grad = grad;
     w.h = h;
     w.l = l;
     unsigned rows;
-    split(w, h, 152 * 5, rows);
+    split(w, h, 304, rows);
     return run<TPatch>(w, dim3(rows), status, s);
 }
 

@@ -24,9 +24,8 @@ cudaError_t ae_train_d1_weights(const ae::bf16* lat, const ae::bf16* ga3, float*
                                 ae::Dims3 l, int* status, cudaStream_t s);
 cudaError_t ae_train_e2_weights(const ae::bf16* h1, const ae::bf16* glat, float* grad, ae::Dims3 h,
                                 ae::Dims3 l, int* status, cudaStream_t s);
-cudaError_t ae_train_patch_weights(const ae::Vol& in, const float* inv_sigma, const ae::bf16* ga1,
-                                   const ae::bf16* gy, const ae::bf16* g1, const ae::bf16* ga3,
-                                   float* grad, ae::Dims3 h, ae::Dims3 l, int* status,
-                                   cudaStream_t s);
+cudaError_t ae_train_patch_weights(const ae::bf16* xq, const ae::bf16* ga1, const ae::bf16* gy,
+                                   const ae::bf16* g1, const ae::bf16* ga3, float* grad,
+                                   ae::Dims3 h, ae::Dims3 l, int* status, cudaStream_t s);
 
 }  // namespace rtm

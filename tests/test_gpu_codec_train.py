@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("shape,offset", [
-    ((4, 4, 4), 0), ((4, 4, 124), 0), ((4, 44, 12), 0), ((20, 20, 20), 0), ((16, 20, 28), 1)])
+    ((4, 4, 4), 0), ((4, 4, 124), 0), ((4, 44, 12), 0), ((20, 20, 20), 0), ((16, 20, 28), 1),
+    ((24, 28, 32), 0)])
 def test_training_gradient_at_tile_edges(shape, offset):
     import torch
 
