@@ -557,9 +557,12 @@ rtm_status rtm_forward_decomposed(const rtm_params *p, int32_t px, int32_t py, c
 
 /* Stencil tuning: z extent of the slab one thread block marches through
  * (0 = automatic) and the plane-load path and tile (0 = automatic: TMA
- * where the driver provides tensor maps; 1 = 16-byte vector loads through
- * registers; 2 = TMA bulk tensor copies into shared-memory rings, 16-row
- * tiles of 256 threads; 3 = the same with 8-row tiles of 128 threads and
+ * where the driver provides tensor maps, with the tile of 3 at radius 4 and
+ * of 2 at radius 8; on grids of one brick per SM, where the slab height is
+ * automatic too, many steps per cooperative launch; 1 = 16-byte vector loads
+ * through registers; 2 = TMA bulk tensor copies into shared-memory rings,
+ * 16-row tiles, at radius 4 of 256 threads, at radius 8 of 128 threads with
+ * two rows each; 3 = the same with 8-row tiles of 128 threads and
  * 4-point vectors at both radii, five blocks per SM at radius 4, four at
  * radius 8). Applies to later
  * calls on every thread, to every kernel mode on the padded grid (the
@@ -598,7 +601,8 @@ rtm_status rtm_set_tuning_mode(int32_t radius, int32_t mode, int32_t zchunk);
 rtm_status rtm_set_test_stall(int32_t kernel, int32_t plane);
 
 /* Enable (1) or disable (0) per-launch CUDA-event timing of the stencil
- * kernels. While enabled, each API call synchronises its stream on return. */
+ * kernels. While enabled, each API call synchronises its stream on return
+ * and every step is a launch of its own. */
 rtm_status rtm_set_timing(int32_t enable);
 rtm_status rtm_stats_get(rtm_stats *out);
 rtm_status rtm_stats_reset(void);

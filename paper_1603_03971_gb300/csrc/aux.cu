@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "band.cuh"
+#include "cells.cuh"
 #include "pdl.cuh"
 #include "rtm_internal.h"
 
@@ -55,38 +56,42 @@ __global__ void k_wavelet(int nt, double dt, double f0, double t0, float* w) {
 
 // c = v^2 dt^2 on the padded grid (edge padding); max v^2 and validity over
 // the model cells
+// *bits = max(*bits, v) for a non-negative v of every thread of a block of at
+// most 1024. Floats of one sign compare as unsigned. Same-address atomics are served
+// one by one (one per warp of 19456: most of the 56 us of a 10 M cell model),
+// so a block sends one, and only if it would change the value
+__device__ __forceinline__ void block_max(float v, unsigned int* bits) {
+    __shared__ float part[32];
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = threadIdx.x < blockDim.x >> 5 ? part[threadIdx.x] : 0.0f;
+        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if (threadIdx.x == 0 && __float_as_uint(v) > *reinterpret_cast<volatile unsigned int*>(bits))
+            atomicMax(bits, __float_as_uint(v));
+    }
+}
+
 __global__ void k_model_prep(Geometry G, const float* __restrict__ vel, int squared, float dt2,
                              float* __restrict__ c, unsigned int* vmax_bits, int* bad) {
-    const long long N = (long long)G.NX * G.NY * G.NZ;
-    const long long stride = (long long)gridDim.x * blockDim.x;
     float local_max = 0.0f;
     int local_bad = 0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-        const long long plane = (long long)G.NX * G.NY;
-        const int z = (int)(i / plane);
-        const int y = (int)((i % plane) / G.NX);
-        const int x = (int)(i % G.NX);
+    for_cells(G.NX, G.NY, G.NZ, [&](int x, int y, int z) {
         const int mx = min(max(x - G.nb, 0), G.nx - 1);
         const int my = min(max(y - G.nb, 0), G.ny - 1);
         const int mz = min(max(z - G.nb, 0), G.nz - 1);
         const float v = vel[((long long)mz * G.ny + my) * G.nx + mx];
         const float v2 = squared ? v : v * v;
-        c[i] = v2 * dt2;
+        c[((long long)z * G.NY + y) * G.NX + x] = v2 * dt2;
         const bool interior = (x - G.nb == mx) && (y - G.nb == my) && (z - G.nb == mz);
         if (interior) {
             if (!(isfinite(v) && v > 0.0f)) local_bad = 1;
             else local_max = fmaxf(local_max, v2);
         }
-    }
-    // warp reduction then one atomic per warp
-    for (int o = 16; o > 0; o >>= 1) {
-        local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
-        local_bad |= __shfl_xor_sync(0xffffffffu, local_bad, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(vmax_bits, __float_as_uint(local_max));  // non-negative floats order as uints
-        if (local_bad) atomicOr(bad, 1);
-    }
+    });
+    if (local_bad) atomicOr(bad, 1);
+    block_max(local_max, vmax_bits);
 }
 
 __global__ void k_fwd_aux(Geometry G, const float* __restrict__ u_cur, float* u_prev,
@@ -138,13 +143,10 @@ __global__ void k_bwd_aux(Geometry G, const float* __restrict__ mu_cur, float* m
 
 __global__ void k_image_finalize(Geometry G, const float* __restrict__ slab,
                                  float* __restrict__ image) {
-    const long long n = (long long)G.nx * G.ny * G.nz;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const long long zy = i / G.nx;
-        const int x = (int)(i % G.nx);
-        image[i] += slab[zy * G.NX + x + G.nb];
-    }
+    for_cells(G.nx, G.ny, G.nz, [&](int x, int y, int z) {
+        const long long zy = (long long)z * G.ny + y;
+        image[zy * G.nx + x] += slab[zy * G.NX + x + G.nb];
+    });
 }
 
 // source illumination: illum[z][y][x] += u^2 of the model columns of a
@@ -156,7 +158,10 @@ __global__ void k_band_copy(Geometry G, int r, float* __restrict__ field,
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += stride) {
         int mx, my, mz;
-        band_cell(b, G.nx, G.ny, G.nz, r, mx, my, mz);
+        if (n < (1LL << 31))
+            band_cell_as<unsigned>((unsigned)b, G.nx, G.ny, G.nz, r, mx, my, mz);
+        else
+            band_cell(b, G.nx, G.ny, G.nz, r, mx, my, mz);
         const long long i =
             ((long long)(mz + G.nb) * G.NY + (my + G.nb)) * G.NX + (mx + G.nb);
         if (to_field)
@@ -210,8 +215,7 @@ __global__ void k_max_nonneg(const float* __restrict__ a, long long n, unsigned 
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
         m = fmaxf(m, a[i]);
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(bits, __float_as_uint(m));
+    block_max(m, bits);
 }
 
 // out = image / (illum + eps_rel * max illum)
@@ -228,11 +232,9 @@ __global__ void k_image_normalize(const float* __restrict__ image, const float* 
 // a[k] = a_k / dx^2
 __global__ void k_image_laplacian(const float* __restrict__ image, int nx, int ny, int nz,
                                   LapWeights w, float* __restrict__ out) {
-    const long long n = (long long)nx * ny * nz;
-    const long long stride = (long long)gridDim.x * blockDim.x;
     const long long sy = nx, sz = (long long)nx * ny;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / sz);
+    for_cells(nx, ny, nz, [&](int x, int y, int z) {
+        const long long i = z * sz + y * sy + x;
         float acc = w.a[0] * image[i];
         for (int k = 1; k <= w.r; k++) {
             float s = 0.f;
@@ -245,7 +247,7 @@ __global__ void k_image_laplacian(const float* __restrict__ image, int nx, int n
             acc = fmaf(w.a[k], s, acc);
         }
         out[i] = -acc;
-    }
+    });
 }
 
 __device__ __forceinline__ void fold_range(int m, int n, int nb, int N, int& lo, int& hi) {

@@ -40,35 +40,38 @@ __host__ __device__ inline long long band_offset(int mx, int my, int mz, int nx,
     return -1;
 }
 
-// model cell of band offset b, 0 <= b < band_cells (the inverse of band_offset)
-__host__ __device__ inline void band_cell(long long b, int nx, int ny, int nz, int r, int& mx,
-                                          int& my, int& mz) {
-    const long long r2 = 2LL * r;
-    const long long zface = r2 * ny * nx;
+// model cell of band offset b, 0 <= b < band_cells (the inverse of
+// band_offset). I: an unsigned type for band_cells below 2^31 (64-bit
+// divisions were most of the copy's work), else long long
+template <class I>
+__host__ __device__ inline void band_cell_as(I b, I nx, I ny, I nz, I r, int& mx, int& my, int& mz) {
+    const I r2 = 2 * r;
+    const I zface = r2 * ny * nx;
     if (b < zface) {
-        const long long fz = b / ((long long)ny * nx), rem = b - fz * ny * nx;
+        const I row = b / nx, fz = row / ny;
         mz = (int)(fz < r ? fz : fz + nz - r2);
-        my = (int)(rem / nx);
-        mx = (int)(rem - (long long)my * nx);
+        my = (int)(row - fz * ny);
+        mx = (int)(b - row * nx);
         return;
     }
     b -= zface;
-    const long long yface = (nz - r2) * r2 * nx;
+    const I yface = (nz - r2) * r2 * nx;
     if (b < yface) {
-        const long long zi = b / (r2 * nx), rem = b - zi * r2 * nx;
-        const int fy = (int)(rem / nx);
+        const I row = b / nx, zi = row / r2, fy = row - zi * r2;
         mz = (int)(zi + r);
-        my = fy < r ? fy : fy + ny - (int)r2;
-        mx = (int)(rem - (long long)fy * nx);
+        my = (int)(fy < r ? fy : fy + ny - r2);
+        mx = (int)(b - row * nx);
         return;
     }
     b -= yface;
-    const long long row = (ny - r2) * r2;
-    const long long zi = b / row, rem = b - zi * row;
-    const int yi = (int)(rem / r2), fx = (int)(rem - yi * r2);
+    const I row = b / r2, fx = b - row * r2, zi = row / (ny - r2);
     mz = (int)(zi + r);
-    my = yi + r;
-    mx = fx < r ? fx : fx + nx - (int)r2;
+    my = (int)(row - zi * (ny - r2) + r);
+    mx = (int)(fx < r ? fx : fx + nx - r2);
+}
+__host__ __device__ inline void band_cell(long long b, int nx, int ny, int nz, int r, int& mx,
+                                          int& my, int& mz) {
+    band_cell_as<long long>(b, nx, ny, nz, r, mx, my, mz);
 }
 
 }  // namespace rtm

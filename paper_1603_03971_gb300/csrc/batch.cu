@@ -19,6 +19,7 @@
 // (ld.global.cg); each block publishes its stores with a device-scope fence
 // before it increments the shot's counter.
 
+#include "cells.cuh"
 #include "batch_internal.h"
 #include "packed_f32x2.cuh"
 #include "stencil_common.cuh"
@@ -321,43 +322,33 @@ __global__ void __launch_bounds__(256, R == 4 ? 2 : 1) k_batch(const __grid_cons
 // sponge profiles of its padded grid
 __global__ void k_batch_prep(BatchShot S, const float* __restrict__ vel, int fnx, int fny, int ox,
                              int oy, int oz, float dt2, float* c, float* gx, float* gy, float* gz) {
-    const long long N = (long long)S.NX * S.NY * S.NZ;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % S.NX);
-        const int y = (int)((i / S.NX) % S.NY);
-        const int z = (int)(i / ((long long)S.NX * S.NY));
+    for_cells(S.NX, S.NY, S.NZ, [&](int x, int y, int z) {
         const int mx = min(max(x - S.nb, 0), S.nx - 1) + ox;
         const int my = min(max(y - S.nb, 0), S.ny - 1) + oy;
         const int mz = min(max(z - S.nb, 0), S.nz - 1) + oz;
         const float v = vel[((long long)mz * fny + my) * fnx + mx];
-        c[i] = v * v * dt2;
-        if (i < S.NX || i < S.NY || i < S.NZ) {
-            const int j = (int)i;
-            auto prof = [&](int n) {
-                const int d = min(j, n - 1 - j);
-                if (d >= S.nb) return 1.0f;
-                const double a = 0.015 * (double)(S.nb - d);
-                return (float)exp(-a * a);
-            };
-            if (j < S.NX) gx[j] = prof(S.NX);
-            if (j < S.NY) gy[j] = prof(S.NY);
-            if (j < S.NZ) gz[j] = prof(S.NZ);
-        }
+        c[((long long)z * S.NY + y) * S.NX + x] = v * v * dt2;
+    });
+    const int n = max(S.NX, max(S.NY, S.NZ));
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+        auto prof = [&](int side) {
+            const int d = min(j, side - 1 - j);
+            if (d >= S.nb) return 1.0f;
+            const double a = 0.015 * (double)(S.nb - d);
+            return (float)exp(-a * a);
+        };
+        if (j < S.NX) gx[j] = prof(S.NX);
+        if (j < S.NY) gy[j] = prof(S.NY);
+        if (j < S.NZ) gz[j] = prof(S.NZ);
     }
 }
 
 __global__ void k_batch_image_add(BatchShot S, const float* __restrict__ slab, int fnx, int fny,
                                   int ox, int oy, int oz, float* __restrict__ img) {
-    const long long n = (long long)S.nx * S.ny * S.nz;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % S.nx);
-        const int y = (int)((i / S.nx) % S.ny);
-        const int z = (int)(i / ((long long)S.nx * S.ny));
+    for_cells(S.nx, S.ny, S.nz, [&](int x, int y, int z) {
         img[((long long)(z + oz) * fny + (y + oy)) * fnx + (x + ox)] +=
             slab[((long long)z * S.ny + y) * S.NX + x + S.nb];
-    }
+    });
 }
 
 }  // namespace

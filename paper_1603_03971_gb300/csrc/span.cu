@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
                 float* band = A.band + (long long)(n - 1) * A.band_stride;
                 for (long long e = j0; e < A.band_stride; e += gridDim.x * T) {
                     int mx, my, mz;
-                    band_cell(e, A.nx, A.ny, A.nz, R, mx, my, mz);
+                    band_cell_as<unsigned>((unsigned)e, A.nx, A.ny, A.nz, R, mx, my, mz);
                     band[e] = __ldcg(cur + (size_t)(mz + A.nb) * plane +
                                      (size_t)(my + A.nb) * A.NX + (mx + A.nb));
                 }
