@@ -94,12 +94,37 @@ __global__ void k_model_prep(Geometry G, const float* __restrict__ vel, int squa
     block_max(local_max, vmax_bits);
 }
 
+// the boundary band of the model region, gathered from a padded field or
+// scattered into it by blocks first, first + 1, ... of a launch
+__device__ __forceinline__ void copy_band(const Geometry& G, const BandCopy& B, long long n, int first) {
+    const long long stride = (long long)(gridDim.x - first) * blockDim.x;
+    for (long long b = (long long)(blockIdx.x - first) * blockDim.x + threadIdx.x; b < n; b += stride) {
+        int mx, my, mz;
+        if (n < (1LL << 31))
+            band_cell_as<unsigned>((unsigned)b, G.nx, G.ny, G.nz, B.r, mx, my, mz);
+        else
+            band_cell(b, G.nx, G.ny, G.nz, B.r, mx, my, mz);
+        const long long i =
+            ((long long)(mz + G.nb) * G.NY + (my + G.nb)) * G.NX + (mx + G.nb);
+        if (B.to_field)
+            B.field[i] = B.band[b];
+        else
+            B.band[b] = B.field[i];
+    }
+}
+__global__ void k_band_copy(Geometry G, BandCopy B, long long n) {
+    pdl_wait();
+    copy_band(G, B, n, 0);
+}
+
 __global__ void k_fwd_aux(Geometry G, const float* __restrict__ u_cur, float* u_prev,
                           const float* __restrict__ c, const float* gx, const float* gy,
                           const float* gz, const int32_t* __restrict__ rec, int nrec,
                           float* data_row, long long src, const float* w_n, float inv_dx3,
-                          int* status) {
+                          int* status, BandCopy B, long long nband) {
     pdl_wait();
+    const int first = nrec / (int)blockDim.x + 1;  // blocks of the points
+    if ((int)blockIdx.x >= first) return copy_band(G, B, nband, first);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < nrec) {
         if (data_row) {
@@ -119,8 +144,11 @@ __global__ void k_bwd_aux(Geometry G, const float* __restrict__ mu_cur, float* m
                           const float* __restrict__ c, const float* gx, const float* gy,
                           const float* gz, const int32_t* __restrict__ rec, int nrec,
                           const float* __restrict__ r_row, long long src, float* src_adj_slot,
-                          float* grad_acc, const float* w_n, float inv_dx3, int* status) {
+                          float* grad_acc, const float* w_n, float inv_dx3, int* status,
+                          BandCopy B, long long nband) {
     pdl_wait();
+    const int first = nrec / (int)blockDim.x + 1;  // blocks of the points
+    if ((int)blockIdx.x >= first) return copy_band(G, B, nband, first);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < nrec) {
         if (r_row) {
@@ -151,26 +179,6 @@ __global__ void k_image_finalize(Geometry G, const float* __restrict__ slab,
 
 // source illumination: illum[z][y][x] += u^2 of the model columns of a
 // snapshot slab [nz][ny][NX]; 16-byte vectors along x when both rows allow
-// boundary band of the model region: gather from a padded field / scatter into it
-__global__ void k_band_copy(Geometry G, int r, float* __restrict__ field,
-                            float* __restrict__ band, long long n, int to_field) {
-    pdl_wait();
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += stride) {
-        int mx, my, mz;
-        if (n < (1LL << 31))
-            band_cell_as<unsigned>((unsigned)b, G.nx, G.ny, G.nz, r, mx, my, mz);
-        else
-            band_cell(b, G.nx, G.ny, G.nz, r, mx, my, mz);
-        const long long i =
-            ((long long)(mz + G.nb) * G.NY + (my + G.nb)) * G.NX + (mx + G.nb);
-        if (to_field)
-            field[i] = band[b];
-        else
-            band[b] = field[i];
-    }
-}
-
 // first element of model row zy = z ny + y: in the slab, or in a padded field
 __device__ __forceinline__ long long model_row(const Geometry& G, long long zy, int padded) {
     if (!padded) return zy * G.NX + G.nb;
@@ -606,23 +614,27 @@ cudaError_t launch_model_prep(const Geometry& G, const float* vel, int squared, 
     return cudaGetLastError();
 }
 
+// Boundary storage copies the band beside the points: as a launch of its own
+// (3-5 us at 150 x 131 x 117) it stood between two dependent kernels of every step
 cudaError_t launch_fwd_aux(const Geometry& G, const float* u_cur, float* u_prev, const float* c,
                            const float* gx, const float* gy, const float* gz,
                            const int32_t* rec, int nrec, float* data_row, long long src,
-                           const float* w_n, float inv_dx3, int* status, cudaStream_t s) {
-    const int n = nrec + 1;
-    return launch_next(k_fwd_aux, (n + 255) / 256, 256, 0, s, G, u_cur, u_prev, c, gx, gy, gz, rec,
-                       nrec, data_row, src, w_n, inv_dx3, status);
+                           const float* w_n, float inv_dx3, int* status, cudaStream_t s,
+                           const BandCopy& band) {
+    const long long nb = band.band ? band_cells(G.nx, G.ny, G.nz, band.r) : 0;
+    return launch_next(k_fwd_aux, nrec / 256 + 1 + (nb ? grid_for(nb, 256) : 0), 256, 0, s, G, u_cur,
+                       u_prev, c, gx, gy, gz, rec, nrec, data_row, src, w_n, inv_dx3, status, band, nb);
 }
 
 cudaError_t launch_bwd_aux(const Geometry& G, const float* mu_cur, float* mu_prev,
                            const float* c, const float* gx, const float* gy, const float* gz,
                            const int32_t* rec, int nrec, const float* r_row, long long src,
                            float* src_adj_slot, float* grad_acc, const float* w_n,
-                           float inv_dx3, int* status, cudaStream_t s) {
-    const int n = nrec + 1;
-    return launch_next(k_bwd_aux, (n + 255) / 256, 256, 0, s, G, mu_cur, mu_prev, c, gx, gy, gz, rec,
-                       nrec, r_row, src, src_adj_slot, grad_acc, w_n, inv_dx3, status);
+                           float inv_dx3, int* status, cudaStream_t s, const BandCopy& band) {
+    const long long nb = band.band ? band_cells(G.nx, G.ny, G.nz, band.r) : 0;
+    return launch_next(k_bwd_aux, nrec / 256 + 1 + (nb ? grid_for(nb, 256) : 0), 256, 0, s, G, mu_cur,
+                       mu_prev, c, gx, gy, gz, rec, nrec, r_row, src, src_adj_slot, grad_acc, w_n,
+                       inv_dx3, status, band, nb);
 }
 
 cudaError_t launch_image_finalize(const Geometry& G, const float* slab, float* image,
@@ -632,11 +644,9 @@ cudaError_t launch_image_finalize(const Geometry& G, const float* slab, float* i
     return cudaGetLastError();
 }
 
-cudaError_t launch_band_copy(const Geometry& G, int r, float* field, float* band, int to_field,
-                             cudaStream_t s) {
-    const long long n = band_cells(G.nx, G.ny, G.nz, r);
-    if (n <= 0) return cudaSuccess;
-    return launch_next(k_band_copy, grid_for(n, 256), 256, 0, s, G, r, field, band, n, to_field);
+cudaError_t launch_band_copy(const Geometry& G, const BandCopy& band, cudaStream_t s) {
+    const long long n = band_cells(G.nx, G.ny, G.nz, band.r);
+    return launch_next(k_band_copy, grid_for(n, 256), 256, 0, s, G, band, n);
 }
 
 cudaError_t launch_illum_add(const Geometry& G, const float* slab, float* illum, int padded,

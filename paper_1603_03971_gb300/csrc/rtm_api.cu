@@ -538,28 +538,40 @@ rtm_status prepare_tables(Ctx& C) {
     return RTM_OK;
 }
 
+// band: boundary storage's copy beside the points (on the grid) or after them
 rtm_status fwd_aux(Ctx& C, const float* cur, float* prev, const int32_t* rec, float* data_row,
-                   const float* w_n) {
-    if (C.taps)
+                   const float* w_n, const BandCopy& band = BandCopy{}) {
+    if (C.taps) {
         CU(launch_fwd_aux_off(C.G, cur, prev, C.base.c, C.base.gx, C.base.gy, C.base.gz, C.taps,
                               C.p->nrec, data_row, w_n, C.inv_dx3, C.status(), C.s));
-    else
+        if (band.band) {
+            CU(launch_band_copy(C.G, band, C.s));
+            count_launch();
+        }
+    } else {
         CU(launch_fwd_aux(C.G, cur, prev, C.base.c, C.base.gx, C.base.gy, C.base.gz, rec,
-                          C.p->nrec, data_row, C.src, w_n, C.inv_dx3, C.status(), C.s));
+                          C.p->nrec, data_row, C.src, w_n, C.inv_dx3, C.status(), C.s, band));
+    }
     count_launch();
     return RTM_OK;
 }
 
 rtm_status bwd_aux(Ctx& C, const float* mcur, float* mprev, const int32_t* rec,
-                   const float* r_row, float* src_adj_slot, float* grad_acc, const float* w_n) {
-    if (C.taps)  // imaging only: no gradient source term
+                   const float* r_row, float* src_adj_slot, float* grad_acc, const float* w_n,
+                   const BandCopy& band = BandCopy{}) {
+    if (C.taps) {  // imaging only: no gradient source term
         CU(launch_bwd_aux_off(C.G, mcur, mprev, C.base.c, C.base.gx, C.base.gy, C.base.gz,
                               C.taps, C.p->nrec, r_row, src_adj_slot, C.inv_dx3, C.status(),
                               C.s));
-    else
+        if (band.band) {
+            CU(launch_band_copy(C.G, band, C.s));
+            count_launch();
+        }
+    } else {
         CU(launch_bwd_aux(C.G, mcur, mprev, C.base.c, C.base.gx, C.base.gy, C.base.gz, rec,
                           C.p->nrec, r_row, C.src, src_adj_slot, grad_acc, w_n, C.inv_dx3,
-                          C.status(), C.s));
+                          C.status(), C.s, band));
+    }
     count_launch();
     return RTM_OK;
 }
@@ -616,7 +628,11 @@ rtm_status run_forward(Ctx& C, const int32_t* rec, float* data, float* u_last) {
             }
         }
         float* row = (data && n >= 1) ? data + (size_t)(n - 1) * p->nrec : nullptr;
-        CHECK(fwd_aux(C, cur, prev, rec, row, C.wav() + n));
+        // the band of u^n goes along with the points of this step
+        BandCopy band;
+        if (p->storage == RTM_STORE_BOUNDARY && n >= 1 && n <= p->nt - 2)
+            band = BandCopy{cur, C.band_of(n), p->radius, 0};
+        CHECK(fwd_aux(C, cur, prev, rec, row, C.wav() + n, band));
         int mode = MODE_FWD;
         float* snap = nullptr;
         if (p->storage == RTM_STORE_ALL) {
@@ -638,11 +654,6 @@ rtm_status run_forward(Ctx& C, const int32_t* rec, float* data, float* u_last) {
             mode = MODE_FWD_SUMSQ;
         }
         CHECK(stencil(C, mode, cur, prev, snap, nullptr, code ? &scal->sumsq : nullptr));
-        if (p->storage == RTM_STORE_BOUNDARY && n + 1 <= p->nt - 2) {
-            // the band of u^{n+1} (now in prev)
-            CU(launch_band_copy(C.G, p->radius, prev, C.band_of(n + 1), 0, C.s));
-            count_launch();
-        }
         if (decim) {  // u^{n+1} (now in prev): every other sample per axis
             CU(launch_decimate(C.G, prev, C.coarse_slot((size_t)((n + 1) / ie - 1)), C.s));
             count_launch();
@@ -781,11 +792,11 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
     CHECK(clear_span(C));
     const int ie = p->image_every;
 
-    auto back_step = [&](int m, float* snap) -> rtm_status {
+    auto back_step = [&](int m, float* snap, const BandCopy& band = BandCopy{}) -> rtm_status {
         float* adj = (src_adj && m < p->nt) ? src_adj + m : nullptr;
         float* gacc = (grad && m < p->nt) ? acc : nullptr;
         CHECK(bwd_aux(C, mcur, mprev, rec, rdata + (size_t)(m - 1) * p->nrec, adj, gacc,
-                      C.wav() + (m < p->nt ? m : 0)));
+                      C.wav() + (m < p->nt ? m : 0), band));
         int mode = MODE_FWD;
         if (grad) mode = MODE_BWD_GRAD;
         else if (m % ie == 0) mode = MODE_BWD_IMAGE;
@@ -870,19 +881,19 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
         float* lo = C.at(C.L.f[p->nt % 2]);        // u^m
         CHECK(back_step(p->nt, p->nt % ie == 0 ? hi : nullptr));
         for (int m = p->nt - 1; m >= 1; m--) {
+            BandCopy band;
             if (m <= p->nt - 2) {
                 // lo = u^{m+1}, hi = u^{m+2}: undo forward step m + 1 (its
                 // source injection is undone by the same pre-adjustment)
                 CHECK(fwd_aux(C, lo, hi, rec, nullptr, C.wav() + m + 1));
                 CHECK(stencil(C, MODE_REV, lo, hi, nullptr, nullptr));
                 // band cells: their stencils reach into the sponge; stored
-                CU(launch_band_copy(C.G, p->radius, hi, C.band_of(m), 1, C.s));
-                count_launch();
+                band = BandCopy{hi, C.band_of(m), p->radius, 1};
                 float* t = lo;
                 lo = hi;
                 hi = t;
             }
-            CHECK(back_step(m, m % ie == 0 ? lo : nullptr));
+            CHECK(back_step(m, m % ie == 0 ? lo : nullptr, band));
         }
     } else if (p->storage == RTM_STORE_ALL) {
         CHECK(back_steps(p->nt, 1, C.snap_slot(0), ie, 1));

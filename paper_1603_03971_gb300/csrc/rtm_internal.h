@@ -109,13 +109,22 @@ cudaError_t launch_sponge(const Geometry& G, float* gx, float* gy, float* gz, cu
 cudaError_t launch_wavelet(int nt, double dt, double f0, double t0, float* w, cudaStream_t s);
 cudaError_t launch_model_prep(const Geometry& G, const float* vel, int squared, double dt,
                               float* c, unsigned int* vmax_bits, int* bad, cudaStream_t s);
+// boundary band of a padded field to copy beside the aux work of a step: into
+// `band`, or back into the field; band NULL: none
+struct BandCopy {
+    float* field = nullptr;
+    float* band = nullptr;
+    int r = 0;
+    int to_field = 0;
+};
 // forward step n: gather d[n-1] = u_cur[rec] (if data_row), then pre-adjust
 // u_prev[s] -= c_s w / (dx^3 g_s^2) so that the stencil adds c_s w / dx^3.
 cudaError_t launch_fwd_aux(const Geometry& G, const float* u_cur, float* u_prev,
                            const float* c, const float* gx, const float* gy,
                            const float* gz, const int32_t* rec, int nrec,
                            float* data_row, long long src, const float* w_n,
-                           float inv_dx3, int* status, cudaStream_t s);
+                           float inv_dx3, int* status, cudaStream_t s,
+                           const BandCopy& band = BandCopy{});
 // backward step m: pre-adjust mu_prev[rec] -= c r / (dx^3 g) (if r_row) so
 // that the stencil adds c g r / dx^3; record the source trace of mu_cur and
 // the source term of the gradient (if requested).
@@ -124,7 +133,7 @@ cudaError_t launch_bwd_aux(const Geometry& G, const float* mu_cur, float* mu_pre
                            const float* gz, const int32_t* rec, int nrec,
                            const float* r_row, long long src, float* src_adj_slot,
                            float* grad_acc, const float* w_n, float inv_dx3,
-                           int* status, cudaStream_t s);
+                           int* status, cudaStream_t s, const BandCopy& band = BandCopy{});
 cudaError_t launch_image_finalize(const Geometry& G, const float* slab, float* image,
                                   cudaStream_t s);
 cudaError_t launch_grad_finalize(const Geometry& G, const float* acc, const float* c,
@@ -160,8 +169,7 @@ struct LapWeights {
 };
 // boundary band of the model region (band.cuh): gather it from a padded
 // field into band storage (to_field = 0) or scatter it back (to_field = 1)
-cudaError_t launch_band_copy(const Geometry& G, int r, float* field, float* band, int to_field,
-                             cudaStream_t s);
+cudaError_t launch_band_copy(const Geometry& G, const BandCopy& band, cudaStream_t s);
 // illum += u^2 over the model region; u: the model slab, or a padded field (padded = 1)
 cudaError_t launch_illum_add(const Geometry& G, const float* slab, float* illum, int padded,
                              cudaStream_t s);
