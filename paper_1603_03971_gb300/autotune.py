@@ -94,7 +94,7 @@ def tune_stencil(radius: int, padded_shape: Tuple[int, int, int], steps: int = 1
     TMA, 8-row tiles of 4-point vectors) and z-slab height for the
     single-shot stencil on a padded grid (NZ, NY, NX), timed on a
     constant-velocity model; trials are keyed "variant/zchunk"."""
-    from . import RtmError, alloc_workspace, make_params, model_prep, set_tuning
+    from . import RtmError, alloc_workspace, make_params, model_prep, set_tuning, set_tuning_mode
 
     key = _key("stencil", radius, padded_shape)
     with _lock:
@@ -112,6 +112,18 @@ def tune_stencil(radius: int, padded_shape: Tuple[int, int, int], steps: int = 1
     dobs = torch.zeros((steps, 1), device="cuda")
     img = torch.zeros((p.nz, p.ny, p.nx), device="cuda")
     results, modes = {}, {}
+
+    def best_of():
+        best = min(results, key=results.get)
+        # within the best variant, the fastest slab height of each mode (its
+        # launches move different bytes per point and balance differently)
+        per_mode = {}
+        for mode in ("fwd", "fwd_snap", "bwd_image"):
+            t = {zc: m[mode] for (v, zc), m in modes.items() if v == best[0] and mode in m}
+            if t:
+                per_mode[mode] = int(min(t, key=t.get))
+        return best, per_mode
+
     try:
         for variant in variants:
             for zc in candidates(NZ, radius):
@@ -121,18 +133,20 @@ def tune_stencil(radius: int, padded_shape: Tuple[int, int, int], steps: int = 1
                         p, c, rec, dobs, img, ws, steps)
                 except RtmError:
                     continue  # a variant this driver cannot run
+        # whole shots of the tuned and of the automatic choice: small grids take
+        # many steps per launch, which a fixed slab height rules out
+        best, per_mode = best_of()
+        set_tuning(radius, int(best[1]), int(best[0]))
+        for mode, zc in per_mode.items():
+            set_tuning_mode(radius, mode, zc)
+        tuned, _ = _time_shot(p, c, rec, dobs, img, ws, steps)
+        set_tuning(radius, 0, 0)
+        automatic, _ = _time_shot(p, c, rec, dobs, img, ws, steps)
     finally:
         set_tuning(radius, 0, 0)
-    best = min(results, key=results.get)
-    # within the best variant, the fastest slab height of each mode (its
-    # launches move different bytes per point and balance differently)
-    per_mode = {}
-    for mode in ("fwd", "fwd_snap", "bwd_image"):
-        t = {zc: m[mode] for (v, zc), m in modes.items() if v == best[0] and mode in m}
-        if t:
-            per_mode[mode] = int(min(t, key=t.get))
     choice = {"zchunk": int(best[1]), "variant": int(best[0]), "ms_per_step": results[best],
               "zchunk_modes": per_mode,
+              "whole_shot": {"tuned": tuned, "automatic": automatic},
               "trials": {"%d/%d" % k: v for k, v in results.items()},
               "trials_modes": {"%d/%d" % k: v for k, v in modes.items()}}
     with _lock:
@@ -194,7 +208,10 @@ def tune_batch(p, apertures, vel: torch.Tensor, nt: int = 8, cache_path: str = C
 
 def apply(radius: int, padded_shape, tune_if_missing: bool = True,
           cache_path: str = CACHE) -> Optional[dict]:
-    """Install the cached (or freshly tuned) stencil choice for this shape."""
+    """Install the cached (or freshly tuned) stencil choice for this shape, or
+    the automatic one (variant and slab heights 0) where whole shots of that
+    were faster by over a tenth: 104^3 at radius 4 takes 4.8 ms for 300 steps
+    each way against 11.8 tuned."""
     from . import set_tuning
 
     cache = load_cache(cache_path)
@@ -202,6 +219,9 @@ def apply(radius: int, padded_shape, tune_if_missing: bool = True,
     if choice is None and tune_if_missing:
         choice = tune_stencil(radius, padded_shape, cache_path=cache_path)
     if choice is not None:
+        t = choice.get("whole_shot")
+        if t and t["automatic"] < 0.9 * t["tuned"]:
+            choice = dict(choice, zchunk=0, variant=0, zchunk_modes={})
         set_tuning(radius, int(choice["zchunk"]), int(choice.get("variant", 0)))
         from . import set_tuning_mode
 

@@ -694,9 +694,9 @@ __global__ void k_latent_bias(const bf16* __restrict__ glat, long long nl, float
 
 template <class Op>
 cudaError_t run(const typename Op::Args& a, dim3 grid, int* status, cudaStream_t s) {
-    static const cudaError_t attr = cudaFuncSetAttribute(
+    const cudaError_t e = cudaFuncSetAttribute(
         k_tc_train<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, train_smem<Op>());
-    if (attr != cudaSuccess) return attr;
+    if (e != cudaSuccess) return e;
     k_tc_train<Op><<<grid, 160, train_smem<Op>(), s>>>(a, status);
     return cudaGetLastError();
 }
