@@ -714,7 +714,8 @@ cudaError_t ae_encode_march(const float* P, const ae::Vol& in, const float* inv_
     S.nitems = (int)(ncol * ((l.nz + S.zc - 1) / S.zc));
     EncArgs a{P, inv_sigma, lat, l, h, take_test_stall(RTM_STALL_ENCODER)};
     const int grid = std::min(nsm, S.nitems);
-    return launch_next(k_encode_march, dim3(grid), dim3(kThreads), kSmem, s, a, map, S, status);
+    // (one CTA per SM: early placement only starts its weights sooner)
+    return launch_dependent(true, k_encode_march, dim3(grid), dim3(kThreads), kSmem, s, a, map, S, status);
 }
 
 }  // namespace rtm
