@@ -29,8 +29,8 @@
 // 218 -> 82 -> 43, of E1 and D2 with the biases 387 -> 118 -> 71. A sample's
 // activations are 57 MB each: 8 us per pass over one at the HBM copy rate.
 // What is left: a CTA's copies are issued slab by slab, about 0.8 us each with
-// their index arithmetic, and the gathers move 3 to 8 times the activations
-// from L2.
+// their index arithmetic (L2 is 12-20 % busy), and tiles of two to four slabs
+// spend most of their time in start-up and epilogue.
 
 #include <cuda_bf16.h>
 #include <stdint.h>
