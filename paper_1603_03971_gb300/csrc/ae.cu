@@ -701,6 +701,10 @@ cudaError_t ae_rms(const Vol& in, AeScalars* sc, cudaStream_t s, float* sigma_ou
 
 cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScalars* sc,
                       float* sigma_out, int* status, cudaStream_t s, bool sumsq_ready) {
+    // k_encode_march stages the weights before it waits for the kernel before
+    // it. So the first kernel of the scale (k_scale here, k_sumsq in ae_rms) is
+    // an ordinary launch: it starts only once everything before the call,
+    // writers of the weights included, has completed
     cudaError_t e = cudaSuccess;
     if (sumsq_ready) {
         k_scale<<<1, 1, 0, s>>>(&sc->sumsq, (long long)in.nx * in.ny * in.nz, &sc->sigma,

@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int g = i / (kARows - NVOX), r = NVOX + i % (kARows - NVOX);
         *reinterpret_cast<uint4*>(atile + g * kATileBytes + r * 16) = make_uint4(0u, 0u, 0u, 0u);
     }
-    pdl_wait();  // the weights are staged while the kernels of the scale drain
+    pdl_wait();  // the weights are staged while the kernels of the scale drain (ae_encode())
     tc::fence_proxy_async();
     tc::tc_fence_before();
     __syncthreads();

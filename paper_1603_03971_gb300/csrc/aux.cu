@@ -117,7 +117,7 @@ __global__ void k_band_copy(Geometry G, BandCopy B, long long n) {
     copy_band(G, B, n, 0);
 }
 
-__global__ void k_fwd_aux(Geometry G, const float* __restrict__ u_cur, float* u_prev,
+__global__ void k_fwd_aux(Geometry G, const float* u_cur, float* u_prev,
                           const float* __restrict__ c, const float* gx, const float* gy,
                           const float* gz, const int32_t* __restrict__ rec, int nrec,
                           float* data_row, long long src, const float* w_n, float inv_dx3,
@@ -140,7 +140,7 @@ __global__ void k_fwd_aux(Geometry G, const float* __restrict__ u_cur, float* u_
     }
 }
 
-__global__ void k_bwd_aux(Geometry G, const float* __restrict__ mu_cur, float* mu_prev,
+__global__ void k_bwd_aux(Geometry G, const float* mu_cur, float* mu_prev,
                           const float* __restrict__ c, const float* gx, const float* gy,
                           const float* gz, const int32_t* __restrict__ rec, int nrec,
                           const float* __restrict__ r_row, long long src, float* src_adj_slot,
@@ -186,8 +186,7 @@ __device__ __forceinline__ long long model_row(const Geometry& G, long long zy, 
     return ((z + G.nb) * G.NY + (zy - z * G.ny) + G.nb) * G.NX + G.nb;
 }
 
-__global__ void k_illum_add(Geometry G, const float* __restrict__ slab,
-                            float* __restrict__ illum, int vec, int padded) {
+__global__ void k_illum_add(Geometry G, const float* slab, float* illum, int vec, int padded) {
     pdl_wait();
     const long long stride = (long long)gridDim.x * blockDim.x;
     if (vec) {
@@ -501,8 +500,7 @@ __global__ void k_finite_scan(const float* __restrict__ f, long long n, int vec,
 // on each axis, coarse[kz][ky][kx] = u[nb + 2 kz][nb + 2 ky][nb + 2 kx] of a
 // padded field; coarse sides are (n + 1) / 2. A block walks coarse rows
 // (ky, kz), its threads along x
-__global__ void k_decimate(Geometry G, const float* __restrict__ u, float* __restrict__ coarse,
-                           int cx, int cy, int cz) {
+__global__ void k_decimate(Geometry G, const float* u, float* coarse, int cx, int cy, int cz) {
     pdl_wait();
     for (int row = blockIdx.x; row < cy * cz; row += gridDim.x) {
         const int ky = row % cy, kz = row / cy;
@@ -528,7 +526,7 @@ __device__ __forceinline__ void lin_axis(int j, int nc, int& i0, float& w1) {
 // writes the even output sample (the kept column) and the odd one (the mean
 // of the two, or a copy past the last kept column)
 __global__ void k_upsample(Geometry G, const float* __restrict__ coarse, int cx, int cy, int cz,
-                           float* __restrict__ slab) {
+                           float* slab) {
     pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;

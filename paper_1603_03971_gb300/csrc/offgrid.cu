@@ -97,7 +97,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 // one warp per point: warps 0 .. nrec - 1 gather d[n-1] = sum_t W_t u^n[t]
 // (if data_row), warp nrec lowers u^{n-1} at the source taps by
 // c W w / (dx^3 g^2) so that the stencil adds c W w / dx^3 to u^{n+1}
-__global__ void k_fwd_aux_off(Geometry G, const float* __restrict__ u_cur, float* u_prev,
+__global__ void k_fwd_aux_off(Geometry G, const float* u_cur, float* u_prev,
                               const float* __restrict__ c, const float* gx, const float* gy,
                               const float* gz, const rtm_point_taps* __restrict__ taps, int nrec,
                               float* data_row, const float* w_n, float inv_dx3, int* status) {
@@ -140,7 +140,7 @@ __global__ void k_fwd_aux_off(Geometry G, const float* __restrict__ u_cur, float
 // one warp per point: warps 0 .. nrec - 1 lower mu^{m-1} at the receiver taps
 // by c W r / (dx^3 g) (overlapping taps of neighbouring receivers: atomics),
 // warp nrec records the source trace sum_t W_t mu^m[t] / g_t (if requested)
-__global__ void k_bwd_aux_off(Geometry G, const float* __restrict__ mu_cur, float* mu_prev,
+__global__ void k_bwd_aux_off(Geometry G, const float* mu_cur, float* mu_prev,
                               const float* __restrict__ c, const float* gx, const float* gy,
                               const float* gz, const rtm_point_taps* __restrict__ taps, int nrec,
                               const float* __restrict__ r_row, float* src_adj_slot,

@@ -4,9 +4,20 @@
 // in the stream drains: it sets up what needs no data and waits in
 // pdl_wait() until that kernel has completed and its writes are visible. On
 // short steps the launch latency between two dependent kernels is a good part
-// of the step (boundary storage runs seven kernels per time step). Every
-// thread of such a kernel calls pdl_wait() before it touches global memory, so
-// a kernel's completion implies that of all kernels before it.
+// of the step (boundary storage runs two kernels per forward and four per
+// backward step). Every thread of such a kernel calls pdl_wait() before it
+// touches what earlier kernels wrote, so a kernel's completion implies that of
+// all kernels before it. (k_encode_march reads its weights before the wait, which
+// the ordinary launch of the kernels of the scale allows: see ae_encode() in
+// ae.cu.)
+//
+// A kernel that is placed early lives while kernels before it still write the
+// fields: it may read those only through coherent loads (plain or at L2). The
+// read-only path (__ldg, or a const __restrict__ pointer) asks for data that
+// nobody writes while the kernel lives; it is for the coefficients, profiles,
+// receiver and tap tables, observed data and stored snapshots of a call. Nor
+// are fields __restrict__: a load through such a pointer may be moved above
+// the wait.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(BX* BY, 2)
         for (int i = 0; i < 2 * R; i++) {
             const int zz = zb - R + i;
             q[h][i] = own[h] && zz >= 0 && zz < A.NZ
-                          ? ld_keep(A.u_cur + (size_t)zz * plane + col + (size_t)h * A.NX)
+                          ? ld_l2(A.u_cur + (size_t)zz * plane + col + (size_t)h * A.NX)
                           : zero4();
         }
 #pragma unroll

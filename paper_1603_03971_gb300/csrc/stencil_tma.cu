@@ -91,9 +91,9 @@ __device__ __forceinline__ Vec<V> vlds(const float* p) {  // shared memory
     return r;
 }
 template <int V>
-__device__ __forceinline__ Vec<V> vld_keep(const float* p) {  // read-only global, keep cached
+__device__ __forceinline__ Vec<V> vld_l2(const float* p) {  // global, coherent at L2
     Vec<V> r;
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
     r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
     return r;
 }
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(16 * BY, (tma_min_blocks<R, MODE, BY>()))
 #pragma unroll
     for (int i = 0; i < 2 * R; i++) {
         const int zz = zb - R + i;
-        q[i] = (own && zz >= 0 && zz < A.NZ) ? vld_keep<V>(A.u_cur + (size_t)zz * plane + col)
+        q[i] = (own && zz >= 0 && zz < A.NZ) ? vld_l2<V>(A.u_cur + (size_t)zz * plane + col)
                                              : vzero<V>();
     }
 #pragma unroll
