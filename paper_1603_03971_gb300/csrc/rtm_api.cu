@@ -448,16 +448,21 @@ SpanArgs span_args(const Ctx& C, const SpanPlan& P, float* prev, float* cur, con
     return a;
 }
 
-// launches a span whose steps are of statistics slot `slot` and leaves the
-// newest state in cur
+// launches a span and leaves the newest state in cur. Its steps are counted
+// under the modes that they run in: those that write or image a snapshot
+// under `slot`, the others as plain steps
 rtm_status run_span(Ctx& C, SpanArgs& a, int slot, float*& prev, float*& cur) {
     a.base = C.span_count;
     CU(launch_span(a, C.s));
     C.span_count += (unsigned int)a.P.nbricks * (unsigned int)(a.nsteps - 1);
+    // the states of the span: lo + 1 .. lo + nsteps
+    const int lo = a.backward ? a.first - a.nsteps : a.first;
+    const int kept = a.snap ? (lo + a.nsteps) / a.every - lo / a.every : 0;
     {
         std::lock_guard<std::mutex> lk(g_mu);
-        g_stats.launches += 1;
-        g_stats.stencil_launches[slot] += a.nsteps;
+        g_stats.launches += a.scatter[0] && a.nrec > 0 ? 2 : 1;  // with the first step's scatter
+        g_stats.stencil_launches[slot] += kept;
+        g_stats.stencil_launches[MODE_FWD] += a.nsteps - kept;
     }
     if (a.nsteps & 1) std::swap(prev, cur);
     return RTM_OK;
