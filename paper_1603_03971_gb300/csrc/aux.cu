@@ -54,8 +54,6 @@ __global__ void k_wavelet(int nt, double dt, double f0, double t0, float* w) {
     w[n] = (float)((1.0 - 2.0 * a) * exp(-a));
 }
 
-// c = v^2 dt^2 on the padded grid (edge padding); max v^2 and validity over
-// the model cells
 // *bits = max(*bits, v) for a non-negative v of every thread of a block of at
 // most 1024. Floats of one sign compare as unsigned. Same-address atomics are served
 // one by one (one per warp of 19456: most of the 56 us of a 10 M cell model),
@@ -73,6 +71,8 @@ __device__ __forceinline__ void block_max(float v, unsigned int* bits) {
     }
 }
 
+// c = v^2 dt^2 on the padded grid (edge padding); max v^2 and validity over
+// the model cells
 __global__ void k_model_prep(Geometry G, const float* __restrict__ vel, int squared, float dt2,
                              float* __restrict__ c, unsigned int* vmax_bits, int* bad) {
     float local_max = 0.0f;
@@ -262,62 +262,20 @@ __device__ __forceinline__ void fold_range(int m, int n, int nb, int N, int& lo,
     hi = (m == n - 1) ? N - 1 : m + nb;
 }
 
-// A sum kept as an unevaluated pair of floats (about 48 bits). GB300 has
-// about two float64 lanes per SM and clock: a float64 divide, sum and
-// conversion per padded cell bounded the gradient's fold
-struct Pair {
-    float hi, lo;
-};
-// s += a + b, |b| small against a (Knuth's two-sum); an infinite or NaN sum
-// stays in hi
-__device__ __forceinline__ void pair_add(Pair& s, float a, float b) {
-    const float t = s.hi + a, bb = t - s.hi;
-    s.lo += ((s.hi - (t - bb)) + (a - bb)) + b;
-    s.hi = t;
-}
-// s += a / c as a rounded quotient and its correction. Products with 1 / c:
-// most cells of a short propagation hold denormal values, and a float divide
-// takes its slow path on those (0.53 against 0.10 ms for the inner cells at 256^3)
-__device__ __forceinline__ void pair_add_ratio(Pair& s, float a, float c) {
-    if (c > 1e-30f && c < 1e30f) {
-        const float rc = 1.0f / c, q = a * rc;
-        pair_add(s, q, fmaf(-q, c, a) * rc);
-    } else {
-        const float q = a / c;
-        pair_add(s, q, fmaf(-q, c, a) / c);
-    }
-}
-// the pair times a double, rounded once
-struct PairScale {
-    double full;
-    float hi, lo;  // hi + lo = full
-    int fits;      // full is well inside the float range
-};
-__device__ __forceinline__ float pair_scaled(const Pair& s, const PairScale& k) {
-    if (!isfinite(s.hi) || !isfinite(s.lo)) return (float)(s.hi * k.full);
-    if (!k.fits) return (float)(((double)s.hi + (double)s.lo) * k.full);
-    const float p = s.hi * k.hi;
-    if (!isfinite(p)) return p;
-    return p + (fmaf(s.hi, k.hi, -p) + fmaf(s.hi, k.lo, s.lo * k.hi));
-}
-__device__ __forceinline__ Pair warp_pair_sum(Pair s) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const float hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
-        const float lo = __shfl_xor_sync(0xffffffffu, s.lo, o);
-        pair_add(s, hi, lo);
-    }
-    return s;
-}
-
 // grad_v2[model cell] = dt^2 * sum over the padded cells copied from that
-// cell of dx^3 acc / c (the transpose of the edge padding). An inner cell has
-// one padded cell, a face cell nb + 1, an edge cell (nb + 1)^2, a corner cell
-// (nb + 1)^3: one thread per model cell left the eight corner threads with
-// 36 000 dependent sums at nb = 32 (57 ms of a 75 ms gradient at 256^3).
-// So a cell's padded cells decide who sums them: a thread (inner cells; z and
-// y faces, where neighbouring threads read neighbouring columns), a warp
-// (x faces, whose padded cells are a row, and edges) or a block (corners).
-// Memory-bound: 329 MB at 256^3, nb = 32, in 0.27 ms over the three kernels
+// cell of dx^3 acc / c (the transpose of the edge padding), in float64. An inner
+// cell has one padded cell, a face cell nb + 1, an edge cell (nb + 1)^2, a corner
+// cell (nb + 1)^3 (2 nb + 1 along a side of a single model cell): one thread per
+// model cell left the eight corner threads with 36 000 dependent sums at nb = 32
+// (57 ms of a 75 ms gradient at 256^3). So a cell's padded cells decide who sums
+// them: a thread (inner cells; z and y faces, where neighbouring threads read
+// neighbouring columns), a warp (x faces, whose padded cells are a row, and
+// edges) or a block (corners). The padded copies of a cell have its coefficient:
+// their values are summed and divided once. Bound by the float64 units, which
+// have about two lanes per SM and clock: 0.35 ms for the inner cells, 0.24 for
+// the faces and edges, 0.03 for the corners at 256^3, nb = 32 (memory: 0.05).
+// Sums and quotients as pairs of floats took 0.27 ms in all, but keep at most 48
+// bits and a float's range
 struct FoldBox {
     int x0, x1, y0, y1, z0, z1;
 };
@@ -336,9 +294,46 @@ __device__ __forceinline__ FoldOwner fold_owner(const FoldBox& b) {
     return y || z ? FOLD_COLUMN : FOLD_CELL;
 }
 
+// a / c in float64 by Newton's iteration: the float reciprocal, one step (48
+// bits), and the quotient corrected by its remainder, so rounded once more. Half
+// the float64 instructions of the operator: inner cells 0.78 -> 0.35 ms at 256^3
+__device__ __forceinline__ double quotient(double a, float c) {
+    if (!(c > 1e-30f && c < 1e30f)) return a / (double)c;
+    const double d = c, x0 = 1.0f / c, x = fma(x0, fma(-d, x0, 1.0), x0), q = a * x;
+    const bool finite = (__double2hiint(q) & 0x7ff00000) != 0x7ff00000;
+    return finite ? fma(fma(-d, q, a), x, q) : q;
+}
+// sum of acc / c over padded cells whose coefficients are mostly c0
+struct FoldSum {
+    float c0;
+    bool shared;          // c0 may divide a sum: 0 / 0 and x / 0 would differ
+    double a = 0.0;       // values over c0
+    double ratios = 0.0;  // quotients by other coefficients
+    __device__ explicit FoldSum(float c) : c0(c), shared(c > 0.f && c < INFINITY) {}
+    __device__ __forceinline__ void add(float v, float c) {
+        if (shared && c == c0)
+            a += (double)v;
+        else
+            ratios += quotient(v, c);
+    }
+    __device__ __forceinline__ double value() const {
+        return shared ? quotient(a, c0) + ratios : ratios;
+    }
+};
+__device__ __forceinline__ double warp_sum(double s) {
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+struct FoldScale {
+    double dx3, dt2;
+};
+__device__ __forceinline__ float fold_scaled(double s, const FoldScale& k) {
+    return (float)(s * k.dx3 * k.dt2);
+}
+
 // inner cells, a row per block and pass
 __global__ void k_grad_finalize(Geometry G, const float* __restrict__ acc,
-                                const float* __restrict__ c, PairScale scale,
+                                const float* __restrict__ c, FoldScale scale,
                                 float* __restrict__ grad) {
     const unsigned rows = (unsigned)G.ny * (unsigned)G.nz;
     for (unsigned row = blockIdx.x; row < rows; row += gridDim.x) {
@@ -348,34 +343,44 @@ __global__ void k_grad_finalize(Geometry G, const float* __restrict__ acc,
         const bool yz_inner = fold_owner(fold_box(G, 1 < G.nx - 1 ? 1 : 0, y, z)) == FOLD_CELL;
         for (int x = threadIdx.x; x < G.nx; x += blockDim.x) {
             if (G.nb > 0 && (!yz_inner || x == 0 || x == G.nx - 1)) continue;
-            Pair s{0.f, 0.f};
-            pair_add_ratio(s, __ldcs(acc + p + x), __ldcs(c + p + x));
-            out[x] = pair_scaled(s, scale);
+            out[x] = fold_scaled(quotient(__ldcs(acc + p + x), __ldcs(c + p + x)), scale);
         }
     }
 }
 
-// sum of a box over `n` threads, thread `t` of them, x fastest (a box holds
-// less than an eighth of the padded grid: 32-bit counts)
-__device__ __forceinline__ Pair fold_sum(const Geometry& G, const FoldBox& b,
-                                         const float* __restrict__ acc,
-                                         const float* __restrict__ c, int t, int n) {
-    const unsigned bx = b.x1 - b.x0 + 1, by = b.y1 - b.y0 + 1, bz = b.z1 - b.z0 + 1;
-    const unsigned cells = bx * by * bz;
-    Pair s{0.f, 0.f};
+// this thread's part of a box's sum: cells t, t + n, .. of `cells`, x fastest
+template <class I>
+__device__ __forceinline__ double fold_part(const Geometry& G, const FoldBox& b,
+                                            const float* __restrict__ acc,
+                                            const float* __restrict__ c, int t, int n, I cells) {
+    const unsigned bx = b.x1 - b.x0 + 1, by = b.y1 - b.y0 + 1;
+    auto at = [&](I k) {
+        const I zy = k / bx, zz = zy / by;
+        return ((long long)(b.z0 + zz) * G.NY + (b.y0 + (long long)(zy - zz * by))) * G.NX +
+               (b.x0 + (long long)(k - zy * bx));
+    };
+    FoldSum s(c[at(0)]);
 #pragma unroll 4
-    for (unsigned k = t; k < cells; k += n) {
-        const unsigned zy = k / bx, zz = zy / by;
-        const long long p = ((long long)(b.z0 + zz) * G.NY + (b.y0 + (zy - zz * by))) * G.NX +
-                            (b.x0 + (k - zy * bx));
-        pair_add_ratio(s, acc[p], c[p]);
+    for (I k = t; k < cells; k += n) {
+        const long long p = at(k);
+        s.add(acc[p], c[p]);
     }
-    return s;
+    return s.value();
+}
+// a box's sum over `n` threads, thread `t` of them (a side of a single model
+// cell is all in one box, so the counts may need 64 bits)
+__device__ __forceinline__ double fold_sum(const Geometry& G, const FoldBox& b,
+                                           const float* __restrict__ acc,
+                                           const float* __restrict__ c, int t, int n) {
+    const long long cells =
+        (long long)(b.x1 - b.x0 + 1) * (b.y1 - b.y0 + 1) * (b.z1 - b.z0 + 1);
+    return cells < (1LL << 31) ? fold_part<unsigned>(G, b, acc, c, t, n, (unsigned)cells)
+                               : fold_part<unsigned long long>(G, b, acc, c, t, n, cells);
 }
 
 // a row of y- or z-face cells, a column of padded cells per thread
 __device__ void fold_columns(const Geometry& G, int y, int z, const float* __restrict__ acc,
-                             const float* __restrict__ c, const PairScale& scale,
+                             const float* __restrict__ c, const FoldScale& scale,
                              float* __restrict__ grad) {
     for (int x = threadIdx.x; x < G.nx; x += blockDim.x) {
         const FoldBox b = fold_box(G, x, y, z);
@@ -384,28 +389,28 @@ __device__ void fold_columns(const Geometry& G, int y, int z, const float* __res
         const int n = along_y ? b.y1 - b.y0 + 1 : b.z1 - b.z0 + 1;
         const long long step = along_y ? G.NX : (long long)G.NX * G.NY;
         long long p = ((long long)b.z0 * G.NY + b.y0) * G.NX + b.x0;
-        Pair s{0.f, 0.f};
+        FoldSum s(c[p]);
 #pragma unroll 8
-        for (int k = 0; k < n; k++, p += step) pair_add_ratio(s, __ldcs(acc + p), __ldcs(c + p));
-        grad[((long long)z * G.ny + y) * G.nx + x] = pair_scaled(s, scale);
+        for (int k = 0; k < n; k++, p += step) s.add(__ldcs(acc + p), __ldcs(c + p));
+        grad[((long long)z * G.ny + y) * G.nx + x] = fold_scaled(s.value(), scale);
     }
 }
 
 __device__ void fold_warp(const Geometry& G, int x, int y, int z, const float* __restrict__ acc,
-                          const float* __restrict__ c, const PairScale& scale,
+                          const float* __restrict__ c, const FoldScale& scale,
                           float* __restrict__ grad) {
     const FoldBox b = fold_box(G, x, y, z);
     if (fold_owner(b) != FOLD_WARP) return;  // the same for the whole warp
     const int lane = threadIdx.x & 31;
-    const Pair s = warp_pair_sum(fold_sum(G, b, acc, c, lane, 32));
-    if (lane == 0) grad[((long long)z * G.ny + y) * G.nx + x] = pair_scaled(s, scale);
+    const double s = warp_sum(fold_sum(G, b, acc, c, lane, 32));
+    if (lane == 0) grad[((long long)z * G.ny + y) * G.nx + x] = fold_scaled(s, scale);
 }
 
 // the face and edge cells. blockIdx.y: 0 and 1 the x faces (a warp per cell),
 // 2 and 3 the z faces, 4 and 5 the y faces (a row of cells per block), 6 the
 // four edges along x (a warp per cell)
 __global__ void k_grad_finalize_faces(Geometry G, const float* __restrict__ acc,
-                                      const float* __restrict__ c, PairScale scale,
+                                      const float* __restrict__ c, FoldScale scale,
                                       float* __restrict__ grad) {
     const int what = blockIdx.y, far_side = what & 1;
     const unsigned warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -439,19 +444,19 @@ __global__ void k_grad_finalize_faces(Geometry G, const float* __restrict__ acc,
 __global__ void __launch_bounds__(1024) k_grad_finalize_corners(Geometry G,
                                                                 const float* __restrict__ acc,
                                                                 const float* __restrict__ c,
-                                                                PairScale scale,
+                                                                FoldScale scale,
                                                                 float* __restrict__ grad) {
-    __shared__ Pair part[32];
+    __shared__ double part[32];
     const int e = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (((e & 1) && G.nx == 1) || ((e & 2) && G.ny == 1) || ((e & 4) && G.nz == 1)) return;
     const int x = e & 1 ? G.nx - 1 : 0, y = e & 2 ? G.ny - 1 : 0, z = e & 4 ? G.nz - 1 : 0;
     const FoldBox b = fold_box(G, x, y, z);
-    Pair s = warp_pair_sum(fold_sum(G, b, acc, c, threadIdx.x, blockDim.x));
+    double s = warp_sum(fold_sum(G, b, acc, c, threadIdx.x, blockDim.x));
     if (lane == 0) part[wid] = s;
     __syncthreads();
     if (wid == 0) {
-        s = warp_pair_sum(part[lane]);
-        if (lane == 0) grad[((long long)z * G.ny + y) * G.nx + x] = pair_scaled(s, scale);
+        s = warp_sum(part[lane]);
+        if (lane == 0) grad[((long long)z * G.ny + y) * G.nx + x] = fold_scaled(s, scale);
     }
 }
 
@@ -678,9 +683,7 @@ cudaError_t launch_image_laplacian(const float* image, int nx, int ny, int nz,
 
 cudaError_t launch_grad_finalize(const Geometry& G, const float* acc, const float* c,
                                  double dx3, double dt2, float* grad_v2, cudaStream_t s) {
-    const double full = dx3 * dt2;
-    const float hi = (float)full;
-    const PairScale scale{full, hi, (float)(full - (double)hi), full > 1e-20 && full < 1e20};
+    const FoldScale scale{dx3, dt2};
     const long long rows = (long long)G.ny * G.nz;
     k_grad_finalize<<<grid_for(rows, 1), 256, 0, s>>>(G, acc, c, scale, grad_v2);
     if (G.nb > 0) {
