@@ -569,23 +569,53 @@ __global__ void k_scale(const double* acc, long long n, float* sigma, float* inv
     if (sigma_out) *sigma_out = (float)r;
 }
 
+// A sum of squares with more than a float64's bits in three floats: GB300 has few
+// float64 lanes, and two float64 operations per sample took half of k_loss. Squares
+// and sums carry their rounding errors along (two-product by fma, Knuth's
+// two-sum; no plain operators, which the compiler may contract). Outside the
+// range where the errors are floats too, a square goes to the float64 part
+struct SquareSum {
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    double beyond = 0.0;
+    __device__ __forceinline__ static float two_sum(float& s, float v) {  // s += v; its error
+        const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b));
+        s = t;
+        return e;
+    }
+    __device__ __forceinline__ void add(float d) {
+        const float m = fabsf(d);
+        if (m == 0.f) return;
+        // the square's 48 bits lie above 2^-149, sums of them below 2^128
+        if (m > 1e-15f && m < 1e15f) {
+            const float p = __fmul_rn(d, d);
+            const float e0 = two_sum(s0, p), e1 = two_sum(s1, e0);
+            const float e2 = two_sum(s1, __fmaf_rn(d, d, -p));
+            s2 = __fadd_rn(s2, __fadd_rn(e1, e2));
+        } else {
+            beyond += (double)d * d;
+        }
+    }
+    __device__ __forceinline__ double value() const {
+        return (double)s0 + ((double)s1 + (double)s2) + beyond;
+    }
+};
+
 // loss += mean((y - x0)^2) * scale; gy = bf16(scale * 2 (y - x0) / n); grad[b4] += sum gy.
 // y and gy are dense; in is read as one array where it is dense too, four
-// values at a time where `vec` says so. The squares are summed as pairs of
-// floats (exact products, about 48 bits): GB300 has few float64 lanes, and two
-// float64 operations per sample took half of the kernel's 54 us at 192^3
+// values at a time where `vec` says so. 23 us at 192^3 (54 with one value at a time
+// and float64 sums; 19 with the squares in pairs of floats, which lost bits and range)
 __global__ void __launch_bounds__(256) k_loss(const float* __restrict__ y, Vol in,
                                               const float* inv_sigma, float scale, int vec, bf16* gy,
                                               double* loss, float* grad) {
     const long long n = (long long)in.nx * in.ny * in.nz;
     const bool dense = in.sy == in.nx && in.sz == (long long)in.nx * in.ny;
     const float s = *inv_sigma;
-    float hi = 0.f, lo = 0.f, gsum = 0.f;
+    SquareSum squares;
+    float gsum = 0.f;
     auto one = [&](float yv, float xv) {
         const float d = yv - xv * s;
-        const float p = d * d, t = hi + p, bb = t - hi;
-        lo += ((hi - (t - bb)) + (p - bb)) + fmaf(d, d, -p);
-        hi = t;
+        squares.add(d);
         const bf16 g = __float2bfloat16_rn(scale * 2.0f * d / (float)n);
         gsum += __bfloat162float(g);
         return g;
@@ -613,7 +643,7 @@ __global__ void __launch_bounds__(256) k_loss(const float* __restrict__ y, Vol i
             gy[i] = one(y[i], in.p[at]);
         }
     }
-    double l = (double)hi + (double)lo;
+    double l = squares.value();
     for (int o = 16; o > 0; o >>= 1) {
         l += __shfl_xor_sync(0xffffffffu, l, o);
         gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
