@@ -389,8 +389,9 @@ rtm_status make_ctx(Ctx& C, const rtm_params* p, const float* c, void* ws, rtm_s
     // 8-row tiles at radius 4 (the faster ones at every shape from 192 x 173 x
     // 159 to 576^3: 454 / 565 / 740 against 459 / 568 / 749 us per launch at
     // 576^3), 16-row tiles with two rows per thread at radius 8 (534 / 592 /
-    // 780 against 645 / 695 / 795)
-    C.variant = var != 0 ? var : (tma_available() ? (p->radius == 4 ? 3 : 2) : 1);
+    // 780 against 645 / 695 / 795). A grid has at most 65535 rows of tiles
+    const bool rows8 = p->radius == 4 && C.d.NY <= 65535 * 8;
+    C.variant = var != 0 ? var : (tma_available() ? (rows8 ? 3 : 2) : 1);
     C.snap_padded = p->storage == RTM_STORE_BOUNDARY;
     set_region(C.base, MODE_FWD);
     // spans replace the automatic choice only: a tuned variant or slab height
