@@ -25,8 +25,8 @@
 //
 // us per 192^3 sample, general engine -> one role for copies and products ->
 // now: E2 99 -> 68 -> 48, D1 109 -> 73 -> 56, D1's data gradient 219 -> 145 ->
-// 103, E2's 175 -> 64 -> 58, weight gradients of E2 241 -> 68 -> 55, of D1
-// 218 -> 82 -> 43, of E1 and D2 with the biases 387 -> 118 -> 71. A sample's
+// 103, E2's 175 -> 64 -> 54, weight gradients of E2 241 -> 68 -> 56, of D1
+// 218 -> 82 -> 47, of E1 and D2 with the biases 387 -> 118 -> 81. A sample's
 // activations are 57 MB each: 8 us per pass over one at the HBM copy rate.
 // What is left: a CTA's copies are issued slab by slab, about 0.8 us each with
 // their index arithmetic (L2 is 12-20 % busy), and tiles of two to four slabs
@@ -303,6 +303,7 @@ struct TE2 {  // h1 -> latent
     static constexpr int kS = 6;
     static constexpr int N = 16;
     static constexpr bool kMN = false;
+    static constexpr int kTurn = 1 << 30;  // one accumulator
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = 27;
@@ -330,6 +331,7 @@ struct TD1 {  // latent -> g1, output parity blockIdx.y
     static constexpr int kS = 2;
     static constexpr int N = 32;
     static constexpr bool kMN = false;
+    static constexpr int kTurn = 1 << 30;  // one accumulator
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = 4;
@@ -364,6 +366,7 @@ struct TD1d {  // ga3 -> glat: dlat[j] = sum_k W3[.,k,.]^T ga3[2j + k - 1]
     static constexpr int kS = 6;
     static constexpr int N = 16;
     static constexpr bool kMN = false;
+    static constexpr int kTurn = 1 << 30;  // one accumulator
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = 64;
@@ -387,6 +390,7 @@ struct TE2d {  // glat -> ga1 at output parity blockIdx.y: (sum of W2^T glat) * 
     static constexpr int kS = 2;
     static constexpr int N = 32;
     static constexpr bool kMN = false;
+    static constexpr int kTurn = 1 << 30;  // one accumulator
     __device__ static void range(const Args&, int& c0, int& c1) {
         c0 = 0;
         c1 = (e2d_taps(blockIdx.y) + 1) / 2;
@@ -448,6 +452,7 @@ struct TE2w {  // dW2[o][tap][i] += sum_v glat[v][o] h1[2v + tap - 1][i]; blockI
     static constexpr int kS = 6;
     static constexpr int N = 16;
     static constexpr bool kMN = true;
+    static constexpr int kTurn = 4;
     __device__ static void range(const Args& a, int& c0, int& c1) { slab_range(a, blockIdx.y, c0, c1); }
     __device__ static Where where(const Args&, int) { return Where{}; }
     __device__ static void load(const Args& a, const Where&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
@@ -481,6 +486,7 @@ struct TD1w {  // dW3[o][k][i] += sum_j ga3[2j + q][o] lat[j + t][i], parity q =
     static constexpr int kS = 6;
     static constexpr int N = 32;
     static constexpr bool kMN = true;
+    static constexpr int kTurn = 4;
     __device__ static void range(const Args& a, int& c0, int& c1) { slab_range(a, blockIdx.y, c0, c1); }
     __device__ static Where where(const Args&, int) { return Where{}; }
     __device__ static void load(const Args& a, const Where&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
@@ -533,6 +539,7 @@ struct TPatch {
     static constexpr int kS = 10;
     static constexpr int N = 32;
     static constexpr bool kMN = true;
+    static constexpr int kTurn = 1;
     __device__ static void range(const Args& a, int& c0, int& c1) { slab_range(a, blockIdx.x, c0, c1); }
     __device__ static Where where(const Args&, int) { return Where{}; }
     __device__ static void load(const Args& a, const Where&, int ch, uint8_t* sA, uint8_t* sB, int tid) {
@@ -585,20 +592,39 @@ struct TPatch {
 // the threads that copy would wait for all of their copies in flight, and with
 // it every slab for the memory's full latency, however deep the ring.
 // Op::kS: stages of 10 KB; two for the products of few slabs (six CTAs per SM),
-// 6 to 10 for the long ones (104 against 127 us with two for D1's gradient)
+// 6 to 10 for the long ones (104 against 127 us with two for D1's gradient).
+//
+// The weight gradients' contractions are as long as the volume, and the tensor
+// cores truncate what they add to an accumulator: over the 180 steps of a CTA
+// at 192^3 the gradients of W1, W4, b1 and b3 lost 4-8 times what float32 sums
+// of the lanes had lost. So two accumulators take turns, Op::kTurn steps each, and
+// warps 5-8 add the finished one to sums in registers, rounded to nearest,
+// while the next is filled. Relative L2 error against float64 sums of the same
+// operands, lanes / one accumulator / turns: W1 3.8e-7 / 3.0e-6 / 2.5e-7, W4
+// 3.7e-7 / 2.3e-6 / 2.6e-7, W2 5.9e-7 / 1.3e-6 / 1.4e-7, W3 9.3e-7 / 2.9e-6 /
+// 1.4e-7 at 192^3; at 64^3 W1 1.2e-7 / 5.4e-7 / 1.2e-7, W3 1.7e-7 / 5.8e-7 / 9e-8.
+// The patch products, whose lanes had summed single voxels, take a turn per step
+// (72 -> 81 us), the others four steps, which cost them 1-2 us
 template <class Op>
 constexpr int train_smem() {
     return Op::kS * tc::kStageBytes + 1024;
 }
+template <class Op>
+constexpr int train_threads() {
+    return Op::kMN ? 288 : 160;
+}
 
 template <class Op>
-__global__ void __launch_bounds__(160) k_tc_train(const __grid_constant__ typename Op::Args args,
-                                                  int* status) {
+__global__ void __launch_bounds__(train_threads<Op>()) k_tc_train(
+    const __grid_constant__ typename Op::Args args, int* status) {
     constexpr int N = Op::N, kS = Op::kS;
+    constexpr int kCols = Op::kMN ? 2 * tc::kTmemCols : tc::kTmemCols;
+    constexpr int kSteps = tc::kBK / 16, kTurn = Op::kTurn;
     extern __shared__ uint8_t raw[];
     uint8_t(*smem)[tc::kStageBytes] = reinterpret_cast<uint8_t(*)[tc::kStageBytes]>(
         (reinterpret_cast<uintptr_t>(raw) + 1023) & ~static_cast<uintptr_t>(1023));
     __shared__ __align__(8) uint64_t full[kS], empty[kS], done;
+    __shared__ __align__(8) uint64_t acc_full[2], acc_free[2];  // kMN: an accumulator's turns
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = tid >> 5;
     int c0, c1;
@@ -610,10 +636,14 @@ __global__ void __launch_bounds__(160) k_tc_train(const __grid_constant__ typena
             tc::mbar_init(&full[s], 128);
             tc::mbar_init(&empty[s], 1);
         }
+        for (int b = 0; b < 2; b++) {
+            tc::mbar_init(&acc_full[b], 1);
+            tc::mbar_init(&acc_free[b], 128);
+        }
         tc::mbar_init(&done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tc::tmem_alloc(&tmem_slot, tc::kTmemCols);
+    if (warp == 0) tc::tmem_alloc(&tmem_slot, kCols);
     if (warp < 4) {
         for (int s = 0; s < kS; s++) Op::init(smem[s] + tc::kABytes, tid);
         tc::fence_proxy_async();
@@ -624,6 +654,9 @@ __global__ void __launch_bounds__(160) k_tc_train(const __grid_constant__ typena
     const uint32_t tmem = tmem_slot;
 
     bool ok = true;
+    float sum[N];
+#pragma unroll
+    for (int n = 0; n < N; n++) sum[n] = 0.f;
     if (warp == 4) {
         if (tid == 128 && nch > 0) {
             // MN-major A and B: transpose bits 15 and 16
@@ -635,16 +668,25 @@ __global__ void __launch_bounds__(160) k_tc_train(const __grid_constant__ typena
                 tc::tc_fence_after();
                 const uint32_t a0 = tc::smem_u32(smem[i % kS]), b0 = a0 + tc::kABytes;
 #pragma unroll
-                for (int s = 0; s < tc::kBK / 16; s++)
-                    tc::mma_bf16(tmem, tc::sdesc(a0 + 256 * s, 128, 512),
-                                 tc::sdesc(b0 + 256 * s, 128, 512), idesc,
-                                 (i > 0 || s > 0) ? 1u : 0u);
-                tc::mma_commit(&empty[i % kS]);
+                for (int s = 0; s < kSteps; s++) {
+                    const int step = kSteps * i + s, turn = step / kTurn, b = turn & 1;
+                    const bool first = step % kTurn == 0;
+                    if (first && turn >= 2) {
+                        ok = tc::mbar_wait(&acc_free[b], (uint32_t)((turn / 2 - 1) & 1));
+                        if (!ok) break;
+                        tc::tc_fence_after();
+                    }
+                    tc::mma_bf16(tmem + b * tc::kTmemCols, tc::sdesc(a0 + 256 * s, 128, 512),
+                                 tc::sdesc(b0 + 256 * s, 128, 512), idesc, first ? 0u : 1u);
+                    if (Op::kMN && (step % kTurn == kTurn - 1 || step == kSteps * nch - 1))
+                        tc::mma_commit(&acc_full[b]);
+                }
+                if (ok) tc::mma_commit(&empty[i % kS]);
             }
             tc::mma_commit(&done);
         }
         __syncwarp();
-    } else {
+    } else if (warp < 4) {
         const typename Op::Where where = Op::where(args, tid);
         for (int j = 0; j < nch; j++) {
             if (j >= kS) ok = tc::mbar_wait(&empty[j % kS], (uint32_t)((j / kS - 1) & 1));
@@ -655,13 +697,32 @@ __global__ void __launch_bounds__(160) k_tc_train(const __grid_constant__ typena
                          : "memory");
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if constexpr (Op::kMN) {
+        for (int turn = 0; turn * kTurn < kSteps * nch; turn++) {
+            const int b = turn & 1;
+            ok = tc::mbar_wait(&acc_full[b], (uint32_t)((turn / 2) & 1));
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc::tc_fence_after();
+            float acc[N];
+            const uint32_t t = tmem + b * tc::kTmemCols + ((uint32_t)((warp & 3) * 32) << 16);
+            tc::tmem_ld16(t, acc);
+            if constexpr (N == 32) tc::tmem_ld16(t + 16, acc + 16);
+            tc::tc_fence_before();
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&acc_free[b]))
+                         : "memory");
+#pragma unroll
+            for (int n = 0; n < N; n++) sum[n] += acc[n];
+        }
     }
-    // the products are done with the stages and the accumulator
+    // the products are done with the stages and the accumulators
     if (nch > 0 && tid <= 128) ok = tc::mbar_wait(&done, 0) && ok;
     ok = __syncthreads_and(ok);
     tc::tc_fence_after();
     if (ok && nch > 0) {
-        if (warp < 4) {
+        if constexpr (Op::kMN) {
+            if (warp > 4) Op::epilogue(args, (warp & 3) * 32 + (tid & 31), nullptr, sum);
+        } else if (warp < 4) {
             float acc[N];
             const uint32_t t = tmem + ((uint32_t)(warp * 32) << 16);
             tc::tmem_ld16(t, acc);
@@ -673,7 +734,7 @@ __global__ void __launch_bounds__(160) k_tc_train(const __grid_constant__ typena
     }
     tc::tc_fence_before();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, tc::kTmemCols);
+    if (warp == 0) tc::tmem_dealloc(tmem, kCols);
 }
 
 // db2 += sum_v glat[v]
@@ -697,7 +758,7 @@ cudaError_t run(const typename Op::Args& a, dim3 grid, int* status, cudaStream_t
     const cudaError_t e = cudaFuncSetAttribute(
         k_tc_train<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, train_smem<Op>());
     if (e != cudaSuccess) return e;
-    k_tc_train<Op><<<grid, 160, train_smem<Op>(), s>>>(a, status);
+    k_tc_train<Op><<<grid, train_threads<Op>(), train_smem<Op>(), s>>>(a, status);
     return cudaGetLastError();
 }
 
