@@ -680,7 +680,9 @@ cudaError_t launch_span_t(const SpanArgs& a, cudaStream_t s) {
         if ((e = encode_box(&M.u[i], a.f[i], a, R)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.P.nbricks);
-    cfg.blockDim = dim3(a.P.threads);
+    // off the grid the block's warps share its receivers too: a small brick's
+    // cells alone would leave them to one or two warps
+    cfg.blockDim = dim3(OFF ? span_threads<R, BWD, PZ>() : a.P.threads);
     cfg.dynamicSmemBytes = a.P.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
