@@ -818,12 +818,23 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
         return RTM_OK;
     };
 
+    // off the grid the source's field pair is scratch while the receivers
+    // propagate, except where its states are still to be recomputed from it.
+    // Without scratch every brick takes all receivers that reach it, in every
+    // step: about 30 ns each at 104^3, on top of 15 us, where a step of launches
+    // takes 25. Binomial shots of 60 steps (104^3 / 40 x 36 x 32) with 256, 1024,
+    // 3969 receivers, spans: 4.3 / 3.3, 5.8 / 5.8, 11.5 / 16.7 ms; with the
+    // receivers' steps as launches, 3969: 5.0 / 3.9
+    const bool scratch = C.taps && p->storage != RTM_STORE_REVOLVE;
+    const bool span_bwd = C.span_bwd.ok && !C.snap_padded &&
+                          (!C.taps || scratch || p->nrec <= 512);
+
     // steps m = hi .. lo; the imaging steps read the snapshot of state m at
     // snap + (m / div - off) * L.snap_elems, or snap itself with div = 0
     auto back_steps = [&](int hi, int lo, float* snap, int div, int off) -> rtm_status {
         if (hi < lo) return RTM_OK;
         const long long stride = div ? (long long)C.L.snap_elems : 0;
-        if (C.span_bwd.ok && !C.snap_padded) {
+        if (span_bwd) {
             SpanArgs a = span_args(C, C.span_bwd, mprev, mcur, rec, hi, hi - lo + 1);
             a.backward = 1;
             a.grad = grad;
@@ -835,9 +846,7 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
             a.off = off;
             a.acc = acc;
             a.illum = C.illum;
-            // the source's field pair is scratch while the receivers propagate,
-            // except where its states are still to be recomputed from it
-            if (C.taps && p->storage != RTM_STORE_REVOLVE)
+            if (scratch)
                 for (int i = 0; i < 2; i++) a.scatter[i] = C.at(C.L.f[i]);
             return run_span(C, a, snap ? (grad ? MODE_BWD_GRAD : MODE_BWD_IMAGE) : MODE_FWD, mprev,
                             mcur);

@@ -65,3 +65,10 @@ def _off_grid(nx, ny, nz, nb, storage, ckpt, nrec):
 def test_off_grid_receivers_of_a_small_grid(nrec):
     spans, launches = _spans_and_launches(4, _off_grid(28, 24, 20, 6, "ckpt", 10, nrec))
     assert spans <= SLACK * launches
+
+
+@pytest.mark.parametrize("grid", [(28, 24, 20, 6), (64, 64, 64, 20)])
+@pytest.mark.parametrize("nrec", [256, 1024, 3969])
+def test_off_grid_receivers_under_binomial_checkpointing(grid, nrec):
+    spans, launches = _spans_and_launches(4, _off_grid(*grid, "revolve", 10, nrec))
+    assert spans <= SLACK * launches
