@@ -826,8 +826,15 @@ rtm_status run_backward(Ctx& C, const int32_t* rec, const float* rdata, float* s
     // 3969 receivers, spans: 4.3 / 3.3, 5.8 / 5.8, 11.5 / 16.7 ms; with the
     // receivers' steps as launches, 3969: 5.0 / 3.9
     const bool scratch = C.taps && p->storage != RTM_STORE_REVOLVE;
-    const bool span_bwd = C.span_bwd.ok && !C.snap_padded &&
-                          (!C.taps || scratch || p->nrec <= 512);
+    // On the grid a brick lists its receivers. Past the list's end every step of
+    // every block looks at all receivers, 0.6 ns each: at 128 x 122 x 112 padded
+    // 34560 receivers made a step 36 us and 691200 387, where launches take 12
+    // and 15. A brick of fewer cells than its list holds does not get there
+    const SpanPlan& P = C.span_bwd;
+    const bool listed = p->nrec <= 16384 || (4 * P.bxv * P.by * P.bz <= kSpanListCap &&
+                                             (size_t)p->nrec <= C.d.N);
+    const bool span_bwd =
+        P.ok && !C.snap_padded && (C.taps ? scratch || p->nrec <= 512 : listed);
 
     // steps m = hi .. lo; the imaging steps read the snapshot of state m at
     // snap + (m / div - off) * L.snap_elems, or snap itself with div = 0

@@ -56,7 +56,6 @@ namespace {
 // planes per thread: a column of 4 shares its z neighbours' loads; grids that
 // leave a block few columns spread them over four times the threads
 constexpr int kColumn = 4;
-constexpr int kListCap = 2048;                           // receivers of a block kept in shared memory
 constexpr int kTapCap = 32;                              // tap tables of a block kept in shared memory
 constexpr unsigned long long kBarrierNs = 20000000000ull;  // bound of a grid barrier: 20 s
 constexpr int kSmemMax = 227 * 1024;
@@ -68,7 +67,7 @@ __host__ __device__ constexpr int span_threads() {
     return PZ == 1 || R == 4 ? 512 : 384;
 }
 
-static_assert(sizeof(rtm_point_taps) * kTapCap <= 4 * kListCap, "tap tables share the list's room");
+static_assert(sizeof(rtm_point_taps) * kTapCap <= 4 * kSpanListCap, "tap tables share the list's room");
 
 struct SpanMaps {
     CUtensorMap u[2];
@@ -217,7 +216,7 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
     if (!BWD && OFF && blockIdx.x == 0 && tid == 0 && taps_outside(A.taps[0], A))
         atomicCAS(A.status, 0, RTM_ERR_INVALID);
 
-    // BWD: the receivers that reach the brick; over kListCap of them every
+    // BWD: the receivers that reach the brick; over kSpanListCap of them every
     // step scans all receivers instead
     int nlist = 0;
     if constexpr (BWD) {
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
                 }
                 if (hit) {
                     const int k = atomicAdd(&s_count, 1);
-                    if (k < kListCap) list[k] = j;
+                    if (k < kSpanListCap) list[k] = j;
                 }
             }
         }
@@ -284,7 +283,7 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
     // the grid barrier is under way
     auto inject = [&](int m) {
         if (nlist == 0) return;
-        const bool all = nlist > kListCap;
+        const bool all = nlist > kSpanListCap;
         const int count = all ? A.nrec : nlist;
         const float* row = A.rdata + (size_t)(m - 1) * A.nrec;
         auto put = [&](int x, int y, int z, float r) {
@@ -770,7 +769,7 @@ SpanPlan span_plan(int R, int NX, int NY, int NZ, int backward) {
                     if (nbricks > sms) break;  // one brick per SM
                     const long long box = (long long)(4 * bxv + 2 * R) * (by + 2 * R) * (bz + 2 * R);
                     const long long smem = (box + 31) / 32 * 128 +
-                                           (backward ? 16LL * bxv * by * bz + 4 * kListCap
+                                           (backward ? 16LL * bxv * by * bz + 4 * kSpanListCap
                                                      : (long long)sizeof(rtm_point_taps) * kTapCap) +
                                            128;
                     if (smem > kSmemMax - 1024) continue;

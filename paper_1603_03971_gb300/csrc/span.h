@@ -29,6 +29,10 @@ struct SpanPlan {
     int threads = 0, smem = 0;
 };
 
+// receivers of a brick that its block keeps in shared memory in a backward span;
+// over them every step looks at all receivers
+constexpr int kSpanListCap = 2048;
+
 struct SpanArgs {
     SpanPlan P;
     const float *c, *gx, *gy, *gz, *wav;

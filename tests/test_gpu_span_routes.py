@@ -72,3 +72,51 @@ def test_off_grid_receivers_of_a_small_grid(nrec):
 def test_off_grid_receivers_under_binomial_checkpointing(grid, nrec):
     spans, launches = _spans_and_launches(4, _off_grid(*grid, "revolve", 10, nrec))
     assert spans <= SLACK * launches
+
+
+@pytest.mark.parametrize("grid", [(28, 24, 20, 6), (64, 64, 64, 20), (96, 90, 80, 16)])
+@pytest.mark.parametrize("planes", [1, 6, 1000])
+def test_receivers_on_the_grid(grid, planes):
+    import torch
+
+    import paper_1603_03971_gb300 as rtm
+
+    nx, ny, nz, nb = grid
+    g = DeviceShot(Case(nx=nx, ny=ny, nz=nz, nb=nb, nt=60, storage="ckpt", ckpt_every=20))
+    z, y, x = np.meshgrid(np.arange(min(planes, nz)), np.arange(ny), np.arange(nx), indexing="ij")
+    rec = torch.from_numpy(np.stack([x, y, z], axis=-1).reshape(-1, 3).astype(np.int32)).cuda()
+    p = g.p.copy(nrec=rec.shape[0])
+    ws = rtm.alloc_workspace(p)
+    dobs = torch.randn((60, p.nrec), device="cuda")
+    img = torch.zeros(rtm.model_shape(p), device="cuda")
+    spans, launches = _spans_and_launches(4, lambda: rtm.shot(p, g.c, rec, dobs, ws, img))
+    assert spans <= SLACK * launches
+
+
+def test_a_brick_over_its_list_takes_all_receivers():
+    import torch
+
+    import paper_1603_03971_gb300 as rtm
+
+    # 16250 receivers in a cube of 25 x 25 x 26 cells: several thousand in a
+    # brick of 104^3, which lists 2048
+    case = Case(nx=64, ny=64, nz=64, nb=20, nt=9, src=(32, 32, 40))
+    g = DeviceShot(case)
+    z, y, x = np.meshgrid(np.arange(26), np.arange(25), np.arange(25), indexing="ij")
+    rec = torch.from_numpy(np.stack([x, y, z], axis=-1).reshape(-1, 3).astype(np.int32)).cuda()
+    p = g.p.copy(nrec=rec.shape[0])
+    ws = rtm.alloc_workspace(p)
+    dobs = torch.from_numpy(case.d_obs(p.nrec).astype(np.float32)).cuda()
+    out = []
+    for variant in (0, 3):
+        rtm.set_tuning(4, 0, variant)
+        try:
+            img = torch.zeros(rtm.model_shape(p), device="cuda")
+            data = torch.empty((p.nt, p.nrec), device="cuda")
+            rtm.shot(p, g.c, rec, dobs, ws, img, data=data)
+            rtm.check(ws)
+        finally:
+            rtm.set_tuning(4, 0, 0)
+        out.append((img.cpu().numpy(), data.cpu().numpy()))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert np.any(out[0][0] != 0)
