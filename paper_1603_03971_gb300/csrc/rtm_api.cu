@@ -399,8 +399,9 @@ rtm_status make_ctx(Ctx& C, const rtm_params* p, const float* c, void* ws, rtm_s
     bool tuned = zc > 0 || var != 0 || timing;
     for (int m = 0; m < MODE_COUNT; m++) tuned = tuned || C.zchunk_mode[m] > 0;
     if (!tuned) {
-        C.span_fwd = span_plan(p->radius, C.d.NX, C.d.NY, C.d.NZ, 0);
-        C.span_bwd = span_plan(p->radius, C.d.NX, C.d.NY, C.d.NZ, 1);
+        const int sms = span_sms(C.s);
+        C.span_fwd = span_plan(p->radius, C.d.NX, C.d.NY, C.d.NZ, 0, sms);
+        C.span_bwd = span_plan(p->radius, C.d.NX, C.d.NY, C.d.NZ, 1, sms);
     }
     return RTM_OK;
 }

@@ -701,15 +701,39 @@ cudaError_t launch_span_r(const SpanArgs& a, cudaStream_t s) {
                        : launch_span_t<R, BWD, kColumn, false>(a, s);
 }
 
-int num_sms() {
+template <class F>
+F driver_entry(const char* name) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPointByVersion(name, &p, 12040, cudaEnableDefault, &q) == cudaSuccess &&
+                   q == cudaDriverEntryPointSuccess
+               ? reinterpret_cast<F>(p)
+               : nullptr;
+}
+
+}  // namespace
+
+// Blocks of a span wait for one another, so all of them have to be resident: a
+// stream of a green context runs on that context's SMs only
+int span_sms(cudaStream_t stream) {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 0;
+    static const auto green_of =
+        driver_entry<CUresult (*)(CUstream, CUgreenCtx*)>("cuStreamGetGreenCtx");
+    static const auto resource_of =
+        driver_entry<CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType)>(
+            "cuGreenCtxGetDevResource");
+    CUgreenCtx green = nullptr;
+    if (green_of && resource_of && green_of(stream, &green) == CUDA_SUCCESS && green) {
+        CUdevResource r;
+        memset(&r, 0, sizeof r);
+        if (resource_of(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return 0;
+        n = std::min(n, (int)r.sm.smCount);
+    }
     return n;
 }
-
-}  // namespace
 
 // wavefronts per 8 lanes of a 16-byte shared-memory load whose lanes run over
 // rows of bxv vectors in a box of row stride bxv + R / 2 vectors (1: no conflict)
@@ -727,10 +751,9 @@ static double conflicts(int bxv, int R) {
     return (double)total / bxv;
 }
 
-SpanPlan span_plan(int R, int NX, int NY, int NZ, int backward) {
+SpanPlan span_plan(int R, int NX, int NY, int NZ, int backward, int sms) {
     SpanPlan best;
     const long long N = (long long)NX * NY * NZ;
-    const int sms = num_sms();
     // a brick's box has to fit the shared memory of one SM
     if (!tma_available() || sms < 1 || N > (long long)sms * (kSmemMax / 4)) return best;
     struct Key {

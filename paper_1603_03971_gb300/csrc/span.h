@@ -69,8 +69,10 @@ struct SpanArgs {
     int* status;
 };
 
-// the tiling for a padded grid, or ok = 0 where the plain launches are used
-SpanPlan span_plan(int radius, int NX, int NY, int NZ, int backward);
+// SMs that work of this stream runs on (0: unknown, no spans)
+int span_sms(cudaStream_t stream);
+// the tiling for a padded grid over `sms` SMs, or ok = 0 where the plain launches are used
+SpanPlan span_plan(int radius, int NX, int NY, int NZ, int backward, int sms);
 // barriers of a launch: what ctrl->count grows by is P.nbricks * (nsteps - 1)
 cudaError_t launch_span(const SpanArgs& a, cudaStream_t s);
 
