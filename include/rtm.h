@@ -582,22 +582,30 @@ rtm_status rtm_set_tuning(int32_t radius, int32_t zchunk, int32_t variant);
  * the per-mode timings of its trials. Applies to the single-shot calls. */
 rtm_status rtm_set_tuning_mode(int32_t radius, int32_t mode, int32_t zchunk);
 
-/* Host-injected wait failure for testing the timeout path of the kernels
- * with mbarrier rings: kernel RTM_STALL_STENCIL (the TMA stencil's plain
- * forward step with 8-row tiles, tuning variant 3, as a separate kernel
- * instance: the others carry no code for it) or RTM_STALL_ENCODER (the
- * z-marching codec encoder); plane >= 0 arms a
+/* Host-injected wait failure for testing the timeout paths: kernel
+ * RTM_STALL_STENCIL (the TMA stencil's plain
+ * forward step with 8-row tiles, tuning variant 3), RTM_STALL_ROWS (the same
+ * step at radius 8 with two rows per thread, tuning variant 2; both as
+ * separate kernel instances: the others carry no code for it),
+ * RTM_STALL_ENCODER (the z-marching codec encoder) or RTM_STALL_SPAN (many
+ * steps per launch); plane >= 0 arms a
  * one-shot stall of that kernel's next launch: block 0's copy of the plane
- * `plane` planes before the last one it copies (0: the last; the encoder
- * takes 0-2) expects 16 bytes more than it delivers, so the bounded wait
+ * `plane` planes before the last one it copies (0: the last; the encoder and
+ * the two-row stencil take 0-2) expects 16 bytes more than it delivers, so the bounded wait
  * for it runs out after about 2 s; the block raises its abort flag, waits
  * (bounded) for every copy it issued and leaves, and the call's status word
  * reads RTM_ERR_TIMEOUT (rtm_check). Every copy lands, and no later copy
  * reuses the stalled ring slot (a wait for a later phase of a barrier whose
- * phase never completes would pass at once); nothing faults. -1 disarms.
+ * phase never completes would pass at once); nothing faults. In a span (of
+ * two steps or more) block 0's wait for the others, before the step `plane`
+ * steps from the span's last, asks for a step that they cannot take without
+ * it, and the bound is 2 s where it is 20 s otherwise: every block leaves, and
+ * so do the spans after it in that call. -1 disarms.
  * Returns RTM_ERR_INVALID for an unknown kernel. */
 #define RTM_STALL_STENCIL 0
 #define RTM_STALL_ENCODER 1
+#define RTM_STALL_ROWS 2
+#define RTM_STALL_SPAN 3
 rtm_status rtm_set_test_stall(int32_t kernel, int32_t plane);
 
 /* Enable (1) or disable (0) per-launch CUDA-event timing of the stencil

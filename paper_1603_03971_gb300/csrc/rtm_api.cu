@@ -65,8 +65,8 @@ int g_zchunk[kMaxRadius + 1] = {0};
 int g_zchunk_mode[kMaxRadius + 1][MODE_COUNT] = {{0}};
 int g_variant[kMaxRadius + 1] = {0};
 // one-shot stalls armed by rtm_set_test_stall (RTM_STALL_*), -1 = none
-constexpr int kStallKernels = 2;
-std::atomic<int> g_test_stall[kStallKernels] = {{-1}, {-1}};
+constexpr int kStallKernels = 4;
+std::atomic<int> g_test_stall[kStallKernels] = {{-1}, {-1}, {-1}, {-1}};
 bool g_timing = false;
 rtm_stats g_stats;
 

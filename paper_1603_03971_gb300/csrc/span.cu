@@ -57,7 +57,7 @@ namespace {
 // leave a block few columns spread them over four times the threads
 constexpr int kColumn = 4;
 constexpr int kTapCap = 32;                              // tap tables of a block kept in shared memory
-constexpr unsigned long long kBarrierNs = 20000000000ull;  // bound of a grid barrier: 20 s
+constexpr unsigned long long kBarrierNs = 20000000000ull;  // bound of a grid barrier: 20 s (SpanArgs)
 constexpr int kSmemMax = 227 * 1024;
 
 // threads of a block: what the registers of one block per SM allow (128, 168
@@ -89,20 +89,20 @@ __device__ __forceinline__ void load_box(float* dst, const CUtensorMap* map, int
 }
 // bounded wait for a box, whose copy follows thread 0's bounded wait for the
 // other blocks. One that runs out ends the span at the next grid barrier
-__device__ __forceinline__ bool poll_box(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool poll_box(uint64_t* bar, uint32_t parity, const SpanArgs& A) {
     const uint32_t a = su32(bar);
     if (mbar_try_wait_sleep(a, parity, 20000)) return true;
     const unsigned long long t0 = wait_now();
     while (!mbar_try_wait_sleep(a, parity, 20000))
-        if (wait_now() - t0 > kBarrierNs + kWaitNs) return false;
+        if (wait_now() - t0 > A.limit_ns + kWaitNs) return false;
     return true;
 }
 
 __device__ __forceinline__ void wait_box(uint64_t* bar, uint32_t parity, const SpanArgs& A) {
-    if (poll_box(bar, parity)) return;
+    if (poll_box(bar, parity, A)) return;
     atomicExch(&A.ctrl->abort, 1);
     if (A.status) atomicCAS(A.status, 0, RTM_ERR_TIMEOUT);
-    if (threadIdx.x == 0) poll_box(bar, parity);  // the copy should land before the block leaves
+    if (threadIdx.x == 0) poll_box(bar, parity, A);  // the copy should land before the block leaves
 }
 
 // thread 0's half of the grid barrier between two steps, split so that what
@@ -114,7 +114,8 @@ __device__ __forceinline__ void grid_arrive(SpanCtrl* ctrl) {
 }
 // false if the wait ran out or another block gave up; otherwise this thread
 // may issue copies of what the other blocks wrote before they arrived
-__device__ __forceinline__ bool grid_wait(SpanCtrl* ctrl, unsigned int target, int* status) {
+__device__ __forceinline__ bool grid_wait(const SpanArgs& A, unsigned int target) {
+    SpanCtrl* const ctrl = A.ctrl;
     unsigned long long t0 = 0;
     bool ok = *reinterpret_cast<volatile int*>(&ctrl->abort) == 0;
     for (long long i = 0; ok; i++) {
@@ -124,9 +125,9 @@ __device__ __forceinline__ bool grid_wait(SpanCtrl* ctrl, unsigned int target, i
         if ((i & 63) == 63) {
             const unsigned long long t = wait_now();
             if (t0 == 0) t0 = t;
-            if (*reinterpret_cast<volatile int*>(&ctrl->abort) || t - t0 > kBarrierNs) {
+            if (*reinterpret_cast<volatile int*>(&ctrl->abort) || t - t0 > A.limit_ns) {
                 atomicExch(&ctrl->abort, 1);
-                if (status) atomicCAS(status, 0, RTM_ERR_TIMEOUT);
+                if (A.status) atomicCAS(A.status, 0, RTM_ERR_TIMEOUT);
                 ok = false;
             }
         }
@@ -337,7 +338,9 @@ __global__ void __launch_bounds__(span_threads<R, BWD, PZ>(), 1)
             if (here) return;
             here = true;
             if (tid == 0) {
-                if (i > 0 && !grid_wait(A.ctrl, A.base + gridDim.x * (unsigned int)i, A.status)) {
+                // (a stalled wait: a step more than the others can get to without block 0)
+                const unsigned int more = i == A.stall && blockIdx.x == 0 ? 1u : 0u;
+                if (i > 0 && !grid_wait(A, A.base + gridDim.x * ((unsigned int)i + more))) {
                     s_ok = 0;  // no copy: the arrival alone completes the phase
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&bar)) : "memory");
                 } else {
@@ -822,8 +825,17 @@ SpanPlan span_plan(int R, int NX, int NY, int NZ, int backward, int sms) {
     return best;
 }
 
-cudaError_t launch_span(const SpanArgs& a, cudaStream_t s) {
+cudaError_t launch_span(SpanArgs a, cudaStream_t s) {
     if (!a.P.ok || a.nsteps < 1) return cudaErrorInvalidValue;
+    a.stall = -1;
+    a.limit_ns = kBarrierNs;
+    if (a.nsteps > 1) {
+        const int stall = take_test_stall(RTM_STALL_SPAN);
+        if (stall >= 0) {
+            a.stall = std::max(1, a.nsteps - 1 - stall);
+            a.limit_ns = kWaitNs;
+        }
+    }
     if (a.radius == 4) return a.backward ? launch_span_r<4, true>(a, s) : launch_span_r<4, false>(a, s);
     if (a.radius == 8) return a.backward ? launch_span_r<8, true>(a, s) : launch_span_r<8, false>(a, s);
     return cudaErrorInvalidValue;

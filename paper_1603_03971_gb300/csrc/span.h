@@ -66,6 +66,8 @@ struct SpanArgs {
     float a[kMaxRadius + 1];
     SpanCtrl* ctrl;
     unsigned int base;   // ctrl->count before this launch
+    int stall;           // step whose wait for the other blocks a test lets run out, or -1
+    unsigned long long limit_ns;  // bound of that wait in every step
     int* status;
 };
 
@@ -74,6 +76,6 @@ int span_sms(cudaStream_t stream);
 // the tiling for a padded grid over `sms` SMs, or ok = 0 where the plain launches are used
 SpanPlan span_plan(int radius, int NX, int NY, int NZ, int backward, int sms);
 // barriers of a launch: what ctrl->count grows by is P.nbricks * (nsteps - 1)
-cudaError_t launch_span(const SpanArgs& a, cudaStream_t s);
+cudaError_t launch_span(SpanArgs a, cudaStream_t s);
 
 }  // namespace rtm

@@ -104,10 +104,11 @@ __device__ __forceinline__ void copy3(float* dst, const CUtensorMap* map, int x,
         : "memory");
 }
 
-template <int MODE>
+// STALL: the instance that takes a test-armed stall (rtm_set_test_stall)
+template <int MODE, bool STALL = false>
 __global__ void __launch_bounds__(BX* BY, 2)
     k_stencil_rows(const __grid_constant__ StepArgs A, const __grid_constant__ RowMaps M,
-                   int* status) {
+                   int* status, int stall) {
     using C = Cfg<MODE>;
     extern __shared__ __align__(128) float dsm[];
     float* uring = dsm;
@@ -149,7 +150,14 @@ __global__ void __launch_bounds__(BX* BY, 2)
         issued = p + 1;
         const int slot = (p - zb) % C::NS;
         float* base = aring + slot * C::NA * APLANE;
-        expect(&bar[slot], (UPLANE + C::NA * APLANE) * 4);
+        uint32_t extra = 0;
+        if constexpr (STALL) {
+            // 16 bytes that never arrive, for one of the last planes of block 0: no
+            // later copy takes its slot and completes the stuck phase's successor
+            if (p == ze - 1 - stall && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
+                extra = 16;
+        }
+        expect(&bar[slot], (UPLANE + C::NA * APLANE) * 4 + extra);
         copy3(uring + slot * UPLANE, &M.u, x0 - R, y0 - R, p, &bar[slot]);
         copy3(base + (C::NA - 1) * APLANE, &M.uh, x0, y0, p + R, &bar[slot]);
         copy3(base, &M.prev, x0, y0, p, &bar[slot]);
@@ -317,7 +325,17 @@ cudaError_t launch_t(const StepArgs& a, int* status, cudaStream_t s) {
         return cudaErrorInvalidValue;
     const dim3 grid((a.xend - a.xorg + TX - 1) / TX, (a.yend - a.yorg + TY - 1) / TY,
                     (a.zend - a.zorg + a.zchunk - 1) / a.zchunk);
-    return launch_next(k_stencil_rows<MODE>, grid, dim3(BX, BY), smem, s, a, M, status);
+    if constexpr (MODE == MODE_FWD) {
+        const int stall = take_test_stall(RTM_STALL_ROWS);
+        if (stall >= 0) {
+            e = cudaFuncSetAttribute(k_stencil_rows<MODE, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+            return launch_next(k_stencil_rows<MODE, true>, grid, dim3(BX, BY), smem, s, a, M, status,
+                               stall < Cfg<MODE>::NS ? stall : Cfg<MODE>::NS - 1);
+        }
+    }
+    return launch_next(k_stencil_rows<MODE>, grid, dim3(BX, BY), smem, s, a, M, status, -1);
 }
 
 // encoded maps of this thread, by every encoding argument: a shot launches its
