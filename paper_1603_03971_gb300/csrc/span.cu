@@ -35,7 +35,11 @@
 // the rest barrier, copy and store latency (3.1 us on the smallest grid).
 //
 // Every cell sees the operations of the plane-marching kernels in their
-// order, so both paths give the same bits.
+// order, so both paths give the same bits, except where receivers meet: those of
+// one cell, and off the grid the taps of neighbours, are summed before they are
+// scaled and added to the field, where the launches add each to the field by
+// itself. There the results differ by roundings, and in either path by the order
+// of the atomic sums (three terms or more).
 
 #include <string.h>
 
