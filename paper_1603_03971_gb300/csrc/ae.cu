@@ -241,7 +241,7 @@ struct OpE2 {  // h1 -> latent
     }
 };
 
-struct OpD1 {  // latent -> g1, one output parity class per blockIdx.y
+struct OpD1 {  // latent -> g1, one output parity class per blockIdx.y: the products of OpD12
     using Args = D1Args;
     static constexpr int N = 32;
     __device__ static void tile(const Args&, int& m0, int& c0, int& c1) {
@@ -314,18 +314,6 @@ struct OpD1 {  // latent -> g1, one output parity class per blockIdx.y
             for (int e = 0; e < 8; e++) w[e] = a.P[kOW3 + o * 1024 + ktap * 16 + i0 + e];
             tc::st_vec8(sB, o, 8 * j, tc::pack8(w));
         }
-    }
-    __device__ static void epilogue(const Args& a, int m0, int row, const float* acc) {
-        const long long v = m0 + row;
-        if (v >= (long long)a.l.nx * a.l.ny * a.l.nz) return;
-        const int q = blockIdx.y, qz = q >> 2, qy = (q >> 1) & 1, qx = q & 1;
-        int x, y, z;
-        decode3(v, a.l.nx, a.l.ny, x, y, z);
-        const long long o = (((long long)(2 * z + qz) * a.h.ny + (2 * y + qy)) * a.h.nx + 2 * x + qx);
-        float f[32];
-#pragma unroll
-        for (int c = 0; c < 32; c++) f[c] = leaky(acc[c] + a.P[kOB3 + c]);
-        store_bf16_row(a.g1 + o * 32, f, 32);
     }
 };
 
@@ -760,7 +748,7 @@ cudaError_t ae_encode(const float* P, const Vol& in, bf16* h1, bf16* lat, AeScal
 cudaError_t ae_decode(const float* P, const bf16* lat, const float* sigma, const Vol& out,
                       int* status, cudaStream_t s) {
     const Dims3 h{out.nx / 2, out.ny / 2, out.nz / 2}, l{out.nx / 4, out.ny / 4, out.nz / 4};
-    D12Args a{D1Args{lat, l, P, nullptr, h}, sigma, out};
+    D12Args a{D1Args{lat, l, P, h}, sigma, out};
     const cudaError_t e = ae_decode_march(a, status, s);
     if (e != cudaErrorNotSupported) return e;
     cudaGetLastError();

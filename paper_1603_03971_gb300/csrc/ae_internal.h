@@ -49,7 +49,7 @@ struct GemmArgs { const bf16* A; const bf16* B; float* C; int M, K; };
 // xq: each voxel's 8 normalised inputs, kept for the weight gradient, or NULL
 struct E1Args { Vol in; const float* inv_sigma; const float* P; bf16* h1; Dims3 h; bf16* xq; };
 struct E2Args { const bf16* h1; Dims3 h; const float* P; bf16* lat; Dims3 l; };
-struct D1Args { const bf16* lat; Dims3 l; const float* P; bf16* g1; Dims3 h; };
+struct D1Args { const bf16* lat; Dims3 l; const float* P; Dims3 h; };
 struct D2Args { const bf16* g1; Dims3 h; const float* P; const float* sigma; Vol out; };
 struct D12Args { D1Args d1; const float* sigma; Vol out; };
 struct D2dArgs { const bf16* gy; Dims3 h; const bf16* g1; const float* P; bf16* ga3; };

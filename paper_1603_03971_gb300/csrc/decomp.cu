@@ -463,7 +463,6 @@ rtm_status rtm_forward_decomposed(const rtm_params* p, int32_t px, int32_t py, c
         a.xend = q.x1;
         a.yorg = q.y0;
         a.yend = q.y1;
-        if (r == 8 && tile_rows == 16) return launch_stencil_rows(MODE_FWD, a, status, stream_of(k));
         return launch_stencil_tma(r, MODE_FWD, a, status, stream_of(k), tile_rows);
     };
     const int npack = (int)hs.size() / 2;

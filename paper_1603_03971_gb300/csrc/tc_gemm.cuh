@@ -66,9 +66,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 __device__ __forceinline__ void st_vec8(uint8_t* slab, int r, int k, uint4 v) {
     *reinterpret_cast<uint4*>(slab + kmajor_off(r, k)) = v;
 }
-__device__ __forceinline__ void st_one(uint8_t* slab, int r, int k, __nv_bfloat16 v) {
-    *reinterpret_cast<__nv_bfloat16*>(slab + kmajor_off(r, k)) = v;
-}
 
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);  // .x = a (low half), .y = b
