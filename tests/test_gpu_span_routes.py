@@ -1,6 +1,6 @@
 """Where many steps per launch are the automatic choice they are not slower
 than the launch-per-step kernels (tuning variant 3), with few and with many
-receivers."""
+receivers; and what a step's receivers cost the launches."""
 import time
 
 import numpy as np
@@ -72,6 +72,14 @@ def test_off_grid_receivers_of_a_small_grid(nrec):
 def test_off_grid_receivers_under_binomial_checkpointing(grid, nrec):
     spans, launches = _spans_and_launches(4, _off_grid(*grid, "revolve", 10, nrec))
     assert spans <= SLACK * launches
+
+
+@pytest.mark.parametrize("nrec", [256, 1024])
+def test_a_few_receivers_off_the_grid_hardly_cost_a_launch_per_step(nrec):
+    """On a grid above the spans' sizes a step is two stencil launches of 30 us;
+    1024 receivers are 0.5 M of its taps, 2 us at the L2 cache's rate."""
+    one, many = (_best_ms(_off_grid(150, 131, 117, 21, "all", 0, n)) for n in (1, nrec))
+    assert many <= SLACK * one
 
 
 @pytest.mark.parametrize("grid", [(28, 24, 20, 6), (64, 64, 64, 20), (96, 90, 80, 16)])
