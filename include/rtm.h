@@ -559,7 +559,10 @@ rtm_status rtm_forward_decomposed(const rtm_params *p, int32_t px, int32_t py, c
  * (0 = automatic) and the plane-load path and tile (0 = automatic: TMA
  * where the driver provides tensor maps, with the tile of 3 at radius 4 and
  * of 2 at radius 8; on grids of one brick per SM, where the slab height is
- * automatic too, many steps per cooperative launch; 1 = 16-byte vector loads
+ * automatic too, many steps per cooperative launch, which takes the whole GPU
+ * while it runs: shots of several streams then run one after another, and on
+ * grids of about 100^3 and up four streams or more get further with a variant
+ * named here; 1 = 16-byte vector loads
  * through registers; 2 = TMA bulk tensor copies into shared-memory rings,
  * 16-row tiles, at radius 4 of 256 threads, at radius 8 of 128 threads with
  * two rows each; 3 = the same with 8-row tiles of 128 threads and

@@ -114,7 +114,9 @@ rtm_status check_batch(const rtm_params* p, int nshots, const rtm_aperture* sh) 
 bool batch_uses_tma(int radius) { return tma_available() && tuning_variant(radius) != 1; }
 // tile rows of the TMA kernel: 8 unless the 16-row tile (variant 2) is
 // selected. Six shots of 170-280 cells: 17.8 against 20.8 ms at radius 4; at
-// radius 8 both take 23.2
+// radius 8 both take 23.2. Many apertures at radius 8 are 2 % faster in 16-row
+// tiles (two rows per thread): 32 of 128-384 cells, 24 steps, 475 against 486 ms;
+// the batch tuner selects them there
 int batch_tile_rows(int radius) { return tuning_variant(radius) == 2 ? 16 : 8; }
 
 Plan make_plan(const rtm_params* p, int nshots, const rtm_aperture* sh, size_t budget,

@@ -85,8 +85,9 @@ cudaError_t launch_stencil_tma(int radius, int mode, const StepArgs& a, int* sta
 // radius 8, 16-row tiles with two rows per thread (stencil_rows.cu)
 cudaError_t launch_stencil_rows(int mode, const StepArgs& a, int* status, cudaStream_t s);
 bool tma_available();
-// z-slab height: of the vector-load kernel's launches by block count, and of a
-// tuning variant's (1-3) launch of a mode by its waves of resident blocks
+// z-slab height: by block count (the decomposed and the allocation-free forward
+// pass), and of a tuning variant's (1-3) launch of a mode by its waves of resident
+// blocks (the single-shot calls)
 int auto_zchunk(int radius, int NX, int NY, int NZ);
 int slab_height(int radius, int variant, int mode, int nx, int ny, int nz);
 

@@ -2,9 +2,8 @@
 // holds.
 //
 // On such grids a step is bound by latencies, not by bytes: at 104^3 padded,
-// radius 4, a launch of the plane-marching stencil took 16 us (a 16-plane
-// march, three planes in flight), the receiver kernel before it 3.7 us, and
-// HBM would need 2.7 us. Here the padded grid is cut into one brick per SM,
+// radius 4, the receiver kernel and the plane-marching stencil take 10 us (21
+// before they were dependent launches), and HBM would need 2.7 us. Here the padded grid is cut into one brick per SM,
 // each block keeps its brick for every step of the span, and blocks meet at a
 // grid barrier between steps. The brick's u^n with its halo arrives as one
 // bulk tensor copy, so a step pays one copy latency; its u^{n-1}, c, snapshot
@@ -17,20 +16,25 @@
 // one step later, from a complete field), so a step has one barrier in either
 // direction.
 //
-// Microseconds per step, forward / forward + snapshot / backward + imaging,
-// against the per-step launches (automatic tile, receiver kernel included):
-//   40 x 36 x 32, r = 4:      3.1 / 3.3 / 3.8     16 / 17 / 18
-//   104^3, r = 4:             6.5 / 7.1 / 8.6     18.5 / 18.5 / 18.6
-//   132 x 120 x 110, r = 4:   9.4 / 10.1 / 13.1   18.6 / 20.6 / 20.6
-//   104^3, r = 8 (forward):   10.9 / 11.5         20.5 / 20.5
-//   104^3, r = 4, off grid:   12.1 / - / 14.7     42 / - / 34     (1024 receivers)
+// Microseconds per step of a 60-step shot that keeps every snapshot, forward /
+// backward + imaging, against the launch-per-step kernels (8-row tiles, receiver
+// kernel included) and against these before they were dependent launches:
+//   40 x 36 x 32, r = 4:      3.8 / 4.3      8.9 / 8.8      21 / 20
+//   64 x 60 x 56, r = 4:      4.0 / 4.7      9.9 / 8.8      21 / 20
+//   104^3, r = 4:             7.5 / 9.3      10.5 / 9.8     21 / 21
+//   128 x 122 x 112, r = 4:   9.9 / 12.2     11.8 / 11.4    21 / 21
+//   104^3, r = 8 (forward):   11.9           11.8           27
+//   104^3, r = 4, off grid:   12.1 / 14.8    28 / 43        34 / 33   (1024 receivers)
 // A brick has to fit one SM's shared memory, which is also where a launch per
-// step catches up: several bricks per SM (192 x 173 x 159, five each) took
-// 21 / 23 / 32 us against 25 / 26 / 27.
+// step has caught up. A span takes every SM: shots of several host threads run
+// one after another (ms per 100-step shot with 1 / 4 / 8 threads, spans against
+// launches: 40 x 36 x 32 0.87 / 0.28 / 0.24 and 1.77 / 0.58 / 0.39; 104^3 1.68 /
+// 1.58 / 1.57 and 2.05 / 1.06 / 1.15). A call cannot see the others, so whoever
+// runs four such shots or more at a time names a variant (rtm_set_tuning).
 // Off the grid a receiver is up to 8^3 taps and its neighbours share bricks:
-// taken by the bricks that they reach, 1024 receivers made a step 13.2 / 39.4
-// us (3969: 17.2 / 120). So the blocks share the receivers out evenly and the
-// data go through one of two padded fields, a step ahead (3969: 15.7 / 19.8).
+// taken by the bricks that they reach, 1024 receivers made a backward step 39
+// us (3969: 120). So the blocks share the receivers out evenly and the data go
+// through one of two padded fields, a step ahead (3969: 20).
 // What is left at 104^3: about 4 us of shared-memory reads and instructions,
 // the rest barrier, copy and store latency (3.1 us on the smallest grid).
 //

@@ -11,13 +11,14 @@
 // registers, so two blocks of 128 threads run per SM: the loads of a plane
 // are independent, so eight warps keep the shared-memory pipe busy.
 //
-// Microseconds per launch at 576^3 (8-row tiles of one row per thread -> here,
-// and of the measured HBM copy rate): forward 645 -> 534 (85 %), forward +
-// snapshot 695 -> 592 (95 %), backward + imaging 795 -> 780 (100 %); 364 x 325
-// x 294: 143 -> 115, 155 -> 123, 169 -> 155. 32 x 32 tiles (2.25 floats of
-// plane per point) took 537 / 624 / 800 at 576^3: their narrower rows cost more
-// than the smaller halo gains. The queue moves every second plane; every plane
-// (8 fewer registers) was the same within 1 %.
+// Microseconds per launch for a 512^3 model in 576^3, automatic slabs (8-row
+// tiles of one row per thread -> here, and of the measured HBM copy rate):
+// forward 663 -> 536 (69 -> 85 %), forward + snapshot 687 -> 584 (78 -> 91 %),
+// backward + imaging 760 -> 728 (91 -> 95 %); a 300^3 model in 364^3: 206 -> 164,
+// 209 -> 180, 225 -> 199. 32 x 32 tiles (2.25 floats of plane per point) took
+// 537 / 624 / 800 at 576^3 without a sponge, where these take 534 / 592 / 780:
+// their narrower rows cost more than the smaller halo gains. The queue moves
+// every second plane; every plane (8 fewer registers) was the same within 1 %.
 //
 // The rings, barriers and epilogues are those of the split-ring instances of
 // stencil_tma.cu, and every cell sees their operations in their order, so the

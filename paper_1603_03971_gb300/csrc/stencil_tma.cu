@@ -57,8 +57,8 @@ struct TmaMaps {
 constexpr int kVec = 4;
 
 // tile: 16 threads along x (V floats each) by BYT rows, one row per thread
-// (16 rows: 256 threads, the default; 8 rows: 128 threads, more blocks per SM
-// and twice the y halo per row, an autotuner choice)
+// (8 rows: 128 threads, more blocks per SM and twice the y halo per row, the
+// automatic choice at radius 4; 16 rows: 256 threads, radius 4 only)
 template <int R, int V, int BYT = 16>
 struct TmaTile {
     static constexpr int BX = 16;          // threads along x, V floats each
