@@ -713,10 +713,10 @@ cudaError_t launch_span_r(const SpanArgs& a, cudaStream_t s) {
 }
 
 template <class F>
-F driver_entry(const char* name) {
+F driver_entry(const char* name, unsigned int version) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
-    return cudaGetDriverEntryPointByVersion(name, &p, 12040, cudaEnableDefault, &q) == cudaSuccess &&
+    return cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &q) == cudaSuccess &&
                    q == cudaDriverEntryPointSuccess
                ? reinterpret_cast<F>(p)
                : nullptr;
@@ -731,13 +731,18 @@ int span_sms(cudaStream_t stream) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 0;
-    static const auto green_of =
-        driver_entry<CUresult (*)(CUstream, CUgreenCtx*)>("cuStreamGetGreenCtx");
+    // (the second version of the call, with the green context)
+    static const auto contexts_of =
+        driver_entry<CUresult (*)(CUstream, CUcontext*, CUgreenCtx*)>("cuStreamGetCtx", 12050);
     static const auto resource_of =
         driver_entry<CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType)>(
-            "cuGreenCtxGetDevResource");
+            "cuGreenCtxGetDevResource", 12040);
+    if (!contexts_of || !resource_of) return n;  // a driver without green contexts
+    CUcontext ctx = nullptr;
     CUgreenCtx green = nullptr;
-    if (green_of && resource_of && green_of(stream, &green) == CUDA_SUCCESS && green) {
+    // fails for the per-thread default stream of a green context
+    if (contexts_of(stream, &ctx, &green) != CUDA_SUCCESS) return 0;
+    if (green) {
         CUdevResource r;
         memset(&r, 0, sizeof r);
         if (resource_of(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return 0;

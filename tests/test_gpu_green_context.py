@@ -2,6 +2,7 @@
 grids that take many steps per launch on the whole device are tiled for those
 SMs, or take the launches, with the same results."""
 import ctypes
+from types import SimpleNamespace
 
 import numpy as np
 import pytest
@@ -69,3 +70,21 @@ def test_shot_on_a_few_sms(grid):
         destroy()
     for a, b in zip(got, want):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("handle", [0, 1, 2, None])  # NULL, legacy, per thread, a created one
+def test_special_streams_take_many_steps_per_launch(handle):
+    import torch
+
+    import paper_1603_03971_gb300 as rtm
+
+    g = DeviceShot(Case(nt=20, storage="all"))
+    dobs = torch.from_numpy(g.case.d_obs(g.nrec).astype(np.float32)).cuda()
+    img = torch.zeros(rtm.model_shape(g.p), device="cuda")
+    stream = torch.cuda.Stream() if handle is None else SimpleNamespace(cuda_stream=handle)
+    torch.cuda.synchronize()
+    rtm.reset_stats()
+    rtm.shot(g.p, g.c, g.rec, dobs, g.ws, img, stream=stream)
+    torch.cuda.synchronize()
+    assert rtm.stats()["launches"] < 20  # 2 x 20 steps
+    rtm.check(g.ws)
