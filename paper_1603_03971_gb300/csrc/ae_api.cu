@@ -21,7 +21,9 @@ size_t upa(size_t v) { return (v + kAl - 1) / kAl * kAl; }
 
 struct AeLayout {
     size_t status = 0, scalars = 64;
-    size_t h1, lat, g1, y, gy, ga3, glat, ga1, xq, grad, packed, total;
+    size_t h1, lat, g1, y, gy, ga3, glat, ga1, grad;
+    size_t coding;  // what encode and decode ask for; training keeps more behind it
+    size_t xq, packed, total;
 };
 
 AeLayout ae_layout(int nx, int ny, int nz) {
@@ -41,8 +43,9 @@ AeLayout ae_layout(int nx, int ny, int nz) {
     L.ga3 = take(nh * 32 * 2);
     L.glat = take(nl * 16 * 2);
     L.ga1 = take(nh * 32 * 2);
-    L.xq = take(nh * 8 * 2);
     L.grad = take((size_t)kNParams * 4);
+    L.coding = o;
+    L.xq = take(nh * 8 * 2);
     L.packed = take(kAePackedBytes);
     L.total = o;
     return L;
@@ -93,7 +96,7 @@ rtm_status rtm_ae_encode(const float* d_params, const float* d_snap, int64_t sy,
     rtm_status st = check_dims(nx, ny, nz);
     if (st != RTM_OK) return st;
     const AeLayout L = ae_layout(nx, ny, nz);
-    if ((st = check_ws(d_ws, ws_bytes, L.total)) != RTM_OK) return st;
+    if ((st = check_ws(d_ws, ws_bytes, L.coding)) != RTM_OK) return st;
     if (!d_params || !d_snap || !d_latent || ((uintptr_t)d_latent % 16))
         return (rtm_status)set_error(RTM_ERR_INVALID, "codec arrays NULL or latent not 16-byte aligned");
     if (sy < nx || sz < sy * ny)
@@ -115,7 +118,7 @@ rtm_status rtm_ae_decode(const float* d_params, const uint16_t* d_latent, const 
     rtm_status st = check_dims(nx, ny, nz);
     if (st != RTM_OK) return st;
     const AeLayout L = ae_layout(nx, ny, nz);
-    if ((st = check_ws(d_ws, ws_bytes, L.total)) != RTM_OK) return st;
+    if ((st = check_ws(d_ws, ws_bytes, L.coding)) != RTM_OK) return st;
     if (!d_params || !d_latent || !d_out || ((uintptr_t)d_latent % 16))
         return (rtm_status)set_error(RTM_ERR_INVALID, "codec arrays NULL or latent not 16-byte aligned");
     if (sy < nx || sz < sy * ny)
