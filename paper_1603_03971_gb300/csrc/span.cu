@@ -3,8 +3,8 @@
 //
 // On such grids a step is bound by latencies, not by bytes: at 104^3 padded,
 // radius 4, the receiver kernel and the plane-marching stencil take 10 us (21
-// before they were dependent launches), and HBM would need 2.7 us. Here the padded grid is cut into one brick per SM,
-// each block keeps its brick for every step of the span, and blocks meet at a
+// before they were dependent launches), and HBM would need 2.7 us. Here the padded
+// grid is cut into one brick per SM, each block keeps its brick for every step of the span, and blocks meet at a
 // grid barrier between steps. The brick's u^n with its halo arrives as one
 // bulk tensor copy, so a step pays one copy latency; its u^{n-1}, c, snapshot
 // and image, which no other block writes, and the receivers' terms are
@@ -24,7 +24,7 @@
 //   104^3, r = 4:             7.5 / 9.3      10.5 / 9.8     21 / 21
 //   128 x 122 x 112, r = 4:   9.9 / 12.2     11.8 / 11.4    21 / 21
 //   104^3, r = 8 (forward):   11.9           11.8           27
-//   104^3, r = 4, off grid:   12.1 / 14.8    28 / 43        34 / 33   (1024 receivers)
+//   104^3, r = 4, off grid:   12.2 / 14.7    26 / 25        34 / 33   (1024 receivers)
 // A brick has to fit one SM's shared memory, which is also where a launch per
 // step has caught up. A span takes every SM: shots of several host threads run
 // one after another (ms per 100-step shot with 1 / 4 / 8 threads, spans against
